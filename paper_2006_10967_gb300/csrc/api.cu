@@ -22,6 +22,7 @@ struct Layout {
   size_t tri_d, tri_f, tri_high;  // dense triangle operators (double, float), mode mask
   size_t wphys;                   // triangles: physical edge quadrature weight per flux point (float-float)
   size_t ffw;                     // hexahedra: face words (KArgs.ffw)
+  size_t vtab;                    // mixed tensor fields with a velocity cache: velocity factors (KArgs.vtab)
   size_t total;
 };
 
@@ -82,6 +83,11 @@ void fill_bulk(const fr_params* prm, const fr_mesh* m, BulkConst<R>& b) {
   b.prm.delta = (R)prm->delta;
   b.prm.nphi = prm->normal == FR_NORMAL_PHI;
   b.prm.noflux = prm->wall == FR_WALL_NOFLUX;
+  b.prm.rdelta = (R)std::min(1.0 / prm->delta, 3.0e38);
+  // see k_vel_tab: uniform a_c, Rider-Kothe (-1, 1, 0), LeVeque (2, -1, -1), rotation (1, 1, 0) without g
+  const double vs[5][3] = {{prm->vel.a[0], prm->vel.a[1], prm->vel.a[2]}, {-1, 1, 0}, {2, -1, -1}, {0, 0, 0}, {1, 1, 0}};
+  for (int c = 0; c < 3; ++c) b.prm.vs[c] = (R)vs[prm->vel.kind][c];
+  b.prm.vel_g = prm->vel.kind != FR_VEL_ROTATION;
   if (m->etype != FR_TRI) {
     const Tensor1D& t = m->t1;
     for (int i = 0; i < t.n; ++i) {
@@ -103,6 +109,45 @@ void fill_bulk(const fr_params* prm, const fr_mesh* m, BulkConst<R>& b) {
       }
     }
   }
+}
+
+// The 1D operators in pairs (LineOps), the pad of odd n zero.
+void fill_line_ops(const fr_mesh* m, LineOps& o) {
+  std::memset(&o, 0, sizeof(o));
+  if (m->etype == FR_TRI) return;
+  const Tensor1D& t = m->t1;
+  auto put = [&](float2& d, int i, double v) { (i & 1 ? d.y : d.x) = (float)v; };
+  for (int i = 0; i < t.n; ++i) {
+    o.lend[i] = make_float2((float)t.lend[0][i], (float)t.lend[1][i]);
+    for (int j = 0; j < t.n; ++j) put(o.D[j][i / 2], i, t.D[i][j]);
+    put(o.gL[i / 2], i, t.gLd[i]);
+    put(o.ngL[i / 2], i, -t.gLd[i]);
+    put(o.gR[i / 2], i, t.gRd[i]);
+    put(o.xp[i / 2], i, t.x[i]);
+  }
+}
+
+// Whether every element's map is affine with a diagonal Jacobian in single
+// precision (flag 2 of every metric record, k_metric_const).
+bool all_diagonal(const fr_mesh& m) {
+  const int nc = m.ncoef, dim = m.dim;
+  for (int64_t e = 0; e < m.E; ++e)
+    for (int c = 0; c < dim; ++c) {
+      const double* g = &m.geo[(e * dim + c) * nc];
+      for (int k = 1; k < nc; ++k)
+        if (k != 1 + c && (float)g[k] != 0.f) return false;
+    }
+  return true;
+}
+
+// The line kernels (kline.cuh) step the mixed fields of quads and hexes that
+// keep their velocity at the points (vel_cache); the block-wide kernels keep
+// FP64 fields, hexes of p = 5 and fields without the cache.
+bool use_line_kernels(const fr_mesh& m, const fr_params& p) {
+  return m.etype != FR_TRI && p.precision == FR_MIXED && p.vel_cache && (m.etype == FR_QUAD || m.order <= 4);
+}
+bool set_line_kernels(const fr_mesh& m, bool gen, KernelSet* ks) {
+  return m.etype == FR_QUAD ? line_kernels_quad(m.order, gen, ks) : line_kernels_hex(m.order, gen, ks);
 }
 
 Layout make_layout(const fr_mesh& m, int precision, int max_blocks, int vel_cache) {
@@ -138,6 +183,7 @@ Layout make_layout(const fr_mesh& m, int precision, int max_blocks, int vel_cach
   L.ep = take(E * sizeof(ElemPar));
   L.mcg = m.etype != FR_TRI ? take(E * kMetricRec * tb) : 0;  // per-element metric records
   L.ffw = m.etype == FR_HEX ? take(E * 6 * sizeof(int2)) : 0;
+  L.vtab = m.etype != FR_TRI && precision == FR_MIXED && vc ? take(E * m.dim * (m.n + 2) * sizeof(float2)) : 0;
   if (m.etype == FR_TRI) {
     const size_t nops = tri_op_count(m);
     L.tri_d = take(nops * sizeof(double));
@@ -631,6 +677,15 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
   A.wdetf = reinterpret_cast<const float2*>(b + L.wdetf);
   A.ep = nullptr;
   A.mcg = L.mcg ? b + L.mcg : nullptr;
+  A.vtab = nullptr;
+  fill_line_ops(m, A.lo);
+  if (use_line_kernels(*m, *prm)) {
+    if (vel_separable(prm->vel.kind)) A.vtab = reinterpret_cast<const float2*>(b + L.vtab);
+    if (!set_line_kernels(*m, !(A.vtab && all_diagonal(*m)), &f->ks)) {
+      delete f;
+      return FR_ECUDA;
+    }
+  }
   f->ep_region = reinterpret_cast<ElemPar*>(b + L.ep);
   A.out = nullptr;
   A.stage = 0;
@@ -749,6 +804,7 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
     if (!f->ks.vcache) err = FR_EUNSUPPORTED;
     else f->ks.vcache(A, s);
   }
+  if (err == FR_OK && A.vtab) f->ks.vtab(A, s);
   if (err == FR_OK) err = stage_and_traces(f, s);
   if (err == FR_OK && ic->precondition && prm->normal == FR_NORMAL_PSI) err = run_precondition(f, s);
   if (err == FR_OK && cudaStreamSynchronize(s) != cudaSuccess) err = FR_ECUDA;
@@ -829,6 +885,14 @@ extern "C" int fr_field_init_batch(const fr_mesh* m, const fr_params* prm, int n
     return FR_ECUDA;
   }
   f->args.ep = f->ep_region;
+  if (use_line_kernels(*m, *prm)) {
+    // the table holds params->vel, the instances' own velocities are in the point cache
+    f->args.vtab = nullptr;
+    if (!set_line_kernels(*m, true, &f->ks)) {
+      fr_field_destroy(f);
+      return FR_ECUDA;
+    }
+  }
   drop_graphs(f);  // the launch arguments changed
   // the batch's pseudo step for the launch arguments is per element; keep a positive value
   rc = FR_OK;
@@ -963,7 +1027,7 @@ extern "C" int fr_rhs(fr_field* f, double t, double* dev_out, void* stream) {
   f->ks.kb[0](a, s);
   a.stage = -1;
   a.out = dev_out;
-  f->ks.ka[0](a, s);
+  f->ks.ka_rate(a, s);
   CK(cudaGetLastError());
   return FR_OK;
 }

@@ -36,6 +36,7 @@ void fill_tri(int64_t E, KernelSet* ks) {
   ks->kb[0] = launch_kb_tri<P, T, 0, TC>;
   ks->kb[1] = launch_kb_tri<P, T, 1, TC>;
   ks->ka[0] = launch_ka_tri<P, T, 0, TC>;
+  ks->ka_rate = ks->ka[0];
   ks->ka[1] = launch_ka_tri<P, T, 1, TC>;
   int et = KBTriLayout<P, T, 0, TC>::ET;
   if (KATriLayout<P, T, 0, TC>::ET < et) et = KATriLayout<P, T, 0, TC>::ET;

@@ -34,6 +34,10 @@ struct PrmT {
   R gamma, eps, tau, tau_psi, tau_pseudo, delta;
   int nphi;    // 1: the sharpening normal comes from phi's gradient (unpreconditioned CPF)
   int noflux;  // 1: zero common normal flux of the physical system at wall flux points
+  R rdelta;    // 1 / delta
+  // separable velocity fields (vel_factors): v_c = vs[c] g prod_b T_cb with g = 1 unless vel_g
+  R vs[3];
+  int vel_g;
 };
 
 struct PhysPrm {
@@ -50,6 +54,14 @@ struct TensorOpsT {
   float2 wff[kMaxN * kMaxN];  // face quadrature weights (products of GL weights) as float-float pairs
 };
 typedef TensorOpsT<double> TensorOps;
+
+// The 1D operators in the pairs that the paired-FP32 line kernels use
+// (kline.cuh): outputs (2p, 2p + 1) of a line, or a line's two ends.
+struct LineOps {
+  float2 D[kMaxN][4];                 // [input m][output pair p]
+  float2 lend[kMaxN];                 // (l_m(-1), l_m(+1))
+  float2 gL[4], ngL[4], gR[4], xp[4];  // end lifts (ngL = -gL) and coordinates by point pair
+};
 
 // Bulk-precision constants of one field, in both precisions.
 template <typename R>
@@ -127,6 +139,7 @@ struct KArgs {
   ElemPar* ep;           // E per-element parameters (batched instances) or nullptr (uniform)
   const float2* wdetf;   // E x nu: w_i det J_i as float-float pairs (mixed path)
   void* mcg;             // tensor elements: E x 16 metric records (bulk type)
+  const float2* vtab;    // mixed tensor fields: E x dim x (n + 2) velocity factors (k_vel_tab), or nullptr
   const float2* wphys;   // triangles: E x nf physical flux-point weights (float-float), equal on both sides
   int stage;             // 1..4 RK stage, -1: write the rate into out
   int use_dev_time;      // KB: t = dstate[DS_TIME] + c_s dt
@@ -136,6 +149,7 @@ struct KArgs {
   PhysPrm prm;
   BulkConst<double> cd;
   BulkConst<float> cf;
+  LineOps lo;
   TriOpsT<double> trid;
   TriOpsT<float> trif;
 };

@@ -11,6 +11,8 @@ typedef void (*LaunchFn)(const KArgs&, cudaStream_t);
 struct KernelSet {
   LaunchFn kb[2] = {nullptr, nullptr};  // [mode]: 0 physical, 1 preconditioning
   LaunchFn ka[2] = {nullptr, nullptr};
+  LaunchFn ka_rate = nullptr;           // ka[0]'s kernel with stage -1 (the rate into KArgs.out)
+  LaunchFn vtab = nullptr;              // fills the velocity factor table (line kernels)
   int max_blocks = 0;                   // upper bound on blocks of any launch (per element count)
   LaunchFn vcache = nullptr;            // fills the spatial velocity cache (nullptr: not supported)
   LaunchFn mconst = nullptr;            // fills the per-element metric records (tensor elements)
@@ -21,6 +23,12 @@ struct KernelSet {
 bool kernels_quad(int order, int precision, int64_t E, int variant, KernelSet* ks);
 bool kernels_hex(int order, int precision, int64_t E, int variant, KernelSet* ks);
 bool kernels_tri(int order, int precision, int64_t E, int variant, KernelSet* ks);
+
+// Replace the physical-step kernels of a mixed tensor field by the line kernels
+// (kline.cuh); false where they are not built (the set is then unchanged) or
+// could not be prepared.  gen: see kb_line.
+bool line_kernels_quad(int order, bool gen, KernelSet* ks);
+bool line_kernels_hex(int order, bool gen, KernelSet* ks);
 
 template <typename K>
 inline void launch_kernel(K kern, size_t smem, int et, const KArgs& A, cudaStream_t s, int threads = kThreads) {

@@ -1,0 +1,112 @@
+"""The warp-per-element kernels of the mixed physical step (fields of quads and
+hexes with a velocity cache) against the block-wide kernels, which the same
+field takes without the cache: same scheme, other arithmetic order.
+
+Tolerances: a mixed residual is within 1e-4 of the FP64 one (float round-off
+times the operator norm), so two mixed residuals differ by at most 2e-4; a
+short march with either agrees with FP64 to 1e-5 (the parity tests' bounds),
+so the two agree to 2e-5."""
+import numpy as np
+import pytest
+
+import synthetic as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def G():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    import paper_2006_10967_gb300 as G
+    return G
+
+
+def _workload(etype, order, ns, jitter, kind, walls, normal="psi", wall="copy"):
+    dim = 3 if etype == "hex" else 2
+    per = (not walls,) * dim
+    rot = 5 if jitter else None
+    grid = S.meshes.hex_grid if dim == 3 else S.meshes.quad_grid
+    mesh = grid(*ns, periodic=per, jitter=jitter, shuffle_seed=6 if jitter else None, rotate_seed=rot)
+    if kind == "stream":
+        vel = S.workloads.random_phase_stream(np.random.default_rng(2))
+    else:
+        vel = S.Velocity(kind, a=(0.6, 0.4, 0.3) if kind == "uniform" else (0.5, 0.5, 0.0),
+                         T=3.0 if kind in ("leveque", "rider_kothe") else 0.0)
+    h = 1.0 / max(ns)
+    w = S.Workload("line", lambda: mesh, order, vel, S.Circle((0.4,) * dim, 0.25, 3 * order / (4 * h)),
+                   t_end=1.0, h=h, precision="mixed", wall=wall)
+    w = S.workloads._finish(w, dim)
+    w.normal = normal
+    w.n_precond = 3
+    w.pseudo_kmax = 3
+    return w, mesh
+
+
+def _rel(a, b):
+    return np.abs(a - b).max() / np.abs(b).max()
+
+
+QUADS = [("quad", p, ns, jit, vel, walls) for p in range(1, 7)
+         for ns, jit, vel, walls in [((1, 1), 0.0, "uniform", True), ((7, 5), 0.1, "stream", False),
+                                     ((13, 9), 0.0, "rotation", False), ((9, 11), 0.1, "rider_kothe", True),
+                                     ((8, 5), 0.0, "rider_kothe", True)]]
+HEXES = [("hex", p, ns, jit, vel, walls) for p in range(1, 6)
+         for ns, jit, vel, walls in [((1, 1, 1), 0.0, "uniform", True), ((3, 4, 5), 0.1, "leveque", True),
+                                     ((5, 3, 3), 0.0, "leveque", False), ((4, 3, 3), 0.1, "uniform", False)]]
+
+
+@pytest.mark.parametrize("etype,order,ns,jitter,vel,walls", QUADS + HEXES)
+def test_line_kernels_agree_with_the_block_wide_ones(G, etype, order, ns, jitter, vel, walls):
+    w, mesh = _workload(etype, order, ns, jitter, vel, walls)
+    M = G.Mesh.from_synthetic(mesh, order)
+    F, B = [G.Field(M, G.make_params(w, "mixed", vel_cache=c, pseudo_fixed=True), ic=w.circle) for c in (True, False)]
+    R, Rb = F.rhs(0.3).cpu().numpy(), B.rhs(0.3).cpu().numpy()
+    for f in (0, 1):
+        assert _rel(R[f], Rb[f]) < 2e-4
+    m0 = F.mass(0)
+    for f in (F, B):
+        f.step(5)  # the preconditioning before the fourth step included
+        assert f.sync() == 0
+    for which in (0, 1):
+        assert _rel(F.get(which), B.get(which)) < 2e-5
+    if not walls:  # the flux balance keeps the mass to round-off
+        assert abs(F.mass(0) - m0) < 1e-13
+
+
+@pytest.mark.parametrize("normal,wall", [("phi", "copy"), ("psi", "noflux"), ("phi", "noflux")])
+@pytest.mark.parametrize("etype,order,ns,jitter,vel", [("quad", 4, (9, 7), 0.1, "rider_kothe"),
+                                                       ("quad", 3, (9, 7), 0.0, "rider_kothe"),
+                                                       ("hex", 3, (4, 3, 3), 0.0, "leveque"),
+                                                       ("hex", 2, (4, 3, 3), 0.1, "leveque")])
+def test_line_kernel_options(G, etype, order, ns, jitter, vel, normal, wall):
+    w, mesh = _workload(etype, order, ns, jitter, vel, True, normal, wall)
+    M = G.Mesh.from_synthetic(mesh, order)
+    F, B = [G.Field(M, G.make_params(w, "mixed", vel_cache=c, pseudo_fixed=True, normal=normal, wall=wall),
+                    ic=w.circle) for c in (True, False)]
+    for f in (F, B):
+        f.step(3)
+        assert f.sync() == 0
+    for which in (0, 1):
+        assert _rel(F.get(which), B.get(which)) < 2e-5
+
+
+@pytest.mark.parametrize("etype,order,ns,vel", [("quad", 4, (9, 7), "rider_kothe"), ("hex", 3, (4, 3, 3), "leveque"),
+                                                ("hex", 4, (3, 3, 2), "leveque"), ("quad", 3, (5, 4), "rotation")])
+def test_an_element_does_not_depend_on_the_rest_of_the_mesh(G, etype, order, ns, vel):
+    """An axis-aligned grid alone (every element takes the diagonal path) and
+    in a union with a jittered one march to the same bits."""
+    w, mesh = _workload(etype, order, ns, 0.0, vel, False)
+    _, other = _workload(etype, order, ns, 0.1, vel, False)
+    A, B = G.Mesh.from_synthetic(mesh, order), G.Mesh.from_synthetic(other, order)
+    U = G.Mesh.concat([B, A])
+    P = G.make_params(w, "mixed", pseudo_fixed=True)
+    alone = G.Field(A, P, ic=w.circle)
+    both = G.Field(U, P, ic=w.circle)
+    for f in (alone, both):
+        f.step(4)
+        assert f.sync() == 0
+    n = B.info.n_elems
+    for which in (0, 1):
+        assert np.array_equal(alone.get(which), both.get(which)[n:])
