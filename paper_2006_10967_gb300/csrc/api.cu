@@ -119,7 +119,10 @@ void fill_line_ops(const fr_mesh* m, LineOps& o) {
   auto put = [&](float2& d, int i, double v) { (i & 1 ? d.y : d.x) = (float)v; };
   for (int i = 0; i < t.n; ++i) {
     o.lend[i] = make_float2((float)t.lend[0][i], (float)t.lend[1][i]);
-    for (int j = 0; j < t.n; ++j) put(o.D[j][i / 2], i, t.D[i][j]);
+    for (int j = 0; j < t.n; ++j) {
+      put(o.D[j][i / 2], i, t.D[i][j]);
+      put(o.V[j][i / 2], i, t.Vinv[i][j]);
+    }
     put(o.gL[i / 2], i, t.gLd[i]);
     put(o.ngL[i / 2], i, -t.gLd[i]);
     put(o.gR[i / 2], i, t.gRd[i]);
@@ -146,8 +149,27 @@ bool all_diagonal(const fr_mesh& m) {
 bool use_line_kernels(const fr_mesh& m, const fr_params& p) {
   return m.etype != FR_TRI && p.precision == FR_MIXED && p.vel_cache && (m.etype == FR_QUAD || m.order <= 4);
 }
+// The preconditioning's line kernels serve every mixed field of those meshes
+// (no velocity enters).
+bool use_line_pseudo(const fr_mesh& m, const fr_params& p) {
+  return m.etype != FR_TRI && p.precision == FR_MIXED && (m.etype == FR_QUAD || m.order <= 4);
+}
+bool set_line_pseudo(const fr_mesh& m, bool gen, KernelSet* ks) {
+  return m.etype == FR_QUAD ? line_pseudo_quad(m.order, gen, ks) : line_pseudo_hex(m.order, gen, ks);
+}
 bool set_line_kernels(const fr_mesh& m, bool gen, KernelSet* ks) {
   return m.etype == FR_QUAD ? line_kernels_quad(m.order, gen, ks) : line_kernels_hex(m.order, gen, ks);
+}
+
+// Blocks of the largest launch (one reduction partial each): the block-wide
+// kernels', the element-wise kernels' or the line kernels'.
+int most_blocks(const fr_mesh& m, const KernelSet& ks, int elementwise) {
+  int64_t n = std::max(ks.max_blocks, elementwise);
+  if (m.etype != FR_TRI && m.nfp <= 32) {
+    const int per = kLineWarps * (32 / m.nfp);
+    n = std::max<int64_t>(n, (m.E + per - 1) / per);
+  }
+  return (int)n;
 }
 
 Layout make_layout(const fr_mesh& m, int precision, int max_blocks, int vel_cache) {
@@ -325,39 +347,76 @@ __device__ __forceinline__ void neu_add(double& s, double& c, double x) {
   s = t;
 }
 
-// Compensated, fixed-order integral of field `fld` with weights wdet.
-__global__ void k_mass(KArgs A, int64_t NU, int fld, int mixed) {
-  __shared__ double ss[kThreads], sc[kThreads];
-  __shared__ bool last;
-  const int64_t n = A.E * NU;
-  double s = 0.0, c = 0.0;
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = g / NU, i = g % NU;
-    neu_add(s, c, A.wdet[g] * u_get(A, mixed, (e * 2 + fld) * NU + i));
+// Block-wide compensated sum in a fixed tree (shuffles within the warps, then
+// the first warp over the warps' values); thread 0 gets the result.
+__device__ __forceinline__ void neu_block(double& s, double& c, double* ss, double* sc) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double s2 = __shfl_down_sync(0xffffffffu, s, o), c2 = __shfl_down_sync(0xffffffffu, c, o);
+    neu_add(s, c, s2);
+    c += c2;
   }
-  ss[threadIdx.x] = s;
-  sc[threadIdx.x] = c;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  if (l == 0) {
+    ss[w] = s;
+    sc[w] = c;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double bs = 0.0, bc = 0.0;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      neu_add(bs, bc, ss[t]);
-      bc += sc[t];
+  if (w == 0) {
+    s = l < kThreads / 32 ? ss[l] : 0.0;
+    c = l < kThreads / 32 ? sc[l] : 0.0;
+#pragma unroll
+    for (int o = kThreads / 64; o > 0; o >>= 1) {
+      const double s2 = __shfl_down_sync(0xffffffffu, s, o), c2 = __shfl_down_sync(0xffffffffu, c, o);
+      neu_add(s, c, s2);
+      c += c2;
     }
-    A.red[2 * blockIdx.x] = bs;
-    A.red[2 * blockIdx.x + 1] = bc;
+  }
+}
+
+// Compensated, fixed-order integral of field `fld` with weights wdet.  Bound by
+// the FP64 pipe (nine instructions a point at 2 lanes a clock): the block and
+// grid sums run as trees, since one thread adding the 256 values of its block
+// and then every block's in turn was a serial FP64 chain of 1.2 ms on 7.1 M
+// points, whatever their number.
+__global__ void __launch_bounds__(kThreads) k_mass(KArgs A, int NU, int fld, int mixed) {
+  __shared__ double ss[kThreads / 32], sc[kThreads / 32];
+  __shared__ bool last;
+  const int64_t n = A.E * NU, stride = (int64_t)gridDim.x * kThreads;
+  double s = 0.0, c = 0.0;
+  // the point's element advances by a fixed quotient and remainder per step
+  int64_t g = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+  int64_t e = g / NU;
+  int i = (int)(g - e * NU);
+  const int64_t qe = stride / NU;
+  const int qi = (int)(stride - qe * NU);
+  for (; g < n; g += stride) {
+    neu_add(s, c, A.wdet[g] * u_get(A, mixed, (e * 2 + fld) * NU + i));
+    e += qe;
+    i += qi;
+    if (i >= NU) {
+      i -= NU;
+      ++e;
+    }
+  }
+  neu_block(s, c, ss, sc);
+  if (threadIdx.x == 0) {
+    A.red[2 * blockIdx.x] = s;
+    A.red[2 * blockIdx.x + 1] = c;
     __threadfence();
     last = atomicAdd(&A.status[ST_COUNTER], 1) == (int)gridDim.x - 1;
   }
   __syncthreads();
-  if (last && threadIdx.x == 0) {
-    __threadfence();
-    double ts = 0.0, tc = 0.0;
-    for (int b = 0; b < (int)gridDim.x; ++b) {
-      neu_add(ts, tc, ((volatile double*)A.red)[2 * b]);
-      tc += ((volatile double*)A.red)[2 * b + 1];
-    }
-    A.dstate[DS_MASS] = ts + tc;
+  if (!last) return;
+  __threadfence();
+  s = c = 0.0;
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += kThreads) {
+    neu_add(s, c, ((volatile double*)A.red)[2 * b]);
+    c += ((volatile double*)A.red)[2 * b + 1];
+  }
+  neu_block(s, c, ss, sc);
+  if (threadIdx.x == 0) {
+    A.dstate[DS_MASS] = s + c;
     A.status[ST_COUNTER] = 0;
   }
 }
@@ -589,7 +648,7 @@ extern "C" int fr_field_workspace_bytes(const fr_mesh* m, const fr_params* prm, 
   if (!get_kernels(*m, prm->precision, prm->variant, &ks)) return FR_EUNSUPPORTED;
   int mg;
   launch_elementwise_grid(m->E * m->nu, &mg);
-  const int mb = ks.max_blocks > mg ? ks.max_blocks : mg;
+  const int mb = most_blocks(*m, ks, mg);
   *bytes = make_layout(*m, prm->precision, mb, prm->vel_cache).total;
   return FR_OK;
 }
@@ -606,7 +665,7 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
   if (!ks.prepared) return FR_ECUDA;
   int mg;
   launch_elementwise_grid(m->E * m->nu, &mg);
-  const int mb = ks.max_blocks > mg ? ks.max_blocks : mg;
+  const int mb = most_blocks(*m, ks, mg);
   const Layout L = make_layout(*m, prm->precision, mb, prm->vel_cache);
   if (ws_bytes < L.total) return FR_ENOMEM;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
@@ -686,6 +745,10 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
       return FR_ECUDA;
     }
   }
+  if (use_line_pseudo(*m, *prm) && !set_line_pseudo(*m, !all_diagonal(*m), &f->ks)) {
+    delete f;
+    return FR_ECUDA;
+  }
   f->ep_region = reinterpret_cast<ElemPar*>(b + L.ep);
   A.out = nullptr;
   A.stage = 0;
@@ -706,6 +769,15 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
   A.prm.pseudo_fixed = prm->pseudo_fixed;
   A.prm.T = prm->vel.T;
   A.prm.rT = prm->vel.T > 0.0 ? 1.0 / prm->vel.T : 0.0;
+  auto split = [](double v, float& h, float& l) {
+    h = (float)v;
+    l = (float)(v - (double)h);
+  };
+  const double rs = M_PI / (4.0 * prm->kappa);
+  split(-rs * (prm->s0 - prm->kappa), A.prm.ramp_c0h, A.prm.ramp_c0l);
+  split(rs * std::log10(2.0), A.prm.ramp_c1h, A.prm.ramp_c1l);
+  split(rs * 2.0 * std::log10(std::exp(1.0)), A.prm.ramp_c2h, A.prm.ramp_c2l);
+  split(prm->nu_max, A.prm.nu_h, A.prm.nu_l);
   fill_bulk<double>(prm, m, A.cd);
   fill_bulk<float>(prm, m, A.cf);
 
@@ -961,6 +1033,16 @@ int copy_field(fr_field* f, int which, void* dst, const void* src, bool to_state
     else CK(cudaMemcpyAsync(dst, f->args.psi0, E * NU * 8, kind, s));
     return FR_OK;
   }
+  if (kind == cudaMemcpyDeviceToDevice) {
+    // one pass between the state and the caller's device array
+    int grid;
+    launch_elementwise_grid(f->E * f->nu, &grid);
+    const int mixed = f->precision == FR_MIXED;
+    if (to_state) k_pack<<<grid, kThreads, 0, s>>>(f->args, f->nu, which, mixed, static_cast<const double*>(src));
+    else k_unpack<<<grid, kThreads, 0, s>>>(f->args, f->nu, which, mixed, static_cast<double*>(dst));
+    CK(cudaGetLastError());
+    return FR_OK;
+  }
   if (f->precision == FR_FP64) {
     if (to_state)
       CK(cudaMemcpy2DAsync(f->args.u + which * NU, 2 * NU * 8, src, NU * 8, NU * 8, E, kind, s));
@@ -1044,7 +1126,7 @@ extern "C" int fr_rhs_pseudo(fr_field* f, double* dev_out, void* stream) {
   f->ks.kb[1](a, s);
   a.stage = -1;
   a.out = dev_out;
-  f->ks.ka[1](a, s);
+  f->ks.ka_rate_pseudo(a, s);
   CK(cudaGetLastError());
   return FR_OK;
 }

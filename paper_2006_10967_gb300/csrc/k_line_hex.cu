@@ -12,4 +12,13 @@ bool line_kernels_hex(int order, bool gen, KernelSet* ks) {
     default: return false;
   }
 }
+bool line_pseudo_hex(int order, bool gen, KernelSet* ks) {
+  switch (order) {
+    case 1: return gen ? fill_line_pseudo<3, 2, true>(ks) : fill_line_pseudo<3, 2, false>(ks);
+    case 2: return gen ? fill_line_pseudo<3, 3, true>(ks) : fill_line_pseudo<3, 3, false>(ks);
+    case 3: return gen ? fill_line_pseudo<3, 4, true>(ks) : fill_line_pseudo<3, 4, false>(ks);
+    case 4: return gen ? fill_line_pseudo<3, 5, true>(ks) : fill_line_pseudo<3, 5, false>(ks);
+    default: return false;
+  }
+}
 }  // namespace frp

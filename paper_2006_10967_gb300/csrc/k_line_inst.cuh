@@ -2,12 +2,9 @@
 #pragma once
 #include "kdispatch.hpp"
 #include "kline.cuh"
+#include "kline_pseudo.cuh"
 
 namespace frp {
-
-// Warps a block: the time factor (FP64) and the element balances (FP64) are
-// computed once a block, so a block holds several warps.
-constexpr int kLineWarps = 4;
 
 template <int DIM, int N>
 unsigned line_grid(int64_t E) {
@@ -57,6 +54,37 @@ bool fill_line(KernelSet* ks) {
                               KBLine<DIM, N>::F * 4 * kLineWarps) == cudaSuccess &&
          prepare_ka_line<DIM, N, GEN, 0>() && prepare_ka_line<DIM, N, GEN, 1>() && prepare_ka_line<DIM, N, GEN, 2>() &&
          prepare_ka_line<DIM, N, GEN, 3>() && prepare_ka_line<DIM, N, GEN, 4>();
+}
+
+template <int DIM, int N, bool GEN>
+void launch_kb_pseudo(const KArgs& A, cudaStream_t s) {
+  kbp_line<DIM, N, GEN, kLineWarps><<<line_grid<DIM, N>(A.E), kLineWarps * 32, KBPLine<DIM, N>::F * 4 * kLineWarps, s>>>(A);
+}
+
+template <int DIM, int N, bool GEN, int SF>
+void launch_kap_stage(const KArgs& A, cudaStream_t s) {
+  kap_line<DIM, N, GEN, kLineWarps, SF>
+      <<<line_grid<DIM, N>(A.E), kLineWarps * 32, KAPLine<DIM, N>::F * 4 * kLineWarps, s>>>(A);
+}
+
+template <int DIM, int N, bool GEN>
+void launch_ka_pseudo(const KArgs& A, cudaStream_t s) {
+  switch (A.stage) {
+    case 0: launch_kap_stage<DIM, N, GEN, 0>(A, s); return;
+    case 1: launch_kap_stage<DIM, N, GEN, 1>(A, s); return;
+    case 2: launch_kap_stage<DIM, N, GEN, 2>(A, s); return;
+    case 3: launch_kap_stage<DIM, N, GEN, 3>(A, s); return;
+    default: launch_kap_stage<DIM, N, GEN, 4>(A, s); return;
+  }
+}
+
+template <int DIM, int N, bool GEN>
+bool fill_line_pseudo(KernelSet* ks) {
+  static_assert(KBPLine<DIM, N>::F * 4 * kLineWarps <= 48 * 1024 && KAPLine<DIM, N>::F * 4 * kLineWarps <= 48 * 1024,
+                "no shared-memory opt-in needed");
+  ks->kb[1] = launch_kb_pseudo<DIM, N, GEN>;
+  ks->ka[1] = launch_ka_pseudo<DIM, N, GEN>;
+  return true;
 }
 
 }  // namespace frp

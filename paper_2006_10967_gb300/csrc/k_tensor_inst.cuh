@@ -70,6 +70,7 @@ void fill_tensor(int64_t E, KernelSet* ks) {
   ks->ka[0] = launch_ka_tensor<DIM, N, T, 0, TA>;
   ks->ka_rate = ks->ka[0];
   ks->ka[1] = launch_ka_tensor<DIM, N, T, 1>;
+  ks->ka_rate_pseudo = ks->ka[1];
   const int et_min = KBLayout<DIM, N, T, 0, TB>::ET < KALayout<DIM, N, T, 0, TA>::ET ? KBLayout<DIM, N, T, 0, TB>::ET
                                                                                       : KALayout<DIM, N, T, 0, TA>::ET;
   const int et_min1 = KBLayout<DIM, N, T, 1>::ET < KALayout<DIM, N, T, 1>::ET ? KBLayout<DIM, N, T, 1>::ET

@@ -38,6 +38,7 @@ void fill_tri(int64_t E, KernelSet* ks) {
   ks->ka[0] = launch_ka_tri<P, T, 0, TC>;
   ks->ka_rate = ks->ka[0];
   ks->ka[1] = launch_ka_tri<P, T, 1, TC>;
+  ks->ka_rate_pseudo = ks->ka[1];
   int et = KBTriLayout<P, T, 0, TC>::ET;
   if (KATriLayout<P, T, 0, TC>::ET < et) et = KATriLayout<P, T, 0, TC>::ET;
   if (KBTriLayout<P, T, 1, TC>::ET < et) et = KBTriLayout<P, T, 1, TC>::ET;

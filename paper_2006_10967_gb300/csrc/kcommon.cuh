@@ -45,6 +45,8 @@ struct PhysPrm {
   int pseudo_fixed;
   double T;   // period of the velocity time factor (<= 0: none)
   double rT;  // 1 / T (0 when T <= 0)
+  // the resolution indicator's ramp in float-float pairs (sensor_nu): z = c0 + k c1 + (log m / 2) c2, nu_max
+  float ramp_c0h, ramp_c0l, ramp_c1h, ramp_c1l, ramp_c2h, ramp_c2l, nu_h, nu_l;
 };
 
 // 1D tensor operators; kernels stage them into shared memory.
@@ -61,6 +63,7 @@ struct LineOps {
   float2 D[kMaxN][4];                 // [input m][output pair p]
   float2 lend[kMaxN];                 // (l_m(-1), l_m(+1))
   float2 gL[4], ngL[4], gR[4], xp[4];  // end lifts (ngL = -gL) and coordinates by point pair
+  float2 V[kMaxN][4];                 // modal transform (Vinv): [input m][mode pair p]
 };
 
 // Bulk-precision constants of one field, in both precisions.
@@ -92,6 +95,7 @@ constexpr int kMetricRec = 16;
 
 struct RKConstF {
   float half_dt, dt, dt6;
+  float r2h, r2l;  // 1 / dt^2 as a float-float pair
   double rdt, ddt, ddt6;
 };
 
@@ -103,6 +107,8 @@ __host__ __device__ __forceinline__ RKConstF rk_const(double dt) {
   c.rdt = 1.0 / dt;
   c.ddt = dt;
   c.ddt6 = dt / 6.0;
+  c.r2h = (float)(c.rdt * c.rdt);
+  c.r2l = (float)(c.rdt * c.rdt - (double)c.r2h);
   return c;
 }
 

@@ -11,7 +11,8 @@ typedef void (*LaunchFn)(const KArgs&, cudaStream_t);
 struct KernelSet {
   LaunchFn kb[2] = {nullptr, nullptr};  // [mode]: 0 physical, 1 preconditioning
   LaunchFn ka[2] = {nullptr, nullptr};
-  LaunchFn ka_rate = nullptr;           // ka[0]'s kernel with stage -1 (the rate into KArgs.out)
+  LaunchFn ka_rate = nullptr;           // the block-wide ka[0], ka[1]: their stage -1 writes the
+  LaunchFn ka_rate_pseudo = nullptr;    // rate into KArgs.out
   LaunchFn vtab = nullptr;              // fills the velocity factor table (line kernels)
   int max_blocks = 0;                   // upper bound on blocks of any launch (per element count)
   LaunchFn vcache = nullptr;            // fills the spatial velocity cache (nullptr: not supported)
@@ -29,6 +30,14 @@ bool kernels_tri(int order, int precision, int64_t E, int variant, KernelSet* ks
 // could not be prepared.  gen: see kb_line.
 bool line_kernels_quad(int order, bool gen, KernelSet* ks);
 bool line_kernels_hex(int order, bool gen, KernelSet* ks);
+// The same for the preconditioning kernels of a mixed tensor field; gen false:
+// every element is affine with a diagonal Jacobian.
+bool line_pseudo_quad(int order, bool gen, KernelSet* ks);
+bool line_pseudo_hex(int order, bool gen, KernelSet* ks);
+
+// Warps a block of the line kernels: the element balances and reductions take
+// FP64 once a block, so a block holds several warps.
+constexpr int kLineWarps = 4;
 
 template <typename K>
 inline void launch_kernel(K kern, size_t smem, int et, const KArgs& A, cudaStream_t s, int threads = kThreads) {

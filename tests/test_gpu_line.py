@@ -110,3 +110,17 @@ def test_an_element_does_not_depend_on_the_rest_of_the_mesh(G, etype, order, ns,
     n = B.info.n_elems
     for which in (0, 1):
         assert np.array_equal(alone.get(which), both.get(which)[n:])
+
+
+@pytest.mark.parametrize("etype,order,ns,jitter,vel,walls", QUADS + HEXES)
+def test_mixed_preconditioning_follows_fp64(G, etype, order, ns, jitter, vel, walls):
+    """The preconditioning in mixed precision against the FP64 field: rate,
+    three iterations and the residual of the last one (the bounds of the mixed
+    residual; the viscosity's ramp is covered by both)."""
+    w, mesh = _workload(etype, order, ns, jitter, vel, walls)
+    M = G.Mesh.from_synthetic(mesh, order)
+    F, D = [G.Field(M, G.make_params(w, p, pseudo_fixed=True), ic=w.circle) for p in ("mixed", "fp64")]
+    assert _rel(F.rhs_pseudo().cpu().numpy(), D.rhs_pseudo().cpu().numpy()) < 1e-4
+    assert F.stats()["last_pseudo_iters"] == D.stats()["last_pseudo_iters"] == 3
+    assert abs(F.stats()["last_pseudo_rms"] / D.stats()["last_pseudo_rms"] - 1) < 1e-4
+    assert _rel(F.get(1), D.get(1)) < 1e-5
