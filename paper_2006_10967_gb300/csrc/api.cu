@@ -166,7 +166,7 @@ bool set_line_kernels(const fr_mesh& m, bool gen, KernelSet* ks) {
 int most_blocks(const fr_mesh& m, const KernelSet& ks, int elementwise) {
   int64_t n = std::max(ks.max_blocks, elementwise);
   if (m.etype != FR_TRI && m.nfp <= 32) {
-    const int per = kLineWarps * (32 / m.nfp);
+    const int per = kPseudoWarps * (32 / m.nfp);
     n = std::max<int64_t>(n, (m.E + per - 1) / per);
   }
   return (int)n;

@@ -7,20 +7,22 @@
 namespace frp {
 
 template <int DIM, int N>
-unsigned line_grid(int64_t E) {
-  constexpr int per = kLineWarps * LL<DIM, N>::EPW;
+unsigned line_grid(int64_t E, int warps) {
+  const int per = warps * LL<DIM, N>::EPW;
   return (unsigned)((E + per - 1) / per);
 }
 
 template <int DIM, int N, bool GEN>
 void launch_kb_line(const KArgs& A, cudaStream_t s) {
-  kb_line<DIM, N, GEN, kLineWarps><<<line_grid<DIM, N>(A.E), kLineWarps * 32, KBLine<DIM, N>::F * 4 * kLineWarps, s>>>(A);
+  constexpr int smem = KBLine<DIM, N, GEN>::F * 4 * kLineWarps;
+  if (A.cf.prm.nphi) kb_line<DIM, N, GEN, true, kLineWarps><<<line_grid<DIM, N>(A.E, kLineWarps), kLineWarps * 32, smem, s>>>(A);
+  else kb_line<DIM, N, GEN, false, kLineWarps><<<line_grid<DIM, N>(A.E, kLineWarps), kLineWarps * 32, smem, s>>>(A);
 }
 
 template <int DIM, int N, bool GEN, int SF>
 void launch_ka_stage(const KArgs& A, cudaStream_t s) {
   ka_line<DIM, N, GEN, kLineWarps, SF>
-      <<<line_grid<DIM, N>(A.E), kLineWarps * 32, KALine<DIM, N, SF>::F * 4 * kLineWarps, s>>>(A);
+      <<<line_grid<DIM, N>(A.E, kLineWarps), kLineWarps * 32, KALine<DIM, N, SF, GEN>::F * 4 * kLineWarps, s>>>(A);
 }
 
 template <int DIM, int N, bool GEN>
@@ -42,7 +44,7 @@ void launch_vel_tab(const KArgs& A, cudaStream_t s) {
 template <int DIM, int N, bool GEN, int SF>
 bool prepare_ka_line() {
   return cudaFuncSetAttribute(ka_line<DIM, N, GEN, kLineWarps, SF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              KALine<DIM, N, SF>::F * 4 * kLineWarps) == cudaSuccess;
+                              KALine<DIM, N, SF, GEN>::F * 4 * kLineWarps) == cudaSuccess;
 }
 
 template <int DIM, int N, bool GEN>
@@ -50,21 +52,20 @@ bool fill_line(KernelSet* ks) {
   ks->kb[0] = launch_kb_line<DIM, N, GEN>;
   ks->ka[0] = launch_ka_line<DIM, N, GEN>;
   ks->vtab = launch_vel_tab<DIM, N>;
-  return cudaFuncSetAttribute(kb_line<DIM, N, GEN, kLineWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              KBLine<DIM, N>::F * 4 * kLineWarps) == cudaSuccess &&
-         prepare_ka_line<DIM, N, GEN, 0>() && prepare_ka_line<DIM, N, GEN, 1>() && prepare_ka_line<DIM, N, GEN, 2>() &&
+  static_assert(KBLine<DIM, N, GEN>::F * 4 * kLineWarps <= 48 * 1024, "no shared-memory opt-in needed");
+  return prepare_ka_line<DIM, N, GEN, 0>() && prepare_ka_line<DIM, N, GEN, 1>() && prepare_ka_line<DIM, N, GEN, 2>() &&
          prepare_ka_line<DIM, N, GEN, 3>() && prepare_ka_line<DIM, N, GEN, 4>();
 }
 
 template <int DIM, int N, bool GEN>
 void launch_kb_pseudo(const KArgs& A, cudaStream_t s) {
-  kbp_line<DIM, N, GEN, kLineWarps><<<line_grid<DIM, N>(A.E), kLineWarps * 32, KBPLine<DIM, N>::F * 4 * kLineWarps, s>>>(A);
+  kbp_line<DIM, N, GEN, kPseudoWarps><<<line_grid<DIM, N>(A.E, kPseudoWarps), kPseudoWarps * 32, KBPLine<DIM, N, GEN>::F * 4 * kPseudoWarps, s>>>(A);
 }
 
 template <int DIM, int N, bool GEN, int SF>
 void launch_kap_stage(const KArgs& A, cudaStream_t s) {
-  kap_line<DIM, N, GEN, kLineWarps, SF>
-      <<<line_grid<DIM, N>(A.E), kLineWarps * 32, KAPLine<DIM, N>::F * 4 * kLineWarps, s>>>(A);
+  kap_line<DIM, N, GEN, kPseudoWarps, SF>
+      <<<line_grid<DIM, N>(A.E, kPseudoWarps), kPseudoWarps * 32, KAPLine<DIM, N, GEN>::F * 4 * kPseudoWarps, s>>>(A);
 }
 
 template <int DIM, int N, bool GEN>
@@ -80,7 +81,7 @@ void launch_ka_pseudo(const KArgs& A, cudaStream_t s) {
 
 template <int DIM, int N, bool GEN>
 bool fill_line_pseudo(KernelSet* ks) {
-  static_assert(KBPLine<DIM, N>::F * 4 * kLineWarps <= 48 * 1024 && KAPLine<DIM, N>::F * 4 * kLineWarps <= 48 * 1024,
+  static_assert(KBPLine<DIM, N, GEN>::F * 4 * kPseudoWarps <= 48 * 1024 && KAPLine<DIM, N, GEN>::F * 4 * kPseudoWarps <= 48 * 1024,
                 "no shared-memory opt-in needed");
   ks->kb[1] = launch_kb_pseudo<DIM, N, GEN>;
   ks->ka[1] = launch_ka_pseudo<DIM, N, GEN>;

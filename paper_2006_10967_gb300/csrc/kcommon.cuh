@@ -567,7 +567,17 @@ __device__ __forceinline__ void pseudo_rms_finish(const KArgs& A, double partial
   if (!last) return;
   __threadfence();
   double s = 0.0;
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) s += ((volatile double*)A.red)[b];
+  // sixteen loads in flight a thread: with one at a time the last block spent
+  // 48 us on the 8,000 partials of 64,000 hexahedra
+  int b = threadIdx.x;
+  for (; b + 15 * (int)blockDim.x < (int)gridDim.x; b += 16 * blockDim.x) {
+    double v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __ldcg(A.red + b + i * blockDim.x);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) s += v[i];
+  }
+  for (; b < (int)gridDim.x; b += blockDim.x) s += __ldcg(A.red + b);
   s = block_sum(s, sh);
   if (threadIdx.x == 0) {
     const double rms = sqrt(s / (double)ndof);

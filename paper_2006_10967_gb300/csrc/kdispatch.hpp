@@ -35,9 +35,12 @@ bool line_kernels_hex(int order, bool gen, KernelSet* ks);
 bool line_pseudo_quad(int order, bool gen, KernelSet* ks);
 bool line_pseudo_hex(int order, bool gen, KernelSet* ks);
 
-// Warps a block of the line kernels: the element balances and reductions take
-// FP64 once a block, so a block holds several warps.
-constexpr int kLineWarps = 4;
+// Warps a block of the line kernels.  Their warps are independent, so small
+// blocks spread best (64^3 hexes p = 3, residual + update: 185 + 183 us with
+// four, 183 + 178 with two); the preconditioning's stage 4 leaves one partial a
+// block for the last block to add up and takes four (stage 4 of 64^3: with two
+// warps a block the update kernel's mean goes from 122 to 151 us).
+constexpr int kLineWarps = 2, kPseudoWarps = 4;
 
 template <typename K>
 inline void launch_kernel(K kern, size_t smem, int et, const KArgs& A, cudaStream_t s, int threads = kThreads) {

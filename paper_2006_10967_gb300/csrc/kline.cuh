@@ -169,9 +169,33 @@ __device__ __forceinline__ void cp_async_8(void* sdst, const void* gsrc) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(sdst);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(gsrc) : "memory");
 }
-__device__ __forceinline__ void warp_fetch(float* dst, const void* src, int nfloats, int lane) {
-  const float2* s = static_cast<const float2*>(src);
-  for (int i = lane; i < nfloats / 2; i += 32) cp_async_8(dst + 2 * i, s + i);
+// A tile's share of an array of PER bytes an element, ne of at most EPW
+// elements: whole tiles in a compile-time count of the widest words that every
+// tile's start allows (arrays start on 256-byte boundaries).
+// `dst` is on a 16-byte boundary (every buffer offset is a multiple of 4 floats).
+template <int EPW, int PER>
+__device__ __forceinline__ void tile_fetch(float* dst, const void* src, int ne, int lane) {
+  constexpr int FULL = EPW * PER, W = FULL % 16 == 0 ? 16 : FULL % 8 == 0 ? 8 : 4;
+  char* d = reinterpret_cast<char*>(dst);
+  const char* s = static_cast<const char*>(src);
+  if (ne == EPW) {
+#pragma unroll
+    for (int r = 0; r < (FULL / W + 31) / 32; ++r) {
+      const int i = r * 32 + lane;
+      if (i < FULL / W) {
+        if constexpr (W == 16) cp_async_16(d + 16 * i, s + 16 * i);
+        else if constexpr (W == 8) cp_async_8(d + 8 * i, s + 8 * i);
+        else cp_async_4(d + 4 * i, s + 4 * i);
+      }
+    }
+  } else {
+    for (int i = lane; i < ne * PER / 4; i += 32) cp_async_4(d + 4 * i, s + 4 * i);
+  }
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int LEFT>
+__device__ __forceinline__ void cp_async_wait_but() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(LEFT) : "memory");
 }
 __device__ __forceinline__ void warp_flush(void* dst, const float* src, int nfloats, int lane) {
   float2* d = static_cast<float2*>(dst);
@@ -212,15 +236,15 @@ __device__ __forceinline__ void jac_col(const float* g, int b, const float2* xi,
   for (int c = 0; c < DIM; ++c) {
     if (DIM == 2) {
       const float* k = g + c * 4;
-      J[c] = fma2(dup2(__ldg(k + 3)), xi[1 - b], dup2(__ldg(k + 1 + b)));
+      J[c] = fma2(dup2(k[3]), xi[1 - b], dup2(k[1 + b]));
     } else {
       const float* k = g + c * 8;
       // other axes p < q; cross coefficients k4 (01), k5 (02), k6 (12), k7 (012)
       const int p = b == 0 ? 1 : 0, q = b == 2 ? 1 : 2;
-      const float kp = __ldg(k + (b == 2 ? 5 : 4));  // with axis p: (01), (01), (02)
-      const float kq = __ldg(k + (b == 0 ? 5 : 6));  // with axis q: (02), (12), (12)
-      const float2 t = fma2(dup2(__ldg(k + 7)), xi[q], dup2(kp));
-      J[c] = fma2(t, xi[p], fma2(dup2(kq), xi[q], dup2(__ldg(k + 1 + b))));
+      const float kp = k[b == 2 ? 5 : 4];  // with axis p: (01), (01), (02)
+      const float kq = k[b == 0 ? 5 : 6];  // with axis q: (02), (12), (12)
+      const float2 t = fma2(dup2(k[7]), xi[q], dup2(kp));
+      J[c] = fma2(t, xi[p], fma2(dup2(kq), xi[q], dup2(k[1 + b])));
     }
   }
 }
@@ -273,14 +297,14 @@ __device__ __forceinline__ float2 metric_all(const float* g, const float2* xi, f
 }
 __device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(1.f / a.x, 1.f / a.y); }
 
-// Multiplier max(|v|, gamma) and the sharpening factor -gamma u (1 - u) / max(|q|, delta)
+// Multiplier max(|v|, gamma) and the sharpening factor gamma u (1 - u) / max(|q|, delta)
 // for a pair: v2 = |v|^2, g2 = |q|^2.
 __device__ __forceinline__ float2 flux_mult(float2 v2, float gamma) {
   return make_float2(fmaxf(sqrtf(v2.x), gamma), fmaxf(sqrtf(v2.y), gamma));
 }
-__device__ __forceinline__ float2 neg_sharp(float2 u, float2 g2, float gamma, float rdelta) {
+__device__ __forceinline__ float2 sharp2(float2 u, float2 g2, float gamma, float rdelta) {
   const float2 r = make_float2(fminf(rsqrtf(g2.x), rdelta), fminf(rsqrtf(g2.y), rdelta));
-  const float2 w = fma2(u, u, make_float2(-u.x, -u.y));  // -u (1 - u)
+  const float2 w = mul2(u, sub2(dup2(1.f), u));
   return mul2(mul2(dup2(gamma), w), r);
 }
 
@@ -324,19 +348,29 @@ __global__ void k_vel_tab(const KArgs A) {
 // each element takes that path or the general one (metric from the map's
 // coefficients, velocity from the point cache), by its own flag, so that an
 // element's result does not depend on what else is in the mesh.
-template <int DIM, int N>
+template <int DIM, int N, bool GEN>
 struct KBLine {
   using L = LL<DIM, N>;
   static constexpr int WARP_F = (2 * (1 + DIM) * L::AS) * L::EPW;  // floats a warp
   static constexpr int IN_F = L::DIRECT ? 0 : ((L::EPW * 2 * L::NU + 3) / 4) * 4;
-  // the state's input buffer and the result's output buffer overlay the arrays
-  static constexpr int F = (WARP_F + 3) / 4 * 4 + IN_F;
+  // read in the middle of the tile, copied in at its start: the velocity table
+  // and, on the general path, the point velocities and the map coefficients
+  static constexpr int TAB_F = (L::EPW * DIM * (N + 2) * 2 + 3) / 4 * 4;
+  static constexpr int VF_F = GEN ? (L::EPW * DIM * L::NF + 3) / 4 * 4 : 0;
+  static constexpr int VU_F = GEN ? (L::EPW * DIM * L::NU + 3) / 4 * 4 : 0;
+  static constexpr int GEO_F = GEN ? L::EPW * L::S::NG : 0;
+  static constexpr int O_IN = (WARP_F + 3) / 4 * 4, O_TAB = O_IN + IN_F, O_VF = O_TAB + TAB_F, O_VU = O_VF + VF_F,
+                       O_GEO = O_VU + VU_F;
+  static constexpr int F = O_GEO + GEO_F;
+  static_assert(O_IN % 4 == 0 && O_TAB % 4 == 0 && O_VF % 4 == 0 && O_VU % 4 == 0 && O_GEO % 4 == 0 && F % 4 == 0,
+                "16-byte boundaries");
 };
 
-template <int DIM, int N, bool GEN, int WPB>
+// NPHI: the interface normal comes from phi (the unpreconditioned method).
+template <int DIM, int N, bool GEN, bool NPHI, int WPB>
 __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
   using L = LL<DIM, N>;
-  using K = KBLine<DIM, N>;
+  using K = KBLine<DIM, N, GEN>;
   constexpr int NU = L::NU, NF = L::NF, NFP = L::NFP, LN = L::LN, EPW = L::EPW, NP = L::NP, AS = L::AS;
   constexpr int NT = N + 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -360,9 +394,10 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
     for (int f = 0; f < 2; ++f)
       grow_get<N>(reinterpret_cast<const float*>(A.ustg) + (e * 2 + f) * NU + l * N, u[f]);
   } else {
-    float* in = wsm + (K::WARP_F + 3) / 4 * 4;
-    const int ne = (int)min((int64_t)EPW, A.E - e0);
-    if (ne > 0) warp_fetch(in, reinterpret_cast<const float*>(A.ustg) + e0 * 2 * NU, ne * 2 * NU, lane);
+    float* in = wsm + K::O_IN;
+    const int ne = (int)max((int64_t)0, min((int64_t)EPW, A.E - e0));
+    tile_fetch<EPW, 2 * NU * 4>(in, reinterpret_cast<const float*>(A.ustg) + e0 * 2 * NU, ne, lane);
+    cp_async_commit();
   }
   int fl[DIM][2];
   float2 o[DIM][2];
@@ -404,6 +439,16 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
       o[a][1] = make_float2(t[1][0], t[1][1]);
     }
   }
+  {
+    const int ne = (int)max((int64_t)0, min((int64_t)EPW, A.E - e0));
+    if (!GEN || A.vtab) tile_fetch<EPW, DIM * NT * 8>(wsm + K::O_TAB, A.vtab + e0 * DIM * NT, ne, lane);
+    if constexpr (GEN) {
+      tile_fetch<EPW, DIM * NF * 4>(wsm + K::O_VF, reinterpret_cast<const float*>(A.vsf) + e0 * DIM * NF, ne, lane);
+      tile_fetch<EPW, DIM * NU * 4>(wsm + K::O_VU, reinterpret_cast<const float*>(A.vsu) + e0 * DIM * NU, ne, lane);
+      tile_fetch<EPW, L::S::NG * 4>(wsm + K::O_GEO, A.geof + e0 * L::S::NG, ne, lane);
+    }
+    cp_async_commit();
+  }
   const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
   const bool diag = !GEN || (A.vtab != nullptr && __ldg(mc + 11) == 2.f);
   float sd[DIM];  // S_aa of the diagonal metric
@@ -423,9 +468,9 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
     eps = P.eps;
   }
   if constexpr (!L::DIRECT) {
-    cp_async_wait_all();
+    cp_async_wait_but<1>();  // the state; the rest follows before the faces
     __syncwarp();
-    const float* in = wsm + (K::WARP_F + 3) / 4 * 4;
+    const float* in = wsm + K::O_IN;
 #pragma unroll
     for (int f = 0; f < 2; ++f) grow_get<N>(in + (es * 2 + f) * NU + l * N, u[f]);
   }
@@ -486,8 +531,9 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
     }
   }
   // the other fields' faces need the axis-0 component of the field that gives the normal
-  const int kn = P.nphi ? 0 : 1;
-  if (lane_ok && diag) row_put<NP>(Q + (kn * DIM) * FA + pline<DIM, N>(0, l), P.nphi ? q[0][0] : q[1][0]);
+  constexpr int kn = NPHI ? 0 : 1;
+  if (lane_ok && diag) row_put<NP>(Q + (kn * DIM) * FA + pline<DIM, N>(0, l), q[kn][0]);
+  cp_async_wait_all();
   __syncwarp();
 #pragma unroll
   for (int f = 0; f < 2; ++f)
@@ -497,7 +543,7 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
   int lc[3];  // the lane's point coordinates on axes 1, 2
   lc[1] = DIM == 3 ? l % N : l;
   lc[2] = DIM == 3 ? l / N : 0;
-  const float* geo = A.geof + e * L::S::NG;
+  const float* geo = wsm + K::O_GEO + es * L::S::NG;
   if (GEN && !diag) {
     // physical gradient q_b = sum_a S[a][b] q~_a / det J, kept in registers and in the rows
 #pragma unroll
@@ -531,7 +577,7 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
   if (GEN) __syncwarp();
 
   // ---- Step 5: the common flux at both ends of the lane's line of every axis ---
-  const float2* vt = diag ? A.vtab + e * DIM * NT : nullptr;  // (A, B) per axis and coordinate
+  const float2* vt = reinterpret_cast<const float2*>(wsm + K::O_TAB) + es * DIM * NT;  // (A, B) per axis and coordinate
   const float gv = P.vel_g ? gfac : 1.f;
   float2 cor[DIM][2];
 #pragma unroll
@@ -543,13 +589,13 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
     if (diag) {
       // the transformed normal is -+S_aa e_a: q along axis a of both fields,
       // and the whole gradient of the field that gives the normal
-      const float2 qn = P.nphi ? qe[a][0] : qe[a][1];
+      const float2 qn = qe[a][kn];
       float2 g2 = mul2(qn, qn);
 #pragma unroll
       for (int b = 0; b < DIM; ++b) {
         if (b == a) continue;
         float v[N];
-        if (a == 0) unpair<N>(P.nphi ? q[0][b] : q[1][b], v);
+        if (a == 0) unpair<N>(q[kn][b], v);
         else if (a == 1) line_get<N, pstride<DIM, N>(1)>(Q + (kn * DIM + b) * FA + pline<DIM, N>(1, l), v);
         else line_get<N, pstride<DIM, N>(2)>(Q + (kn * DIM + b) * FA + pline<DIM, N>(2, l), v);
         const float2 t = line_ends<N>(O, v);
@@ -565,13 +611,13 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
 #pragma unroll
         for (int b = 0; b < DIM; ++b) {
           if (b == a) continue;
-          const float2 ab = __ldg(vt + b * NT + (i == 0 ? (DIM == 2 ? l : j1) : j2));
+          const float2 ab = vt[b * NT + (i == 0 ? (DIM == 2 ? l : j1) : j2)];
           ++i;
 #pragma unroll
           for (int c = 0; c < DIM; ++c) kc[c] = __fmul_rn(kc[c], c == b ? ab.x : ab.y);
         }
       }
-      const float2 e0v = __ldg(vt + a * NT + N), e1v = __ldg(vt + a * NT + N + 1);
+      const float2 e0v = vt[a * NT + N], e1v = vt[a * NT + N + 1];
       const float2 Ae = make_float2(e0v.x, e1v.x), Be = make_float2(e0v.y, e1v.y);
       float ko = 0.f;  // sum of the other components' squares
 #pragma unroll
@@ -580,11 +626,11 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
       const float2 va = mul2(Ae, dup2(kc[a]));
       const float2 v2 = fma2(va, va, mul2(mul2(Be, Be), dup2(ko)));
       const float2 M = flux_mult(v2, P.gamma);
-      const float2 ns = neg_sharp(pL, g2, P.gamma, P.rdelta);
-      const float2 vis = mul2(M, fma2(ns, qn, mul2(dup2(eps), qe[a][0])));
+      const float2 sh = sharp2(pL, g2, P.gamma, P.rdelta);
+      const float2 nvis = fma2(sh, qn, mul2(dup2(-eps), qe[a][0]));  // minus the viscous flux over M
       const float saa = sd[a], pm = fabsf(saa);
       const float2 sg = make_float2(-saa, saa);
-      Fp = fma2(dup2(__fmul_rn(pm, P.tau)), dp, mul2(sg, sub2(mul2(ap, va), vis)));
+      Fp = fma2(dup2(__fmul_rn(pm, P.tau)), dp, mul2(sg, fma2(M, nvis, mul2(ap, va))));
       Fs = fma2(dup2(__fmul_rn(pm, P.tau_psi)), ds, mul2(sg, mul2(as, va)));
     } else if (GEN) {
       float2 qf[2][DIM];
@@ -613,13 +659,13 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
       }
       metric_row<DIM>(geo, a, xi, Sr);
       const float2 sgn = make_float2(-1.f, 1.f);
-      const float* vf = reinterpret_cast<const float*>(A.vsf) + e * DIM * NF + 2 * a * NFP + l;
+      const float* vf = wsm + K::O_VF + es * DIM * NF + 2 * a * NFP + l;
       float2 vn = dup2(0.f), v2 = dup2(0.f), g2 = dup2(0.f), pm2 = dup2(0.f), qp = dup2(0.f), qs = dup2(0.f);
 #pragma unroll
       for (int c = 0; c < DIM; ++c) {
-        const float2 v = mul2(dup2(gfac), make_float2(__ldg(vf + c * NF), __ldg(vf + c * NF + NFP)));
+        const float2 v = mul2(dup2(gfac), make_float2(vf[c * NF], vf[c * NF + NFP]));
         const float2 pn = mul2(sgn, Sr[c]);
-        const float2 qn = P.nphi ? qf[0][c] : qf[1][c];
+        const float2 qn = qf[kn][c];
         vn = fma2(v, pn, vn);
         v2 = fma2(v, v, v2);
         pm2 = fma2(pn, pn, pm2);
@@ -629,9 +675,9 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
       }
       const float2 pm = make_float2(sqrtf(pm2.x), sqrtf(pm2.y));
       const float2 M = flux_mult(v2, P.gamma);
-      const float2 ns = neg_sharp(pL, g2, P.gamma, P.rdelta);
-      const float2 vis = mul2(M, fma2(ns, qs, mul2(dup2(eps), qp)));
-      Fp = fma2(mul2(pm, dup2(P.tau)), dp, sub2(mul2(ap, vn), vis));
+      const float2 sh = sharp2(pL, g2, P.gamma, P.rdelta);
+      const float2 nvis = fma2(sh, qs, mul2(dup2(-eps), qp));
+      Fp = fma2(mul2(pm, dup2(P.tau)), dp, fma2(M, nvis, mul2(ap, vn)));
       Fs = fma2(mul2(pm, dup2(P.tau_psi)), ds, mul2(as, vn));
     }
     // R ends carry no flux here (ka lifts minus the partner's); no-flux walls none at all
@@ -677,7 +723,7 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
       for (int c = 0; c < DIM; ++c) kc[c] = P.vs[c] * gv;
 #pragma unroll
       for (int b = 1; b < DIM; ++b) {
-        const float2 ab = __ldg(vt + b * NT + lc[b]);
+        const float2 ab = vt[b * NT + lc[b]];
 #pragma unroll
         for (int c = 0; c < DIM; ++c) kc[c] = __fmul_rn(kc[c], c == b ? ab.x : ab.y);
       }
@@ -690,18 +736,18 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
     for (int p = 0; p < NP; ++p) {
       float2 v[DIM], v2, Sm[3][3];
       if (diag) {
-        const float2 t0 = __ldg(vt + 2 * p), t1 = 2 * p + 1 < N ? __ldg(vt + 2 * p + 1) : make_float2(0.f, 0.f);
+        const float2 t0 = vt[2 * p], t1 = 2 * p + 1 < N ? vt[2 * p + 1] : make_float2(0.f, 0.f);
         const float2 Ax = make_float2(t0.x, t1.x), Bx = make_float2(t0.y, t1.y);
         v[0] = mul2(Ax, k[0]);
 #pragma unroll
         for (int c = 1; c < DIM; ++c) v[c] = mul2(Bx, k[c]);
         v2 = fma2(v[0], v[0], mul2(mul2(Bx, Bx), dup2(ko)));
       } else if (GEN) {
-        const float* vc = reinterpret_cast<const float*>(A.vsu) + e * DIM * NU + l * N + 2 * p;
+        const float* vc = wsm + K::O_VU + es * DIM * NU + l * N + 2 * p;
         v2 = dup2(0.f);
 #pragma unroll
         for (int c = 0; c < DIM; ++c) {
-          v[c] = mul2(dup2(gfac), make_float2(__ldg(vc + c * NU), 2 * p + 1 < N ? __ldg(vc + c * NU + 1) : 0.f));
+          v[c] = mul2(dup2(gfac), make_float2(vc[c * NU], 2 * p + 1 < N ? vc[c * NU + 1] : 0.f));
           v2 = fma2(v[c], v[c], v2);
         }
         float2 xi[3];
@@ -713,17 +759,16 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
       float2 qs[DIM], g2 = dup2(0.f);
 #pragma unroll
       for (int c = 0; c < DIM; ++c) {
-        qs[c] = P.nphi ? q[0][c][p] : q[1][c][p];
+        qs[c] = q[kn][c][p];
         g2 = fma2(qs[c], qs[c], g2);
       }
       const float2 M = flux_mult(v2, P.gamma);
-      const float2 nM = make_float2(-M.x, -M.y);
-      const float2 ns = neg_sharp(u[0][p], g2, P.gamma, P.rdelta);
+      const float2 sh = sharp2(u[0][p], g2, P.gamma, P.rdelta);
       float2 f0[DIM], f1[DIM];
 #pragma unroll
       for (int c = 0; c < DIM; ++c) {
-        const float2 t = fma2(ns, qs[c], mul2(dup2(eps), q[0][c][p]));
-        f0[c] = fma2(nM, t, mul2(u[0][p], v[c]));
+        const float2 t = fma2(sh, qs[c], mul2(dup2(-eps), q[0][c][p]));
+        f0[c] = fma2(M, t, mul2(u[0][p], v[c]));
         f1[c] = mul2(u[1][p], v[c]);
       }
 #pragma unroll
@@ -798,13 +843,13 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
     if constexpr (L::DIRECT) {
       if (act) grow_put<N>(rp + (e * 2 + f) * NU + l * N, dv[f]);
     } else if (lane_ok) {
-      grow_put<N>(wsm + (K::WARP_F + 3) / 4 * 4 + (es * 2 + f) * NU + l * N, dv[f]);
+      grow_put<N>(wsm + K::O_IN + (es * 2 + f) * NU + l * N, dv[f]);
     }
   }
   if constexpr (!L::DIRECT) {
     __syncwarp();
     const int ne = (int)min((int64_t)EPW, A.E - e0);
-    if (ne > 0) warp_flush(rp + e0 * 2 * NU, wsm + (K::WARP_F + 3) / 4 * 4, ne * 2 * NU, lane);
+    if (ne > 0) warp_flush(rp + e0 * 2 * NU, wsm + K::O_IN, ne * 2 * NU, lane);
   }
 }
 
@@ -812,7 +857,7 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
 // R-side lift, RK4 update and next-stage traces (ka_tensor's work), one line a
 // lane.  SF: the RK stage 1..4, or 0 to recompute the traces of ustg alone.
 // GEN false: every element is affine (1 / det J from the record).
-template <int DIM, int N, int SF>
+template <int DIM, int N, int SF, bool GEN>
 struct KALine {
   using L = LL<DIM, N>;
   // rows of both fields; face corrections of the axes > 0: [axis][end][field][other][row]
@@ -820,8 +865,14 @@ struct KALine {
   static constexpr int COR_F = (DIM - 1) * 2 * 2 * L::OTH * L::RS * L::EPW;
   // input and output buffer of the strided forms: rp (later the stage value), u, acc, w det J
   static constexpr int C = L::EPW * L::NU;
-  static constexpr int IN_F = L::DIRECT ? 0 : ((C * (2 + (SF >= 1 ? 4 : 0) + (SF >= 1 ? 2 : 0) + (SF == 4 ? 2 : 0)) + 3) / 4) * 4;
-  static constexpr int F = (ROWS_F + 3) / 4 * 4 + (SF >= 1 ? (COR_F + 3) / 4 * 4 : 0) + IN_F;
+  static constexpr int O_U = (2 * C + 3) / 4 * 4, O_A = (O_U + 4 * C + 3) / 4 * 4;  // 16-byte boundaries
+  static constexpr int IN_F = L::DIRECT ? 0 : SF == 0 ? O_U : (O_A + 2 * C + 3) / 4 * 4;
+  static constexpr int O_IN = (ROWS_F + 3) / 4 * 4 + (SF >= 1 ? (COR_F + 3) / 4 * 4 : 0);
+  // stage 4: w det J pairs; general path: the map coefficients
+  static constexpr int O_W = O_IN + IN_F, O_GEO = O_W + (SF == 4 ? (2 * C + 3) / 4 * 4 : 0);
+  static constexpr int F = O_GEO + (SF >= 1 && GEN ? L::EPW * L::S::NG : 0);
+  static_assert(O_IN % 4 == 0 && O_U % 4 == 0 && O_A % 4 == 0 && O_W % 4 == 0 && O_GEO % 4 == 0 && F % 4 == 0,
+                "16-byte boundaries");
 };
 
 // (hi, lo) += f: error-free sum of the high parts, the errors beside
@@ -885,9 +936,10 @@ __device__ __forceinline__ void line_tree(float2& a, float2& b, int l) {
 template <int DIM, int N, bool GEN, int WPB, int SF>
 __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(const KArgs A) {
   using L = LL<DIM, N>;
-  using K = KALine<DIM, N, SF>;
+  using K = KALine<DIM, N, SF, GEN>;
   constexpr int NU = L::NU, NF = L::NF, NFP = L::NFP, LN = L::LN, EPW = L::EPW, NP = L::NP, AS = L::AS;
-  constexpr int NEL = WPB * EPW;
+  constexpr int NEL = WPB * EPW;  // at most 16 elements a warp: one thread an element and field
+  static_assert(2 * NEL <= WPB * 32, "the block's threads finish the elements' balances");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ float2 balS[SF >= 1 ? 2 * NEL : 1];  // element flux balances
   __shared__ float2 incS[SF == 4 ? 2 * NEL : 1];  // stage 4: element sums of w det J * increment
@@ -937,11 +989,21 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
     }
   } else if (ne > 0) {
     const float* src = SF == 0 ? ustg : reinterpret_cast<const float*>(A.rp);
-    warp_fetch(in, src + e0 * 2 * NU, ne * 2 * NU, lane);
-    if constexpr (SF >= 1) warp_fetch(in + K::C * 2, U + e0 * 2 * NU, ne * 4 * NU, lane);
-    if constexpr (SF >= 2) warp_fetch(in + K::C * 6, acc + e0 * 2 * NU, ne * 2 * NU, lane);
-    if constexpr (SF == 4)
-      if (cons) warp_fetch(in + K::C * 8, A.wdetf + e0 * NU, ne * 2 * NU, lane);
+    tile_fetch<EPW, 2 * NU * 4>(in, src + e0 * 2 * NU, ne, lane);
+    if constexpr (SF >= 1) tile_fetch<EPW, 2 * NU * 8>(in + K::O_U, U + e0 * 2 * NU, ne, lane);
+    if constexpr (SF >= 2) tile_fetch<EPW, 2 * NU * 4>(in + K::O_A, acc + e0 * 2 * NU, ne, lane);
+    cp_async_commit();
+  }
+  if constexpr (SF >= 1) {
+    if (SF == 4 && cons && ne > 0) tile_fetch<EPW, NU * 8>(wsm + K::O_W, A.wdetf + e0 * NU, ne, lane);
+    if (GEN && ne > 0) tile_fetch<EPW, L::S::NG * 4>(wsm + K::O_GEO, A.geof + e0 * L::S::NG, ne, lane);
+    cp_async_commit();
+  }
+  float aff = 1.f, rdet = 0.f;  // record: affine flag, 1 / det J
+  if constexpr (SF >= 1) {
+    const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
+    rdet = __ldg(mc + 10);
+    if (GEN) aff = DIM == 3 ? __ldg(mc + 11) : 0.f;
   }
   int fl[DIM][2];
   [[maybe_unused]] int32_t w2[DIM][2];
@@ -994,11 +1056,15 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
   }
   double ta = 0.0;  // this thread's element balance so far (finished by the first threads of the block)
   const int64_t gt = (int64_t)blockIdx.x * NEL * 2 + threadIdx.x;
-  if (SF >= 2 && cons && threadIdx.x < 2 * NEL && gt < 2 * A.E) ta = A.tacc[gt];
+  float2 rW = make_float2(0.f, 0.f);  // stage 4: 1 / W
+  if (SF >= 2 && cons && threadIdx.x < 2 * NEL && gt < 2 * A.E) {
+    ta = A.tacc[gt];
+    if (SF == 4) rW = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(A.mcg) + (gt / 2) * kMetricRec + 12);
+  }
   [[maybe_unused]] RKConstF rk;
   if constexpr (SF >= 1) rk = A.ep ? A.ep[e].rk : A.rk;
   if constexpr (!L::DIRECT) {
-    cp_async_wait_all();
+    cp_async_wait_but<(SF >= 1)>();
     __syncwarp();
 #pragma unroll
     for (int f = 0; f < 2; ++f) {
@@ -1006,10 +1072,10 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
       grow_get<N>(in + r, y[f]);
       if constexpr (SF >= 1)
 #pragma unroll
-        for (int j = 0; j < N; ++j) u[f][j] = reinterpret_cast<const float2*>(in + K::C * 2)[r + j];
+        for (int j = 0; j < N; ++j) u[f][j] = reinterpret_cast<const float2*>(in + K::O_U)[r + j];
       if constexpr (SF >= 2)
 #pragma unroll
-        for (int j = 0; j < N; ++j) ac[f][j] = in[K::C * 6 + r + j];
+        for (int j = 0; j < N; ++j) ac[f][j] = in[K::O_A + r + j];
     }
   }
 
@@ -1053,6 +1119,7 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
       if (lane_ok && l == 0) balS[(warp * EPW + es) * 2] = v[0];
       if (lane_ok && l == LineTree<LN>::LB) balS[(warp * EPW + es) * 2 + 1] = v[1];
     }
+    cp_async_wait_all();
     __syncwarp();
     const int lc1 = DIM == 3 ? l % N : l, lc2 = l / N;
     float gl[3], gr[3];
@@ -1064,10 +1131,9 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
     }
     float2 rdj[NP];
     if (GEN) {
-      const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
-      if (DIM == 3 && __ldg(mc + 11) != 0.f) {
+      if (DIM == 3 && aff != 0.f) {
 #pragma unroll
-        for (int p = 0; p < NP; ++p) rdj[p] = dup2(__ldg(mc + 10));
+        for (int p = 0; p < NP; ++p) rdj[p] = dup2(rdet);
       } else {
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
@@ -1075,13 +1141,12 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
           xi[0] = O.xp[p];
           xi[1] = dup2(A.cf.ops.x[lc1]);
           xi[2] = dup2(A.cf.ops.x[DIM == 3 ? lc2 : 0]);
-          rdj[p] = rcp2(metric_all<DIM>(A.geof + e * L::S::NG, xi, Sm));
+          rdj[p] = rcp2(metric_all<DIM>(wsm + K::O_GEO + es * L::S::NG, xi, Sm));
         }
       }
     } else {
-      const float r = __ldg(reinterpret_cast<const float*>(A.mcg) + e * kMetricRec + 10);
 #pragma unroll
-      for (int p = 0; p < NP; ++p) rdj[p] = dup2(r);
+      for (int p = 0; p < NP; ++p) rdj[p] = dup2(rdet);
     }
     float bad = 0.f;   // becomes NaN when a new value is not finite
     float inc[2][N];   // stage 4: the increments
@@ -1138,17 +1203,8 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
         float2 wd[2 * NP], v[2];
 #pragma unroll
         for (int j = 0; j < 2 * NP; ++j) wd[j] = make_float2(0.f, 0.f);
-        if constexpr (L::DIRECT) {
 #pragma unroll
-          for (int j = 0; j < N; j += 2) {
-            const float4 t = *reinterpret_cast<const float4*>(A.wdetf + e * NU + l * N + j);
-            wd[j] = make_float2(t.x, t.y);
-            wd[j + 1] = make_float2(t.z, t.w);
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < N; ++j) wd[j] = reinterpret_cast<const float2*>(in + K::C * 8)[es * NU + l * N + j];
-        }
+        for (int j = 0; j < N; ++j) wd[j] = reinterpret_cast<const float2*>(wsm + K::O_W)[es * NU + l * N + j];
 #pragma unroll
         for (int f = 0; f < 2; ++f) {
           float2 sh = dup2(0.f), sl = dup2(0.f);
@@ -1163,15 +1219,13 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
         if (lane_ok && l == 0) incS[(warp * EPW + es) * 2] = v[0];
         if (lane_ok && l == LineTree<LN>::LB) incS[(warp * EPW + es) * 2 + 1] = v[1];
         __syncthreads();
-        for (int t = threadIdx.x; t < 2 * NEL; t += WPB * 32) {
+        if (const int t = threadIdx.x; t < 2 * NEL) {
           const int64_t g = (int64_t)blockIdx.x * NEL * 2 + t;
           if (g < 2 * A.E) {
-            const float* mc = reinterpret_cast<const float*>(A.mcg) + (g / 2) * kMetricRec;
             const double Te = -((double)balS[t].x + (double)balS[t].y);
-            const double prev = t == (int)threadIdx.x ? ta : A.tacc[g];
-            const double tgt = (A.ep ? A.ep[g / 2].rk.ddt6 : A.rk.ddt6) * (prev + Te);
-            const double S = (double)incS[t].x + (double)incS[t].y, rW = (double)mc[12] + (double)mc[13];
-            const double d = (tgt - S) * rW;
+            const double tgt = (A.ep ? A.ep[g / 2].rk.ddt6 : A.rk.ddt6) * (ta + Te);
+            const double S = (double)incS[t].x + (double)incS[t].y;
+            const double d = (tgt - S) * ((double)rW.x + (double)rW.y);
             const float dh = (float)d;
             dltS[t] = make_float2(dh, (float)(d - (double)dh));
           }
@@ -1223,16 +1277,16 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
           grow_put<N>(in + r, y[f]);
 #pragma unroll
           for (int j = 0; j < N; ++j) {
-            if constexpr (SF < 4) in[K::C * 6 + r + j] = ac[f][j];
-            else reinterpret_cast<float2*>(in + K::C * 2)[r + j] = u[f][j];
+            if constexpr (SF < 4) in[K::O_A + r + j] = ac[f][j];
+            else reinterpret_cast<float2*>(in + K::O_U)[r + j] = u[f][j];
           }
         }
       }
       __syncwarp();
       if (ne > 0) {
         warp_flush(ustg + e0 * 2 * NU, in, ne * 2 * NU, lane);
-        if constexpr (SF < 4) warp_flush(acc + e0 * 2 * NU, in + K::C * 6, ne * 2 * NU, lane);
-        else warp_flush(U + e0 * 2 * NU, in + K::C * 2, ne * 4 * NU, lane);
+        if constexpr (SF < 4) warp_flush(acc + e0 * 2 * NU, in + K::O_A, ne * 2 * NU, lane);
+        else warp_flush(U + e0 * 2 * NU, in + K::O_U, ne * 4 * NU, lane);
       }
     }
   }
@@ -1274,12 +1328,11 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
     if (cons) {
       // element mass rates, accumulated with the RK4 weights in FP64 by the block's first threads
       __syncthreads();
-      for (int t = threadIdx.x; t < 2 * NEL; t += WPB * 32) {
+      if (const int t = threadIdx.x; t < 2 * NEL) {
         const int64_t g = (int64_t)blockIdx.x * NEL * 2 + t;
         if (g < 2 * A.E) {
           const double Te = -((double)balS[t].x + (double)balS[t].y);
-          const double prev = SF == 1 ? 0.0 : (t == (int)threadIdx.x ? ta : A.tacc[g]);
-          A.tacc[g] = SF == 1 ? Te : prev + 2.0 * Te;
+          A.tacc[g] = SF == 1 ? Te : ta + 2.0 * Te;
         }
       }
     }

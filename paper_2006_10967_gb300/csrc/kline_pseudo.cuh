@@ -23,12 +23,14 @@ __device__ __forceinline__ void rows_flush(float* dst, const float* src, int pit
   for (int i = lane; i < ne * NU; i += 32) dst[(i / NU) * pitch + i % NU] = src[i];
 }
 
-template <int DIM, int N>
+template <int DIM, int N, bool GEN>
 struct KBPLine {
   using L = LL<DIM, N>;
   static constexpr int WARP_F = (2 + DIM) * L::AS * L::EPW;  // psi, modes, gradient
   static constexpr int IN_F = L::DIRECT ? 0 : (L::EPW * L::NU + 3) / 4 * 4;
-  static constexpr int F = (WARP_F + 3) / 4 * 4 + IN_F;
+  static constexpr int O_GEO = (WARP_F + 3) / 4 * 4 + IN_F;
+  static constexpr int F = O_GEO + (GEN ? L::EPW * L::S::NG : 0);
+  static_assert(O_GEO % 4 == 0 && F % 4 == 0, "16-byte boundaries");
 };
 
 // quotient of two float-float values
@@ -91,7 +93,7 @@ __device__ __forceinline__ float sensor_nu(const PhysPrm& P, float2 lo, float2 h
 template <int DIM, int N, bool GEN, int WPB>
 __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / WPB) kbp_line(const KArgs A) {
   using L = LL<DIM, N>;
-  using K = KBPLine<DIM, N>;
+  using K = KBPLine<DIM, N, GEN>;
   constexpr int NU = L::NU, NF = L::NF, NFP = L::NFP, LN = L::LN, EPW = L::EPW, NP = L::NP, AS = L::AS;
   if (*(volatile int32_t*)&A.status[ST_PSEUDO_DONE]) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -114,6 +116,8 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
   const float* ug = reinterpret_cast<const float*>(A.ustg);
   if constexpr (L::DIRECT) grow_get<N>(ug + (e * 2 + 1) * NU + l * N, u);
   else rows_fetch<NU>(in, ug + (e0 * 2 + 1) * NU, 2 * NU, ne, lane);
+  cp_async_commit();
+  if (GEN && ne > 0) tile_fetch<EPW, L::S::NG * 4>(wsm + K::O_GEO, A.geof + e0 * L::S::NG, ne, lane);
   int fl[DIM][2];
   float2 o[DIM];
   [[maybe_unused]] int32_t w2[DIM][2];
@@ -167,10 +171,11 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
   for (int a = 0; a < DIM; ++a) sd[a] = __ldg(mc + a * 4);
   const float det = __ldg(mc + 9), rdet = __ldg(mc + 10);
   if constexpr (!L::DIRECT) {
-    cp_async_wait_all();
+    cp_async_wait_but<0>();
     __syncwarp();
     grow_get<N>(in + es * NU + l * N, u);
   }
+  if (GEN) cp_async_wait_all();
 
   constexpr int FA = AS * EPW;
   float* U = wsm + es * AS;
@@ -287,7 +292,7 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
   for (int a = 1; a < DIM; ++a) row_get<NP>(Q + a * FA + pline<DIM, N>(0, l), q[a]);
 
   const int lc1 = DIM == 3 ? l % N : l, lc2 = DIM == 3 ? l / N : 0;
-  const float* geo = A.geof + e * L::S::NG;
+  const float* geo = wsm + K::O_GEO + es * L::S::NG;
   float2 xi[3];
   xi[1] = dup2(A.cf.ops.x[lc1]);
   xi[2] = dup2(A.cf.ops.x[lc2]);
@@ -450,7 +455,7 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
 }
 
 // ---- update kernel ---------------------------------------------------------------
-template <int DIM, int N>
+template <int DIM, int N, bool GEN>
 struct KAPLine {
   using L = LL<DIM, N>;
   static constexpr int ROWS_F = (L::AS * L::EPW + 3) / 4 * 4;
@@ -458,7 +463,9 @@ struct KAPLine {
   // input and output buffer of the strided forms: the rate (later the stage value), accumulator, solution pairs
   static constexpr int C = (L::EPW * L::NU + 3) / 4 * 4;
   static constexpr int IN_F = L::DIRECT ? 0 : 4 * C;
-  static constexpr int F = ROWS_F + COR_F + IN_F;
+  static constexpr int O_GEO = ROWS_F + COR_F + IN_F;
+  static constexpr int F = O_GEO + (GEN ? L::EPW * L::S::NG : 0);
+  static_assert(O_GEO % 4 == 0 && F % 4 == 0, "16-byte boundaries");
 };
 
 // SF: stage 1..4, or 0 to recompute the traces of psi alone.  GEN false: every
@@ -466,7 +473,7 @@ struct KAPLine {
 template <int DIM, int N, bool GEN, int WPB, int SF>
 __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
   using L = LL<DIM, N>;
-  using K = KAPLine<DIM, N>;
+  using K = KAPLine<DIM, N, GEN>;
   constexpr int NU = L::NU, NF = L::NF, NFP = L::NFP, LN = L::LN, EPW = L::EPW, NP = L::NP;
   if (*(volatile int32_t*)&A.status[ST_PSEUDO_DONE]) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -514,6 +521,10 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
     if constexpr (SF >= 1)
       for (int i = lane; i < ne * NU; i += 32) cp_async_8(in + 2 * K::C + 2 * i, U + r0 + (i / NU) * 2 * NU + i % NU);
   }
+  if (GEN && SF >= 1 && ne > 0) tile_fetch<EPW, L::S::NG * 4>(R0 + K::O_GEO, A.geof + e0 * L::S::NG, ne, lane);
+  const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
+  const float rdet = __ldg(mc + 10);
+  const bool aff = !GEN || (DIM == 3 && __ldg(mc + 11) != 0.f);
   int fl[DIM][2];
   float2 F[DIM];
   [[maybe_unused]] int32_t w2[DIM][2];
@@ -551,8 +562,8 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
       F[a] = make_float2(t[0], t[1]);
     }
   }
+  if constexpr (!L::DIRECT || GEN) cp_async_wait_all();
   if constexpr (!L::DIRECT) {
-    cp_async_wait_all();
     __syncwarp();
     const int rl = es * NU + l * N;
     grow_get<N>(in + rl, y);
@@ -590,20 +601,18 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
 #pragma unroll
       for (int p = 0; p < NP; ++p) y[p] = fma2(dup2(gl), r0[p], fma2(dup2(gr), r1[p], y[p]));
     }
-    const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
-    const bool aff = !GEN || (DIM == 3 && __ldg(mc + 11) != 0.f);
     float bad = 0.f;
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       float2 rdj;
       if (aff) {
-        rdj = dup2(__ldg(mc + 10));
+        rdj = dup2(rdet);
       } else {
         float2 xi[3], Sm[3][3];
         xi[0] = O.xp[p];
         xi[1] = dup2(A.cf.ops.x[lc1]);
         xi[2] = dup2(A.cf.ops.x[lc2]);
-        rdj = rcp2(metric_all<DIM>(A.geof + e * L::S::NG, xi, Sm));
+        rdj = rcp2(metric_all<DIM>(R0 + K::O_GEO + es * L::S::NG, xi, Sm));
       }
       const float2 R = mul2(make_float2(-y[p].x, -y[p].y), rdj);
       float dh[2] = {0.f, 0.f}, dl[2] = {0.f, 0.f};
