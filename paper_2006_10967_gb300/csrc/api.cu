@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "field.cuh"
+#include "tripack.hpp"
 
 using namespace frp;
 
@@ -20,6 +21,7 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 struct Layout {
   size_t status, dstate, red, geo, geof, fnbr, wdet, ustg, u, acc, rp, tr, fc, psi0, xfer, vsu, vsf, tacc, wdetf, ep, mcg;
   size_t tri_d, tri_f, tri_high;  // dense triangle operators (double, float), mode mask
+  size_t tri_pack;                // their packed form (TriPack)
   size_t wphys;                   // triangles: physical edge quadrature weight per flux point (float-float)
   size_t ffw;                     // hexahedra: face words (KArgs.ffw)
   size_t vtab;                    // mixed tensor fields with a velocity cache: velocity factors (KArgs.vtab)
@@ -37,6 +39,23 @@ void pack_tri(const TriRef& t, std::vector<R>& out) {
   out.clear();
   for (const std::vector<double>* v : {&t.xu, &t.xf, &t.nref, &t.L, &t.Dr, &t.Ds, &t.LIFT, &t.Vinv})
     for (double x : *v) out.push_back((R)x);
+}
+
+// The operators as rows of output pairs (TriPack), pads zero.
+std::vector<float> pack_tri_pairs(const TriRef& t) {
+  const TriPack k(t.p);
+  std::vector<float> out(k.size, 0.f);
+  for (int j = 0; j < k.nu; ++j) {
+    for (int f = 0; f < k.nf; ++f) out[k.o_l + ((f / k.n) * k.nu + j) * k.npe * 2 + f % k.n] = (float)t.L[f * k.nu + j];
+    for (int i = 0; i < k.nu; ++i) {
+      out[k.o_d + j * k.npu * 2 + i] = (float)t.Dr[i * k.nu + j];
+      out[k.o_d + (k.nu + j) * k.npu * 2 + i] = (float)t.Ds[i * k.nu + j];
+      out[k.o_v + j * k.npu * 2 + i] = (float)t.Vinv[i * k.nu + j];
+    }
+  }
+  for (int f = 0; f < k.nf; ++f)
+    for (int i = 0; i < k.nu; ++i) out[k.o_lift + f * k.npu * 2 + i] = (float)t.LIFT[i * k.nf + f];
+  return out;
 }
 
 template <typename R>
@@ -211,6 +230,7 @@ Layout make_layout(const fr_mesh& m, int precision, int max_blocks, int vel_cach
     L.tri_d = take(nops * sizeof(double));
     L.tri_f = take(nops * sizeof(float));
     L.tri_high = take(NU);
+    L.tri_pack = take(TriPack(m.order).size * sizeof(float));
     L.wphys = take(E * NF * 2 * sizeof(float));
   }
   L.total = off;
@@ -800,13 +820,19 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
   std::vector<float> geof(m->geo.begin(), m->geo.end());
   up(L.geof, geof.data(), geof.size() * sizeof(float));
   std::vector<double> trid;
-  std::vector<float> trif;
+  std::vector<float> trif, tripack;
   if (m->etype == FR_TRI) {
     pack_tri(m->tri, trid);
     pack_tri(m->tri, trif);
     up(L.tri_d, trid.data(), trid.size() * sizeof(double));
     up(L.tri_f, trif.data(), trif.size() * sizeof(float));
     up(L.tri_high, m->tri.high.data(), m->tri.high.size());
+    tripack = pack_tri_pairs(m->tri);
+    up(L.tri_pack, tripack.data(), tripack.size() * sizeof(float));
+    A.tripack = reinterpret_cast<const float*>(b + L.tri_pack);
+    // variant 0 of the mixed path at p <= 4 (variant 1: tensor cores; p = 5 has
+    // more values an element than a thread's registers)
+    if (prm->precision == FR_MIXED && prm->variant == 0 && m->order <= 4) reg_kernels_tri(m->order, prm->vel_cache, &f->ks);
     const uint8_t* hi = reinterpret_cast<const uint8_t*>(b + L.tri_high);
     A.trid = tri_pointers<double>(m->tri, reinterpret_cast<const double*>(b + L.tri_d), hi);
     A.trif = tri_pointers<float>(m->tri, reinterpret_cast<const float*>(b + L.tri_f), hi);

@@ -156,6 +156,7 @@ struct KArgs {
   BulkConst<double> cd;
   BulkConst<float> cf;
   LineOps lo;
+  const float* tripack;  // triangles: the operators in output pairs (TriPack)
   TriOpsT<double> trid;
   TriOpsT<float> trif;
 };

@@ -35,6 +35,11 @@ bool line_kernels_hex(int order, bool gen, KernelSet* ks);
 bool line_pseudo_quad(int order, bool gen, KernelSet* ks);
 bool line_pseudo_hex(int order, bool gen, KernelSet* ks);
 
+// Triangles of p <= 4 in mixed precision: the thread-per-element kernels for the
+// preconditioning and, when asked (the field has its velocity cache), the
+// physical step.
+bool reg_kernels_tri(int order, bool physical, KernelSet* ks);
+
 // Warps a block of the line kernels.  Their warps are independent, so small
 // blocks spread best (64^3 hexes p = 3, residual + update: 185 + 183 us with
 // four, 183 + 178 with two); the preconditioning's stage 4 leaves one partial a

@@ -124,3 +124,36 @@ def test_mixed_preconditioning_follows_fp64(G, etype, order, ns, jitter, vel, wa
     assert F.stats()["last_pseudo_iters"] == D.stats()["last_pseudo_iters"] == 3
     assert abs(F.stats()["last_pseudo_rms"] / D.stats()["last_pseudo_rms"] - 1) < 1e-4
     assert _rel(F.get(1), D.get(1)) < 1e-5
+
+
+TRIS = [(p, mk, vel, walls) for p in range(1, 5)
+        for mk, vel, walls in [(lambda: S.tri_split(1, 1, periodic=(False, False)), "uniform", True),
+                               (lambda: S.tri_split(7, 5, shuffle_seed=3), "stream", False),
+                               (lambda: S.tri_delaunay(9, seed=2, shuffle_seed=13), "rider_kothe", True)]]
+
+
+@pytest.mark.parametrize("order,mk,vel,walls", TRIS)
+@pytest.mark.parametrize("normal,wall", [("psi", "copy"), ("phi", "noflux")])
+def test_triangle_thread_kernels_agree_with_the_block_wide_ones(G, order, mk, vel, walls, normal, wall):
+    """Triangles of p <= 4 with the velocity cache (one thread an element)
+    against the same field without it (the block-wide kernels)."""
+    w, _ = _workload("quad", order, (8, 8), 0.0, vel, walls, normal, wall)
+    mesh = mk()
+    M = G.Mesh.from_synthetic(mesh, order)
+    F, B = [G.Field(M, G.make_params(w, "mixed", vel_cache=c, pseudo_fixed=True, normal=normal, wall=wall), ic=w.circle)
+            for c in (True, False)]
+    D = G.Field(M, G.make_params(w, "fp64", pseudo_fixed=True, normal=normal, wall=wall), ic=w.circle)
+    if normal == "psi":
+        assert _rel(F.rhs_pseudo().cpu().numpy(), D.rhs_pseudo().cpu().numpy()) < 1e-4
+        assert abs(F.stats()["last_pseudo_rms"] / D.stats()["last_pseudo_rms"] - 1) < 1e-4
+    R, Rb = F.rhs(0.3).cpu().numpy(), B.rhs(0.3).cpu().numpy()
+    for f in (0, 1):
+        assert _rel(R[f], Rb[f]) < 2e-4
+    m0 = F.mass(0)
+    for f in (F, B):
+        f.step(5)
+        assert f.sync() == 0
+    for which in (0, 1):
+        assert _rel(F.get(which), B.get(which)) < 2e-5
+    if not walls:
+        assert abs(F.mass(0) - m0) < 1e-13
