@@ -176,14 +176,15 @@ bool use_line_pseudo(const fr_mesh& m, const fr_params& p) {
 bool set_line_pseudo(const fr_mesh& m, bool gen, KernelSet* ks) {
   return m.etype == FR_QUAD ? line_pseudo_quad(m.order, gen, ks) : line_pseudo_hex(m.order, gen, ks);
 }
-bool set_line_kernels(const fr_mesh& m, bool gen, KernelSet* ks) {
-  return m.etype == FR_QUAD ? line_kernels_quad(m.order, gen, ks) : line_kernels_hex(m.order, gen, ks);
+bool set_line_kernels(const fr_mesh& m, bool gen, bool tab, KernelSet* ks) {
+  return m.etype == FR_QUAD ? line_kernels_quad(m.order, gen, tab, ks) : line_kernels_hex(m.order, gen, tab, ks);
 }
 
 // Blocks of the largest launch (one reduction partial each): the block-wide
 // kernels', the element-wise kernels' or the line kernels'.
 int most_blocks(const fr_mesh& m, const KernelSet& ks, int elementwise) {
   int64_t n = std::max(ks.max_blocks, elementwise);
+  if (m.etype == FR_TRI) n = std::max<int64_t>(n, (m.E + 31) / 32);  // a warp a block (ka_trir)
   if (m.etype != FR_TRI && m.nfp <= 32) {
     const int per = kPseudoWarps * (32 / m.nfp);
     n = std::max<int64_t>(n, (m.E + per - 1) / per);
@@ -313,13 +314,41 @@ int check_params(const fr_params* p) {
   } while (0)
 
 // ---- small kernels ---------------------------------------------------------
+// float -> double by moving the bits: exact, and on the integer units, where
+// the conversion instruction takes the FP64 pipe (2 lanes a clock).
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu, e = m >> 23;
+  if (e - 1u < 254u) return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+  return m == 0 ? __hiloint2double((int)u, 0) : (double)x;  // zero; subnormal, infinite, NaN
+}
 // The solution u is double in the FP64 path and a float-float pair
 // (hi, lo) in the mixed path; these helpers read and write one value.
 __device__ __forceinline__ double u_get(const KArgs& A, int mixed, int64_t g) {
   if (!mixed) return A.u[g];
   const float2 v = reinterpret_cast<const float2*>(A.u)[g];
-  return (double)v.x + (double)v.y;
+  return widen(v.x) + widen(v.y);
 }
+
+// The values of a grid-stride loop over E x NU points, value by value as
+// (index, element, point): the element advances by a fixed quotient and
+// remainder a step instead of a 64-bit division a point.
+struct PointLoop {
+  int64_t g, n, stride, e, qe;
+  int i, NU, qi;
+  __device__ __forceinline__ PointLoop(int64_t E, int NU_)
+      : g(blockIdx.x * (int64_t)blockDim.x + threadIdx.x), n(E * NU_), stride((int64_t)gridDim.x * blockDim.x),
+        e(g / NU_), qe(stride / NU_), i((int)(g - e * NU_)), NU(NU_), qi((int)(stride - qe * NU_)) {}
+  __device__ __forceinline__ bool more() const { return g < n; }
+  __device__ __forceinline__ void next() {
+    g += stride;
+    e += qe;
+    i += qi;
+    if (i >= NU) {
+      i -= NU;
+      ++e;
+    }
+  }
+};
 __device__ __forceinline__ void u_put(const KArgs& A, int mixed, int64_t g, double x) {
   if (!mixed) {
     A.u[g] = x;
@@ -330,40 +359,37 @@ __device__ __forceinline__ void u_put(const KArgs& A, int mixed, int64_t g, doub
 }
 
 template <typename T>
-__global__ void k_reset_psi(KArgs A, int64_t NU, int mixed) {
-  const int64_t n = A.E * NU;
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = g / NU, i = g % NU;
-    const double p0 = u_get(A, mixed, (e * 2 + 0) * NU + i) - 0.5;
-    A.psi0[g] = p0;
-    u_put(A, mixed, (e * 2 + 1) * NU + i, p0);
-    reinterpret_cast<T*>(A.ustg)[(e * 2 + 1) * NU + i] = (T)p0;
+__global__ void k_reset_psi(KArgs A, int NU, int mixed) {
+  for (PointLoop p(A.E, NU); p.more(); p.next()) {
+    const double p0 = u_get(A, mixed, (p.e * 2 + 0) * NU + p.i) - 0.5;
+    A.psi0[p.g] = p0;
+    u_put(A, mixed, (p.e * 2 + 1) * NU + p.i, p0);
+    reinterpret_cast<T*>(A.ustg)[(p.e * 2 + 1) * NU + p.i] = (T)p0;
   }
 }
 
 template <typename T>
-__global__ void k_to_stage(KArgs A, int64_t NU, int mixed) {
+__global__ void k_to_stage(KArgs A, int NU, int mixed) {
   const int64_t n = A.E * 2 * NU;
   for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x)
     reinterpret_cast<T*>(A.ustg)[g] = (T)u_get(A, mixed, g);
 }
 
 // field `fld` of u <-> contiguous double buffer
-__global__ void k_unpack(KArgs A, int64_t NU, int fld, int mixed, double* out) {
-  const int64_t n = A.E * NU;
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x)
-    out[g] = u_get(A, mixed, (g / NU * 2 + fld) * NU + g % NU);
+__global__ void k_unpack(KArgs A, int NU, int fld, int mixed, double* out) {
+  for (PointLoop p(A.E, NU); p.more(); p.next()) out[p.g] = u_get(A, mixed, (p.e * 2 + fld) * NU + p.i);
 }
-__global__ void k_pack(KArgs A, int64_t NU, int fld, int mixed, const double* in) {
-  const int64_t n = A.E * NU;
-  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x)
-    u_put(A, mixed, (g / NU * 2 + fld) * NU + g % NU, in[g]);
+__global__ void k_pack(KArgs A, int NU, int fld, int mixed, const double* in) {
+  for (PointLoop p(A.E, NU); p.more(); p.next()) u_put(A, mixed, (p.e * 2 + fld) * NU + p.i, in[p.g]);
 }
 
 // Neumaier two-term accumulation
 __device__ __forceinline__ void neu_add(double& s, double& c, double x) {
   const double t = s + x;
-  c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
+  // the larger magnitude first; compared as integers, off the FP64 pipe
+  const bool big = (__double_as_longlong(s) & 0x7fffffffffffffffll) >= (__double_as_longlong(x) & 0x7fffffffffffffffll);
+  const double a = big ? s : x, b = big ? x : s;
+  c += (a - t) + b;
   s = t;
 }
 
@@ -395,30 +421,16 @@ __device__ __forceinline__ void neu_block(double& s, double& c, double* ss, doub
 }
 
 // Compensated, fixed-order integral of field `fld` with weights wdet.  Bound by
-// the FP64 pipe (nine instructions a point at 2 lanes a clock): the block and
+// the FP64 pipe (six instructions a point at 2 lanes a clock): the block and
 // grid sums run as trees, since one thread adding the 256 values of its block
 // and then every block's in turn was a serial FP64 chain of 1.2 ms on 7.1 M
 // points, whatever their number.
 __global__ void __launch_bounds__(kThreads) k_mass(KArgs A, int NU, int fld, int mixed) {
   __shared__ double ss[kThreads / 32], sc[kThreads / 32];
   __shared__ bool last;
-  const int64_t n = A.E * NU, stride = (int64_t)gridDim.x * kThreads;
   double s = 0.0, c = 0.0;
-  // the point's element advances by a fixed quotient and remainder per step
-  int64_t g = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-  int64_t e = g / NU;
-  int i = (int)(g - e * NU);
-  const int64_t qe = stride / NU;
-  const int qi = (int)(stride - qe * NU);
-  for (; g < n; g += stride) {
-    neu_add(s, c, A.wdet[g] * u_get(A, mixed, (e * 2 + fld) * NU + i));
-    e += qe;
-    i += qi;
-    if (i >= NU) {
-      i -= NU;
-      ++e;
-    }
-  }
+  for (PointLoop p(A.E, NU); p.more(); p.next())
+    neu_add(s, c, A.wdet[p.g] * u_get(A, mixed, (p.e * 2 + fld) * NU + p.i));
   neu_block(s, c, ss, sc);
   if (threadIdx.x == 0) {
     A.red[2 * blockIdx.x] = s;
@@ -758,14 +770,15 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
   A.mcg = L.mcg ? b + L.mcg : nullptr;
   A.vtab = nullptr;
   fill_line_ops(m, A.lo);
+  const bool diagonal = m->etype != FR_TRI && all_diagonal(*m);
   if (use_line_kernels(*m, *prm)) {
     if (vel_separable(prm->vel.kind)) A.vtab = reinterpret_cast<const float2*>(b + L.vtab);
-    if (!set_line_kernels(*m, !(A.vtab && all_diagonal(*m)), &f->ks)) {
+    if (!set_line_kernels(*m, !diagonal, A.vtab != nullptr, &f->ks)) {
       delete f;
       return FR_ECUDA;
     }
   }
-  if (use_line_pseudo(*m, *prm) && !set_line_pseudo(*m, !all_diagonal(*m), &f->ks)) {
+  if (use_line_pseudo(*m, *prm) && !set_line_pseudo(*m, !diagonal, &f->ks)) {
     delete f;
     return FR_ECUDA;
   }
@@ -986,7 +999,7 @@ extern "C" int fr_field_init_batch(const fr_mesh* m, const fr_params* prm, int n
   if (use_line_kernels(*m, *prm)) {
     // the table holds params->vel, the instances' own velocities are in the point cache
     f->args.vtab = nullptr;
-    if (!set_line_kernels(*m, true, &f->ks)) {
+    if (!set_line_kernels(*m, !all_diagonal(*m), false, &f->ks)) {
       fr_field_destroy(f);
       return FR_ECUDA;
     }

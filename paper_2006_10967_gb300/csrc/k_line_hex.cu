@@ -3,12 +3,12 @@
 #include "k_line_inst.cuh"
 
 namespace frp {
-bool line_kernels_hex(int order, bool gen, KernelSet* ks) {
+bool line_kernels_hex(int order, bool gen, bool tab, KernelSet* ks) {
   switch (order) {
-    case 1: return gen ? fill_line<3, 2, true>(ks) : fill_line<3, 2, false>(ks);
-    case 2: return gen ? fill_line<3, 3, true>(ks) : fill_line<3, 3, false>(ks);
-    case 3: return gen ? fill_line<3, 4, true>(ks) : fill_line<3, 4, false>(ks);
-    case 4: return gen ? fill_line<3, 5, true>(ks) : fill_line<3, 5, false>(ks);
+    case 1: return fill_line<3, 2>(gen, tab, ks);
+    case 2: return fill_line<3, 3>(gen, tab, ks);
+    case 3: return fill_line<3, 4>(gen, tab, ks);
+    case 4: return fill_line<3, 5>(gen, tab, ks);
     default: return false;
   }
 }

@@ -12,11 +12,13 @@ unsigned line_grid(int64_t E, int warps) {
   return (unsigned)((E + per - 1) / per);
 }
 
-template <int DIM, int N, bool GEN>
+template <int DIM, int N, bool GEN, bool TAB>
 void launch_kb_line(const KArgs& A, cudaStream_t s) {
-  constexpr int smem = KBLine<DIM, N, GEN>::F * 4 * kLineWarps;
-  if (A.cf.prm.nphi) kb_line<DIM, N, GEN, true, kLineWarps><<<line_grid<DIM, N>(A.E, kLineWarps), kLineWarps * 32, smem, s>>>(A);
-  else kb_line<DIM, N, GEN, false, kLineWarps><<<line_grid<DIM, N>(A.E, kLineWarps), kLineWarps * 32, smem, s>>>(A);
+  constexpr int smem = KBLine<DIM, N, GEN, TAB>::F * 4 * kLineWarps;
+  static_assert(smem <= 48 * 1024, "no shared-memory opt-in needed");
+  const unsigned grid = line_grid<DIM, N>(A.E, kLineWarps);
+  if (A.cf.prm.nphi) kb_line<DIM, N, GEN, TAB, true, kLineWarps><<<grid, kLineWarps * 32, smem, s>>>(A);
+  else kb_line<DIM, N, GEN, TAB, false, kLineWarps><<<grid, kLineWarps * 32, smem, s>>>(A);
 }
 
 template <int DIM, int N, bool GEN, int SF>
@@ -48,13 +50,18 @@ bool prepare_ka_line() {
 }
 
 template <int DIM, int N, bool GEN>
-bool fill_line(KernelSet* ks) {
-  ks->kb[0] = launch_kb_line<DIM, N, GEN>;
+bool fill_line_set(bool tab, KernelSet* ks) {
+  if constexpr (GEN) ks->kb[0] = launch_kb_line<DIM, N, true, false>;
+  else ks->kb[0] = tab ? launch_kb_line<DIM, N, false, true> : launch_kb_line<DIM, N, false, false>;
   ks->ka[0] = launch_ka_line<DIM, N, GEN>;
   ks->vtab = launch_vel_tab<DIM, N>;
-  static_assert(KBLine<DIM, N, GEN>::F * 4 * kLineWarps <= 48 * 1024, "no shared-memory opt-in needed");
   return prepare_ka_line<DIM, N, GEN, 0>() && prepare_ka_line<DIM, N, GEN, 1>() && prepare_ka_line<DIM, N, GEN, 2>() &&
          prepare_ka_line<DIM, N, GEN, 3>() && prepare_ka_line<DIM, N, GEN, 4>();
+}
+
+template <int DIM, int N>
+bool fill_line(bool gen, bool tab, KernelSet* ks) {
+  return gen ? fill_line_set<DIM, N, true>(tab, ks) : fill_line_set<DIM, N, false>(tab, ks);
 }
 
 template <int DIM, int N, bool GEN>

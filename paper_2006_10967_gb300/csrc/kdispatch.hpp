@@ -27,9 +27,9 @@ bool kernels_tri(int order, int precision, int64_t E, int variant, KernelSet* ks
 
 // Replace the physical-step kernels of a mixed tensor field by the line kernels
 // (kline.cuh); false where they are not built (the set is then unchanged) or
-// could not be prepared.  gen: see kb_line.
-bool line_kernels_quad(int order, bool gen, KernelSet* ks);
-bool line_kernels_hex(int order, bool gen, KernelSet* ks);
+// could not be prepared.  gen, tab: see KBLine.
+bool line_kernels_quad(int order, bool gen, bool tab, KernelSet* ks);
+bool line_kernels_hex(int order, bool gen, bool tab, KernelSet* ks);
 // The same for the preconditioning kernels of a mixed tensor field; gen false:
 // every element is affine with a diagonal Jacobian.
 bool line_pseudo_quad(int order, bool gen, KernelSet* ks);

@@ -66,20 +66,25 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, make
 
 // ---- layout -----------------------------------------------------------------
 // Elements per warp, padded row (RS), plane (PS) and array (AS) strides of the
-// warp-private arrays, in floats.  The strides spread the words that the 32
-// lanes of an axis-1 or axis-2 line pass touch over the 32 banks: for
-// hexahedra of N = 4, lane (x, z) of element es reads x + 20 z + 80 es (+ 4 m)
-// and lane (x, y) reads x + 4 y + 80 es (+ 20 m), both 32 different banks.
+// warp-private arrays, in floats.  A row (axis-0 line) moves in 8-byte words,
+// or one 16-byte word for N = 4; a line of another axis in 4-byte words.  The
+// strides come from counting the shared-memory wavefronts of one row and one
+// line access over the 32 banks: (row, axis-1 line, axis-2 line) in wavefronts
+// for quads N = 3..7 (4,6) (4,4) (6,10) (6,12) (8,14), where dense rows of
+// 2 NP floats with arrays padded for the lines alone gave (8,6) (8,4) (21,10)
+// (18,6) (36,7); for hexes N = 3, 4, 5 (4,6,6) (8,4,4) (6,15,5).
 template <int DIM, int N>
 struct LL {
   using S = TS<DIM, N>;
   static constexpr int NU = S::NU, NF = S::NF, NFP = S::NFP, LN = S::NFP;
   static constexpr int EPW = 32 / LN;
   static constexpr int NP = (N + 1) / 2;
-  static constexpr int RS = 2 * NP;
-  static constexpr int PS = DIM == 3 ? (N == 2 ? 4 : N == 3 ? 12 : N == 4 ? 20 : 38) : N * RS;
-  static constexpr int AS = DIM == 3 ? (N == 2 ? 8 : N == 3 ? 44 : N == 4 ? 80 : 190)
-                                     : (N == 2 ? 4 : N == 3 ? 12 : N == 4 ? 20 : N == 5 ? 38 : N == 6 ? 38 : 72);
+  static constexpr int RS = DIM == 3 ? (N == 3 ? 6 : 2 * NP) : (N == 3 ? 6 : N == 4 ? 8 : N == 5 || N == 7 ? 10 : 2 * NP);
+  static constexpr int PS = DIM == 3 ? (N == 2 ? 4 : N == 3 ? 18 : N == 4 ? 20 : 30) : N * RS;
+  static constexpr int AS = DIM == 3 ? (N == 2 ? 8 : N == 3 ? 54 : N == 4 ? 80 : 150) : (N == 4 ? 36 : N * RS);
+  static constexpr bool V4 = N == 4;  // a row is one 16-byte word
+  static_assert(RS % 2 == 0 && PS % 2 == 0 && AS % 2 == 0, "rows on 8-byte boundaries");
+  static_assert(!V4 || (RS % 4 == 0 && PS % 4 == 0 && AS % 4 == 0), "rows on 16-byte boundaries");
   static constexpr bool FULL = 32 % LN == 0;  // every lane owns a line
   // rows read and written as vectors straight from global memory (a whole
   // number of 8- or 16-byte words, neighbouring lanes contiguous); other N
@@ -103,19 +108,19 @@ __host__ __device__ constexpr int pstride(int a) {
   return a == 0 ? 1 : (a == 1 ? LL<DIM, N>::RS : LL<DIM, N>::PS);
 }
 
-// one padded row (2 NP floats, 8-byte aligned; 16 for N = 4)
-template <int NP>
+// one padded row (2 NP floats, 8-byte aligned; 16 for V4)
+template <int NP, bool V4>
 __device__ __forceinline__ void row_put(float* p, const float2* v) {
-  if constexpr (NP == 2) {
+  if constexpr (V4) {
     *reinterpret_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
   } else {
 #pragma unroll
     for (int i = 0; i < NP; ++i) reinterpret_cast<float2*>(p)[i] = v[i];
   }
 }
-template <int NP>
+template <int NP, bool V4>
 __device__ __forceinline__ void row_get(const float* p, float2* v) {
-  if constexpr (NP == 2) {
+  if constexpr (V4) {
     const float4 q = *reinterpret_cast<const float4*>(p);
     v[0] = make_float2(q.x, q.y);
     v[1] = make_float2(q.z, q.w);
@@ -344,20 +349,22 @@ __global__ void k_vel_tab(const KArgs A) {
 
 // ---- residual kernel ----------------------------------------------------------
 // GEN false: every element of the mesh is axis-aligned and affine (record flag
-// 2) and the velocity separable (A.vtab), so only that path is compiled; true:
-// each element takes that path or the general one (metric from the map's
-// coefficients, velocity from the point cache), by its own flag, so that an
-// element's result does not depend on what else is in the mesh.
-template <int DIM, int N, bool GEN>
+// 2), so only that path is compiled; true: each element takes that path or the
+// general one (metric from the map's coefficients) by its own flag, so that an
+// element's result does not depend on what else is in the mesh.  Axis-aligned
+// elements take the velocity from the factor table where the field has one
+// (TAB; with GEN known at run time), the others from the point cache.
+template <int DIM, int N, bool GEN, bool TAB>
 struct KBLine {
   using L = LL<DIM, N>;
   static constexpr int WARP_F = (2 * (1 + DIM) * L::AS) * L::EPW;  // floats a warp
   static constexpr int IN_F = L::DIRECT ? 0 : ((L::EPW * 2 * L::NU + 3) / 4) * 4;
   // read in the middle of the tile, copied in at its start: the velocity table
   // and, on the general path, the point velocities and the map coefficients
-  static constexpr int TAB_F = (L::EPW * DIM * (N + 2) * 2 + 3) / 4 * 4;
-  static constexpr int VF_F = GEN ? (L::EPW * DIM * L::NF + 3) / 4 * 4 : 0;
-  static constexpr int VU_F = GEN ? (L::EPW * DIM * L::NU + 3) / 4 * 4 : 0;
+  static constexpr bool PTS = GEN || !TAB;  // point velocities may be read
+  static constexpr int TAB_F = GEN || TAB ? (L::EPW * DIM * (N + 2) * 2 + 3) / 4 * 4 : 0;
+  static constexpr int VF_F = PTS ? (L::EPW * DIM * L::NF + 3) / 4 * 4 : 0;
+  static constexpr int VU_F = PTS ? (L::EPW * DIM * L::NU + 3) / 4 * 4 : 0;
   static constexpr int GEO_F = GEN ? L::EPW * L::S::NG : 0;
   static constexpr int O_IN = (WARP_F + 3) / 4 * 4, O_TAB = O_IN + IN_F, O_VF = O_TAB + TAB_F, O_VU = O_VF + VF_F,
                        O_GEO = O_VU + VU_F;
@@ -367,10 +374,10 @@ struct KBLine {
 };
 
 // NPHI: the interface normal comes from phi (the unpreconditioned method).
-template <int DIM, int N, bool GEN, bool NPHI, int WPB>
-__global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
+template <int DIM, int N, bool GEN, bool TAB, bool NPHI, int WPB>
+__global__ void __launch_bounds__(WPB * 32, (GEN ? 16 : 20) / WPB) kb_line(const KArgs A) {
   using L = LL<DIM, N>;
-  using K = KBLine<DIM, N, GEN>;
+  using K = KBLine<DIM, N, GEN, TAB>;
   constexpr int NU = L::NU, NF = L::NF, NFP = L::NFP, LN = L::LN, EPW = L::EPW, NP = L::NP, AS = L::AS;
   constexpr int NT = N + 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -441,16 +448,17 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
   }
   {
     const int ne = (int)max((int64_t)0, min((int64_t)EPW, A.E - e0));
-    if (!GEN || A.vtab) tile_fetch<EPW, DIM * NT * 8>(wsm + K::O_TAB, A.vtab + e0 * DIM * NT, ne, lane);
-    if constexpr (GEN) {
+    if (GEN ? A.vtab != nullptr : TAB) tile_fetch<EPW, DIM * NT * 8>(wsm + K::O_TAB, A.vtab + e0 * DIM * NT, ne, lane);
+    if constexpr (K::PTS) {
       tile_fetch<EPW, DIM * NF * 4>(wsm + K::O_VF, reinterpret_cast<const float*>(A.vsf) + e0 * DIM * NF, ne, lane);
       tile_fetch<EPW, DIM * NU * 4>(wsm + K::O_VU, reinterpret_cast<const float*>(A.vsu) + e0 * DIM * NU, ne, lane);
-      tile_fetch<EPW, L::S::NG * 4>(wsm + K::O_GEO, A.geof + e0 * L::S::NG, ne, lane);
     }
+    if constexpr (GEN) tile_fetch<EPW, L::S::NG * 4>(wsm + K::O_GEO, A.geof + e0 * L::S::NG, ne, lane);
     cp_async_commit();
   }
   const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
-  const bool diag = !GEN || (A.vtab != nullptr && __ldg(mc + 11) == 2.f);
+  const bool diag = !GEN || __ldg(mc + 11) == 2.f;
+  const bool tab = GEN ? diag && A.vtab != nullptr : TAB;
   float sd[DIM];  // S_aa of the diagonal metric
 #pragma unroll
   for (int a = 0; a < DIM; ++a) sd[a] = __ldg(mc + a * 4);
@@ -493,7 +501,7 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
   }
   if (lane_ok) {
 #pragma unroll
-    for (int f = 0; f < 2; ++f) row_put<NP>(U + f * FA + pline<DIM, N>(0, l), u[f]);
+    for (int f = 0; f < 2; ++f) row_put<NP, L::V4>(U + f * FA + pline<DIM, N>(0, l), u[f]);
   }
   __syncwarp();
 #pragma unroll
@@ -532,13 +540,13 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
   }
   // the other fields' faces need the axis-0 component of the field that gives the normal
   constexpr int kn = NPHI ? 0 : 1;
-  if (lane_ok && diag) row_put<NP>(Q + (kn * DIM) * FA + pline<DIM, N>(0, l), q[kn][0]);
+  if (lane_ok && diag) row_put<NP, L::V4>(Q + (kn * DIM) * FA + pline<DIM, N>(0, l), q[kn][0]);
   cp_async_wait_all();
   __syncwarp();
 #pragma unroll
   for (int f = 0; f < 2; ++f)
 #pragma unroll
-    for (int a = 1; a < DIM; ++a) row_get<NP>(Q + (f * DIM + a) * FA + pline<DIM, N>(0, l), q[f][a]);
+    for (int a = 1; a < DIM; ++a) row_get<NP, L::V4>(Q + (f * DIM + a) * FA + pline<DIM, N>(0, l), q[f][a]);
 
   int lc[3];  // the lane's point coordinates on axes 1, 2
   lc[1] = DIM == 3 ? l % N : l;
@@ -571,7 +579,7 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
 #pragma unroll
       for (int f = 0; f < 2; ++f)
 #pragma unroll
-        for (int b = 0; b < DIM; ++b) row_put<NP>(Q + (f * DIM + b) * FA + pline<DIM, N>(0, l), q[f][b]);
+        for (int b = 0; b < DIM; ++b) row_put<NP, L::V4>(Q + (f * DIM + b) * FA + pline<DIM, N>(0, l), q[f][b]);
     }
   }
   if (GEN) __syncwarp();
@@ -601,30 +609,42 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
         const float2 t = line_ends<N>(O, v);
         g2 = fma2(t, t, g2);
       }
-      // velocity factors: v_c = s_c g prod_b (b == c ? A : B)_b
-      float kc[DIM];
-      const int j1 = l % N, j2 = l / N;  // the line's coordinates on the two other axes, lowest first
+      float2 va, v2;
+      if (tab) {
+        // velocity factors: v_c = s_c g prod_b (b == c ? A : B)_b
+        float kc[DIM];
+        const int j1 = l % N, j2 = l / N;  // the line's coordinates on the two other axes, lowest first
 #pragma unroll
-      for (int c = 0; c < DIM; ++c) kc[c] = P.vs[c] * gv;
-      {
-        int i = 0;
+        for (int c = 0; c < DIM; ++c) kc[c] = P.vs[c] * gv;
+        {
+          int i = 0;
 #pragma unroll
-        for (int b = 0; b < DIM; ++b) {
-          if (b == a) continue;
-          const float2 ab = vt[b * NT + (i == 0 ? (DIM == 2 ? l : j1) : j2)];
-          ++i;
+          for (int b = 0; b < DIM; ++b) {
+            if (b == a) continue;
+            const float2 ab = vt[b * NT + (i == 0 ? (DIM == 2 ? l : j1) : j2)];
+            ++i;
 #pragma unroll
-          for (int c = 0; c < DIM; ++c) kc[c] = __fmul_rn(kc[c], c == b ? ab.x : ab.y);
+            for (int c = 0; c < DIM; ++c) kc[c] = __fmul_rn(kc[c], c == b ? ab.x : ab.y);
+          }
+        }
+        const float2 e0v = vt[a * NT + N], e1v = vt[a * NT + N + 1];
+        const float2 Ae = make_float2(e0v.x, e1v.x), Be = make_float2(e0v.y, e1v.y);
+        float ko = 0.f;  // sum of the other components' squares
+#pragma unroll
+        for (int c = 0; c < DIM; ++c)
+          if (c != a) ko = __fmaf_rn(kc[c], kc[c], ko);
+        va = mul2(Ae, dup2(kc[a]));
+        v2 = fma2(va, va, mul2(mul2(Be, Be), dup2(ko)));
+      } else {
+        const float* vf = wsm + K::O_VF + es * DIM * NF + 2 * a * NFP + l;
+        v2 = dup2(0.f);
+#pragma unroll
+        for (int c = 0; c < DIM; ++c) {
+          const float2 v = mul2(dup2(gfac), make_float2(vf[c * NF], vf[c * NF + NFP]));
+          if (c == a) va = v;
+          v2 = fma2(v, v, v2);
         }
       }
-      const float2 e0v = vt[a * NT + N], e1v = vt[a * NT + N + 1];
-      const float2 Ae = make_float2(e0v.x, e1v.x), Be = make_float2(e0v.y, e1v.y);
-      float ko = 0.f;  // sum of the other components' squares
-#pragma unroll
-      for (int c = 0; c < DIM; ++c)
-        if (c != a) ko = __fmaf_rn(kc[c], kc[c], ko);
-      const float2 va = mul2(Ae, dup2(kc[a]));
-      const float2 v2 = fma2(va, va, mul2(mul2(Be, Be), dup2(ko)));
       const float2 M = flux_mult(v2, P.gamma);
       const float2 sh = sharp2(pL, g2, P.gamma, P.rdelta);
       const float2 nvis = fma2(sh, qn, mul2(dup2(-eps), qe[a][0]));  // minus the viscous flux over M
@@ -717,7 +737,7 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
   {
     float2 k[DIM];  // diagonal metric: velocity factors of the line
     float ko = 0.f;
-    if (diag) {
+    if (tab) {
       float kc[DIM];
 #pragma unroll
       for (int c = 0; c < DIM; ++c) kc[c] = P.vs[c] * gv;
@@ -735,14 +755,14 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       float2 v[DIM], v2, Sm[3][3];
-      if (diag) {
+      if (tab) {
         const float2 t0 = vt[2 * p], t1 = 2 * p + 1 < N ? vt[2 * p + 1] : make_float2(0.f, 0.f);
         const float2 Ax = make_float2(t0.x, t1.x), Bx = make_float2(t0.y, t1.y);
         v[0] = mul2(Ax, k[0]);
 #pragma unroll
         for (int c = 1; c < DIM; ++c) v[c] = mul2(Bx, k[c]);
         v2 = fma2(v[0], v[0], mul2(mul2(Bx, Bx), dup2(ko)));
-      } else if (GEN) {
+      } else {
         const float* vc = wsm + K::O_VU + es * DIM * NU + l * N + 2 * p;
         v2 = dup2(0.f);
 #pragma unroll
@@ -750,6 +770,8 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
           v[c] = mul2(dup2(gfac), make_float2(vc[c * NU], 2 * p + 1 < N ? vc[c * NU + 1] : 0.f));
           v2 = fma2(v[c], v[c], v2);
         }
+      }
+      if (GEN && !diag) {
         float2 xi[3];
         xi[0] = O.xp[p];
 #pragma unroll
@@ -801,7 +823,7 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
 #pragma unroll
     for (int f = 0; f < 2; ++f)
 #pragma unroll
-      for (int a = 1; a < DIM; ++a) row_put<NP>(Q + (f * DIM + a) * FA + pline<DIM, N>(0, l), q[f][a]);
+      for (int a = 1; a < DIM; ++a) row_put<NP, L::V4>(Q + (f * DIM + a) * FA + pline<DIM, N>(0, l), q[f][a]);
   }
   __syncwarp();
 
@@ -836,7 +858,7 @@ __global__ void __launch_bounds__(WPB * 32, 16 / WPB) kb_line(const KArgs A) {
 #pragma unroll
     for (int a = 1; a < DIM; ++a) {
       float2 t[NP];
-      row_get<NP>(Q + (f * DIM + a) * FA + pline<DIM, N>(0, l), t);
+      row_get<NP, L::V4>(Q + (f * DIM + a) * FA + pline<DIM, N>(0, l), t);
 #pragma unroll
       for (int p = 0; p < NP; ++p) dv[f][p] = add2(dv[f][p], t[p]);
     }
@@ -1160,8 +1182,8 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
         const int other = DIM == 3 ? (a == 1 ? lc2 : lc1) : 0;
         const float* s = C0 + (((((a - 1) * 2) * 2 + f) * EPW + es) * L::OTH + other) * L::RS;
         float2 r0[NP], r1[NP];
-        row_get<NP>(s, r0);
-        row_get<NP>(s + 2 * EPW * L::OTH * L::RS, r1);
+        row_get<NP, L::V4>(s, r0);
+        row_get<NP, L::V4>(s + 2 * EPW * L::OTH * L::RS, r1);
 #pragma unroll
         for (int p = 0; p < NP; ++p) y[f][p] = fma2(dup2(gl[a]), r0[p], fma2(dup2(gr[a]), r1[p], y[f][p]));
       }
@@ -1294,7 +1316,7 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
   // ---- flux-point traces of the new stage value (Step 1 of the next stage) ------
   if (lane_ok) {
 #pragma unroll
-    for (int f = 0; f < 2; ++f) row_put<NP>(R0 + (f * EPW + es) * AS + pline<DIM, N>(0, l), y[f]);
+    for (int f = 0; f < 2; ++f) row_put<NP, L::V4>(R0 + (f * EPW + es) * AS + pline<DIM, N>(0, l), y[f]);
   }
   __syncwarp();
   float* tr = reinterpret_cast<float*>(A.tr);

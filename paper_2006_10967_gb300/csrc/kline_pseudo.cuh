@@ -199,8 +199,8 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
       for (int m = 1; m < N; ++m) c[p] = fma2(O.V[m][p], dup2(v[m]), c[p]);
     }
     if (lane_ok) {
-      row_put<NP>(U + pline<DIM, N>(0, l), u);
-      row_put<NP>(C + pline<DIM, N>(0, l), c);
+      row_put<NP, L::V4>(U + pline<DIM, N>(0, l), u);
+      row_put<NP, L::V4>(C + pline<DIM, N>(0, l), c);
     }
   }
   __syncwarp();
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
   }
   __syncwarp();
 #pragma unroll
-  for (int a = 1; a < DIM; ++a) row_get<NP>(Q + a * FA + pline<DIM, N>(0, l), q[a]);
+  for (int a = 1; a < DIM; ++a) row_get<NP, L::V4>(Q + a * FA + pline<DIM, N>(0, l), q[a]);
 
   const int lc1 = DIM == 3 ? l % N : l, lc2 = DIM == 3 ? l / N : 0;
   const float* geo = wsm + K::O_GEO + es * L::S::NG;
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
     }
     if (lane_ok) {
 #pragma unroll
-      for (int b = 0; b < DIM; ++b) row_put<NP>(Q + b * FA + pline<DIM, N>(0, l), q[b]);
+      for (int b = 0; b < DIM; ++b) row_put<NP, L::V4>(Q + b * FA + pline<DIM, N>(0, l), q[b]);
     }
   }
   if (GEN) __syncwarp();
@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
   }
   if (lane_ok) {
 #pragma unroll
-    for (int a = 1; a < DIM; ++a) row_put<NP>(Q + a * FA + pline<DIM, N>(0, l), q[a]);
+    for (int a = 1; a < DIM; ++a) row_put<NP, L::V4>(Q + a * FA + pline<DIM, N>(0, l), q[a]);
   }
   __syncwarp();
 
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
 #pragma unroll
   for (int a = 1; a < DIM; ++a) {
     float2 t[NP];
-    row_get<NP>(Q + a * FA + pline<DIM, N>(0, l), t);
+    row_get<NP, L::V4>(Q + a * FA + pline<DIM, N>(0, l), t);
 #pragma unroll
     for (int p = 0; p < NP; ++p) dv[p] = add2(dv[p], t[p]);
   }
@@ -596,8 +596,8 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
       const float gl = A.cf.ops.gLd[me], gr = -A.cf.ops.gRd[me];
       const float* s = C0 + (((a - 1) * 2 * EPW + es) * L::OTH + other) * L::RS;
       float2 r0[NP], r1[NP];
-      row_get<NP>(s, r0);
-      row_get<NP>(s + EPW * L::OTH * L::RS, r1);
+      row_get<NP, L::V4>(s, r0);
+      row_get<NP, L::V4>(s + EPW * L::OTH * L::RS, r1);
 #pragma unroll
       for (int p = 0; p < NP; ++p) y[p] = fma2(dup2(gl), r0[p], fma2(dup2(gr), r1[p], y[p]));
     }
@@ -692,7 +692,7 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
   }
 
   // ---- traces of the new stage value
-  if (lane_ok) row_put<NP>(R0 + es * L::AS + pline<DIM, N>(0, l), y);
+  if (lane_ok) row_put<NP, L::V4>(R0 + es * L::AS + pline<DIM, N>(0, l), y);
   __syncwarp();
   float* tr = reinterpret_cast<float*>(A.tr);
 #pragma unroll

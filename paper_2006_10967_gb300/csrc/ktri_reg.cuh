@@ -49,13 +49,14 @@ struct TriReg {
   static constexpr int N = P + 1, NU = S::NU, NF = S::NF, NPE = TriPack(P).npe, NPU = TriPack(P).npu;
   static constexpr int O_L = TriPack(P).o_l, O_D = TriPack(P).o_d, O_LIFT = TriPack(P).o_lift, O_V = TriPack(P).o_v,
                        SIZE = TriPack(P).size;
-  static constexpr int TB = 64;  // threads a block
+  static constexpr int TB = 32;  // threads a block
   // floats an element of the residual kernel's buffers: state (then the
   // divergence), velocities at the points, at the flux points (then the fluxes)
   static constexpr int KB_F = 2 * NU + 2 * NU + 2 * NF;
   static constexpr size_t KB_SMEM = ((size_t)SIZE + TB * KB_F) * 4;
-  // update kernel: rp (then the stage value), solution pairs, accumulator, traces
-  static constexpr int KA_F = 2 * NU + 4 * NU + 2 * NU + 2 * NF;
+  // update kernel: rp (then the stage value), solution pairs, accumulator, face
+  // weights (then traces), w det J pairs
+  static constexpr int KA_F = 2 * NU + 4 * NU + 2 * NU + 2 * NF + 2 * NU;
   static_assert(SIZE % 4 == 0 && O_D % 4 == 0 && O_LIFT % 4 == 0 && O_V % 4 == 0, "16-byte boundaries");
   static constexpr size_t KA_SMEM = ((size_t)SIZE + TB * KA_F) * 4;
 };
@@ -401,7 +402,8 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
   float* yb = ops + R::SIZE + warp * 32 * R::KA_F;
   float* sb = yb + 32 * 2 * NU;   // solution pairs
   float* ab = sb + 32 * 4 * NU;   // accumulator
-  float* tb = ab + 32 * 2 * NU;   // traces
+  float* tb = ab + 32 * 2 * NU;   // face weights, later the traces
+  float* wb = tb + 32 * 2 * NF;   // w det J pairs (stage 4)
   const int64_t e0 = ((int64_t)blockIdx.x * R::TB) + warp * 32;
   const int ne = (int)max((int64_t)0, min((int64_t)32, A.E - e0));
   const bool act = lane < ne;
@@ -417,6 +419,10 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
   if (SF >= 1) tile_fetch<32, 2 * NU * 8>(sb, reinterpret_cast<const float2*>(A.u) + e0 * 2 * NU, ne, lane);
   // acc: at stage 1 only the other field's half of a preconditioning row is kept
   if (SF >= 2 || (SF == 1 && MODE == 1)) tile_fetch<32, 2 * NU * 4>(ab, reinterpret_cast<const float*>(A.acc) + e0 * 2 * NU, ne, lane);
+  if (cons) {
+    tile_fetch<32, NF * 8>(tb, A.wphys + e0 * NF, ne, lane);
+    if (SF == 4) tile_fetch<32, NU * 8>(wb, A.wdetf + e0 * NU, ne, lane);
+  }
   float phi_keep[MODE == 1 ? NU : 1];  // preconditioning: phi's stage value
   if (MODE == 1 && SF >= 1)
 #pragma unroll
@@ -478,7 +484,7 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
 #pragma unroll
       for (int k = 0; k < N; ++k) {
         if (cons) {
-          const float2 w = __ldg(A.wphys + e * NF + ed * N + k);
+          const float2 w = reinterpret_cast<const float2*>(tb)[lane * NF + ed * N + k];
 #pragma unroll
           for (int f = 0; f < NFLD; ++f) bal[f] = ff_add(bal[f], ff_mul(w, isl ? F[f][ed][k] : -F[f][ed][k]));
         }
@@ -511,7 +517,7 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
     for (int j = 0; j < NU; ++j) {
       float2 wd = make_float2(0.f, 0.f);
       if (SF == 4 && cons) {
-        wd = __ldg(A.wdetf + e * NU + j);
+        wd = reinterpret_cast<const float2*>(wb)[lane * NU + j];
         W = ff_add(W, wd);
       }
 #pragma unroll
@@ -580,7 +586,8 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
 #pragma unroll
       for (int j = 0; j < NU; ++j) yr[j] = phi_keep[j];
   }
-  // ---- traces of the new stage value
+  // ---- traces of the new stage value (psi's alone are packed across the lanes' weights)
+  if (NFLD == 1) __syncwarp();
   float* trr = tb + lane * NFLD * NF;
 #pragma unroll
   for (int ed = 0; ed < 3; ++ed) {

@@ -93,7 +93,8 @@ def test_line_kernel_options(G, etype, order, ns, jitter, vel, normal, wall):
 
 
 @pytest.mark.parametrize("etype,order,ns,vel", [("quad", 4, (9, 7), "rider_kothe"), ("hex", 3, (4, 3, 3), "leveque"),
-                                                ("hex", 4, (3, 3, 2), "leveque"), ("quad", 3, (5, 4), "rotation")])
+                                                ("hex", 4, (3, 3, 2), "leveque"), ("quad", 3, (5, 4), "rotation"),
+                                                ("quad", 5, (5, 4), "stream")])
 def test_an_element_does_not_depend_on_the_rest_of_the_mesh(G, etype, order, ns, vel):
     """An axis-aligned grid alone (every element takes the diagonal path) and
     in a union with a jittered one march to the same bits."""
