@@ -231,6 +231,7 @@ KArgs shadow_args(const fr_field* f, const AdjRecord& R) {
   a.fc = R.ws + R.off_fc64;
   a.mcg = R.ws + R.off_mc64;
   a.vsu = a.vsf = nullptr;
+  a.vtabd = nullptr;
   a.tacc = nullptr;
   a.ep = nullptr;
   return a;

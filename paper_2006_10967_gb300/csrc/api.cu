@@ -24,6 +24,7 @@ struct Layout {
   size_t tri_pack;                // their packed form (TriPack)
   size_t wphys;                   // triangles: physical edge quadrature weight per flux point (float-float)
   size_t ffw;                     // hexahedra: face words (KArgs.ffw)
+  size_t vtab64;                  // FP64 tensor fields with a separable velocity: its tables (KArgs.vtabd)
   size_t vtab;                    // mixed tensor fields with a velocity cache: velocity factors (KArgs.vtab)
   size_t total;
 };
@@ -192,7 +193,8 @@ int most_blocks(const fr_mesh& m, const KernelSet& ks, int elementwise) {
   return (int)n;
 }
 
-Layout make_layout(const fr_mesh& m, int precision, int max_blocks, int vel_cache) {
+Layout make_layout(const fr_mesh& m, const fr_params& prm, int max_blocks) {
+  const int precision = prm.precision, vel_cache = prm.vel_cache;
   Layout L{};
   const size_t E = (size_t)m.E, NU = m.nu, NF = m.nf, NG = (size_t)m.dim * m.ncoef;
   const size_t tb = precision == FR_FP64 ? 8 : 4;
@@ -225,6 +227,9 @@ Layout make_layout(const fr_mesh& m, int precision, int max_blocks, int vel_cach
   L.ep = take(E * sizeof(ElemPar));
   L.mcg = m.etype != FR_TRI ? take(E * kMetricRec * tb) : 0;  // per-element metric records
   L.ffw = m.etype == FR_HEX ? take(E * 6 * sizeof(int2)) : 0;
+  L.vtab64 = m.etype != FR_TRI && precision == FR_FP64 && vel_separable(prm.vel.kind)
+                 ? take(E * m.dim * (m.n + 2) * 2 * sizeof(double))
+                 : 0;
   L.vtab = m.etype != FR_TRI && precision == FR_MIXED && vc ? take(E * m.dim * (m.n + 2) * sizeof(float2)) : 0;
   if (m.etype == FR_TRI) {
     const size_t nops = tri_op_count(m);
@@ -355,7 +360,7 @@ __device__ __forceinline__ void u_put(const KArgs& A, int mixed, int64_t g, doub
     return;
   }
   const float hi = (float)x;
-  reinterpret_cast<float2*>(A.u)[g] = make_float2(hi, (float)(x - (double)hi));
+  reinterpret_cast<float2*>(A.u)[g] = make_float2(hi, (float)(x - widen(hi)));
 }
 
 template <typename T>
@@ -681,7 +686,7 @@ extern "C" int fr_field_workspace_bytes(const fr_mesh* m, const fr_params* prm, 
   int mg;
   launch_elementwise_grid(m->E * m->nu, &mg);
   const int mb = most_blocks(*m, ks, mg);
-  *bytes = make_layout(*m, prm->precision, mb, prm->vel_cache).total;
+  *bytes = make_layout(*m, *prm, mb).total;
   return FR_OK;
 }
 
@@ -698,7 +703,7 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
   int mg;
   launch_elementwise_grid(m->E * m->nu, &mg);
   const int mb = most_blocks(*m, ks, mg);
-  const Layout L = make_layout(*m, prm->precision, mb, prm->vel_cache);
+  const Layout L = make_layout(*m, *prm, mb);
   if (ws_bytes < L.total) return FR_ENOMEM;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
 
@@ -739,7 +744,9 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
   f->precision = prm->precision;
   f->prm = *prm;
   f->ks = ks;
+  // enough threads to fill the FP64 pipes; more blocks add reductions of their own
   launch_elementwise_grid(ndof, &f->mass_grid);
+  f->mass_grid = std::min(f->mass_grid, 152 * 4);
 
   char* b = reinterpret_cast<char*>(ws);
   KArgs& A = f->args;
@@ -769,6 +776,7 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
   A.ep = nullptr;
   A.mcg = L.mcg ? b + L.mcg : nullptr;
   A.vtab = nullptr;
+  A.vtabd = L.vtab64 ? reinterpret_cast<const double*>(b + L.vtab64) : nullptr;
   fill_line_ops(m, A.lo);
   const bool diagonal = m->etype != FR_TRI && all_diagonal(*m);
   if (use_line_kernels(*m, *prm)) {
@@ -806,6 +814,7 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
     h = (float)v;
     l = (float)(v - (double)h);
   };
+  A.prm.ramp_lo = (float)(std::pow(10.0, prm->s0 - prm->kappa) * (1.0 - 1e-5));
   const double rs = M_PI / (4.0 * prm->kappa);
   split(-rs * (prm->s0 - prm->kappa), A.prm.ramp_c0h, A.prm.ramp_c0l);
   split(rs * std::log10(2.0), A.prm.ramp_c1h, A.prm.ramp_c1l);
@@ -916,6 +925,7 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
     else f->ks.vcache(A, s);
   }
   if (err == FR_OK && A.vtab) f->ks.vtab(A, s);
+  if (err == FR_OK && A.vtabd) f->ks.vtab64(A, s);
   if (err == FR_OK) err = stage_and_traces(f, s);
   if (err == FR_OK && ic->precondition && prm->normal == FR_NORMAL_PSI) err = run_precondition(f, s);
   if (err == FR_OK && cudaStreamSynchronize(s) != cudaSuccess) err = FR_ECUDA;

@@ -71,8 +71,10 @@ void launch_kb_pseudo(const KArgs& A, cudaStream_t s) {
 
 template <int DIM, int N, bool GEN, int SF>
 void launch_kap_stage(const KArgs& A, cudaStream_t s) {
-  kap_line<DIM, N, GEN, kPseudoWarps, SF>
-      <<<line_grid<DIM, N>(A.E, kPseudoWarps), kPseudoWarps * 32, KAPLine<DIM, N, GEN>::F * 4 * kPseudoWarps, s>>>(A);
+  constexpr int smem = KAPLine<DIM, N, GEN>::F * 4 * kPseudoWarps;
+  unsigned grid = line_grid<DIM, N>(A.E, kPseudoWarps);
+  if (SF == 4 && grid > kPseudoBlocks) grid = kPseudoBlocks;
+  kap_line<DIM, N, GEN, kPseudoWarps, SF><<<grid, kPseudoWarps * 32, smem, s>>>(A);
 }
 
 template <int DIM, int N, bool GEN>

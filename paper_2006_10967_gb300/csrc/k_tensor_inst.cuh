@@ -56,6 +56,26 @@ bool prepare_tensor() {
   return ok;
 }
 
+template <int DIM, int N>
+void launch_vel_tab64(const KArgs& A, cudaStream_t s) {
+  k_vel_tab64<DIM, N><<<152 * 8, kThreads, 0, s>>>(A);
+}
+
+// FP64 fields are bound by the FP64 pipe of the busiest SM (16 clocks a warp
+// instruction whatever its active lanes), so by its number of warps: one-warp
+// tiles are taken where they leave fewer there, 8 % allowed for the per-block
+// time factor.  256 quads p = 3: residual and update kernels of 11 and 4 blocks
+// (three and eight warps on an SM) against 32 blocks of one warp; 13,824 hexes
+// p = 3: 52 against 46 warps on the busiest SM.
+template <typename Tile, typename One>
+bool one_warp_better(int64_t E) {
+  const auto busiest = [&](int et, int threads) {
+    const int64_t blocks = (E + et - 1) / et;
+    return (double)((blocks + 151) / 152 * (threads / 32));
+  };
+  return 1.08 * busiest(One::ET, One::THREADS) < busiest(Tile::ET, Tile::THREADS);
+}
+
 // TB, TA: the tile divisors of the physical-step residual and update
 // kernels (the kernel variant; the preconditioning kernels keep the default
 // tiles)
@@ -71,6 +91,15 @@ void fill_tensor(int64_t E, KernelSet* ks) {
   ks->ka_rate = ks->ka[0];
   ks->ka[1] = launch_ka_tensor<DIM, N, T, 1>;
   ks->ka_rate_pseudo = ks->ka[1];
+  if constexpr (sizeof(T) == 8) {
+    ks->vtab64 = launch_vel_tab64<DIM, N>;
+    ks->prepared = ks->prepared && prepare_tensor<DIM, N, T, 0, 0>();
+    if (one_warp_better<KBLayout<DIM, N, T, 0, TB>, KBLayout<DIM, N, T, 0, 0>>(E)) ks->kb[0] = launch_kb_tensor<DIM, N, T, 0, 0>;
+    if (one_warp_better<KALayout<DIM, N, T, 0, TA>, KALayout<DIM, N, T, 0, 0>>(E)) {
+      ks->ka[0] = launch_ka_tensor<DIM, N, T, 0, 0>;
+      ks->ka_rate = ks->ka[0];
+    }
+  }
   const int et_min = KBLayout<DIM, N, T, 0, TB>::ET < KALayout<DIM, N, T, 0, TA>::ET ? KBLayout<DIM, N, T, 0, TB>::ET
                                                                                       : KALayout<DIM, N, T, 0, TA>::ET;
   const int et_min1 = KBLayout<DIM, N, T, 1>::ET < KALayout<DIM, N, T, 1>::ET ? KBLayout<DIM, N, T, 1>::ET

@@ -46,7 +46,8 @@ struct PhysPrm {
   double T;   // period of the velocity time factor (<= 0: none)
   double rT;  // 1 / T (0 when T <= 0)
   // the resolution indicator's ramp in float-float pairs (sensor_nu): z = c0 + k c1 + (log m / 2) c2, nu_max
-  float ramp_c0h, ramp_c0l, ramp_c1h, ramp_c1l, ramp_c2h, ramp_c2l, nu_h, nu_l;
+  // and an energy ratio certainly below it (1e-5 under 10^(s0 - kappa))
+  float ramp_lo, ramp_c0h, ramp_c0l, ramp_c1h, ramp_c1l, ramp_c2h, ramp_c2l, nu_h, nu_l;
 };
 
 // 1D tensor operators; kernels stage them into shared memory.
@@ -146,6 +147,7 @@ struct KArgs {
   const float2* wdetf;   // E x nu: w_i det J_i as float-float pairs (mixed path)
   void* mcg;             // tensor elements: E x 16 metric records (bulk type)
   const float2* vtab;    // mixed tensor fields: E x dim x (n + 2) velocity factors (k_vel_tab), or nullptr
+  const double* vtabd;   // FP64 tensor fields: E x dim x (n + 2) x 2 separable velocity tables, or nullptr
   const float2* wphys;   // triangles: E x nf physical flux-point weights (float-float), equal on both sides
   int stage;             // 1..4 RK stage, -1: write the rate into out
   int use_dev_time;      // KB: t = dstate[DS_TIME] + c_s dt

@@ -14,6 +14,7 @@ struct KernelSet {
   LaunchFn ka_rate = nullptr;           // the block-wide ka[0], ka[1]: their stage -1 writes the
   LaunchFn ka_rate_pseudo = nullptr;    // rate into KArgs.out
   LaunchFn vtab = nullptr;              // fills the velocity factor table (line kernels)
+  LaunchFn vtab64 = nullptr;            // fills the separable velocity tables (FP64 tensor fields)
   int max_blocks = 0;                   // upper bound on blocks of any launch (per element count)
   LaunchFn vcache = nullptr;            // fills the spatial velocity cache (nullptr: not supported)
   LaunchFn mconst = nullptr;            // fills the per-element metric records (tensor elements)
@@ -46,6 +47,8 @@ bool reg_kernels_tri(int order, bool physical, KernelSet* ks);
 // block for the last block to add up and takes four (stage 4 of 64^3: with two
 // warps a block the update kernel's mean goes from 122 to 151 us).
 constexpr int kLineWarps = 2, kPseudoWarps = 4;
+// Blocks of the preconditioning's stage 4 update: six of 128 threads on each SM.
+constexpr unsigned kPseudoBlocks = 152 * 6;
 
 template <typename K>
 inline void launch_kernel(K kern, size_t smem, int et, const KArgs& A, cudaStream_t s, int threads = kThreads) {

@@ -52,7 +52,9 @@ __device__ __forceinline__ float2 ff_div(float2 a, float2 b) {
 // the FP64 evaluation was (log10 and sin in FP64 took a warp 3000 cycles of the
 // FP64 pipe wherever one of its elements lies in the ramp).
 __device__ __forceinline__ float sensor_nu(const PhysPrm& P, float2 lo, float2 hi, float2 nu_max) {
-  if (!(lo.x + hi.x > 0.f) || !(hi.x > 0.f)) return 0.f;
+  const float tot = lo.x + hi.x;
+  if (!(tot > 0.f) || !(hi.x > 0.f)) return 0.f;
+  if (hi.x < P.ramp_lo * tot) return 0.f;  // most elements: flat or resolved
   const float2 r = ff_div(hi, ff_add(lo, hi));
   // r = m 2^k
   int k = (__float_as_int(r.x) >> 23) - 127;
@@ -470,6 +472,11 @@ struct KAPLine {
 
 // SF: stage 1..4, or 0 to recompute the traces of psi alone.  GEN false: every
 // element is affine.
+//
+// Stage 4 leaves one partial of the residual a block, so its grid is resident
+// and every warp walks over tiles (one tile a warp and 8,000 partials cost
+// stage 4 of 64,000 hexes p = 3 58.6 us where the other stages take 24); the
+// other stages make one pass.
 template <int DIM, int N, bool GEN, int WPB, int SF>
 __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
   using L = LL<DIM, N>;
@@ -483,16 +490,20 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
   float* in = C0 + K::COR_F;
   const int es = L::FULL ? lane / LN : min(lane / LN, EPW - 1), l = lane - (lane / LN) * LN;
   const bool lane_ok = L::FULL || lane < EPW * LN;
-  const int64_t e0 = ((int64_t)blockIdx.x * WPB + warp) * EPW;
-  const int64_t eraw = e0 + es;
-  const bool act = lane_ok && eraw < A.E;
-  const int64_t e = eraw < A.E ? eraw : A.E - 1;
-  const int ne = (int)max((int64_t)0, min((int64_t)EPW, A.E - e0));
   float* ustg = reinterpret_cast<float*>(A.ustg);
   float* acc = reinterpret_cast<float*>(A.acc);
   float2* U = reinterpret_cast<float2*>(A.u);
   const float* fcA = reinterpret_cast<const float*>(A.fc);
   const LineOps& O = A.lo;
+  [[maybe_unused]] float2 sum = make_float2(0.f, 0.f);  // stage 4: squared residuals
+
+#pragma unroll 1
+  for (int64_t e0 = ((int64_t)blockIdx.x * WPB + warp) * EPW; e0 < A.E;
+       e0 += SF == 4 ? (int64_t)gridDim.x * WPB * EPW : A.E) {
+  const int64_t eraw = e0 + es;
+  const bool act = lane_ok && eraw < A.E;
+  const int64_t e = eraw < A.E ? eraw : A.E - 1;
+  const int ne = (int)min((int64_t)EPW, A.E - e0);
 
   // ---- loads
   float2 y[NP], u[N];
@@ -719,24 +730,29 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
   }
 
   if constexpr (SF == 4) {
+    // 1 / dtau^2 times the lane's squared changes
+    const RKConstF& rk = A.ep ? A.ep[e].rkp : A.rk;
+    if (act) sum = ff_add(sum, ff_mul2(ff_add(make_float2(sh.x, sl.x), make_float2(sh.y, sl.y)), make_float2(rk.r2h, rk.r2l)));
+    __syncwarp();  // the tile's buffers are read
+  }
+  }  // tiles
+
+  if constexpr (SF == 4) {
     // RMS of the pseudo-time residual: float-float to the warp's sum, FP64 over the block
     __shared__ double part[WPB];
     __shared__ double red_sh[32];
-    float2 v = ff_add(make_float2(sh.x, sl.x), make_float2(sh.y, sl.y));
-    const RKConstF& rk = A.ep ? A.ep[e].rkp : A.rk;
-    v = ff_mul2(v, make_float2(rk.r2h, rk.r2l));
-    if (!act) v = make_float2(0.f, 0.f);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       float2 t;
-      t.x = __shfl_xor_sync(0xffffffffu, v.x, o);
-      t.y = __shfl_xor_sync(0xffffffffu, v.y, o);
-      v = ff_add(v, t);
+      t.x = __shfl_xor_sync(0xffffffffu, sum.x, o);
+      t.y = __shfl_xor_sync(0xffffffffu, sum.y, o);
+      sum = ff_add(sum, t);
     }
-    if (lane == 0) part[warp] = (double)v.x + (double)v.y;
+    if (lane == 0) part[warp] = (double)sum.x + (double)sum.y;
     __syncthreads();
     double s = 0.0;
-    for (int w = 0; w < WPB; ++w) s += part[w];
+    if (threadIdx.x == 0)
+      for (int w = 0; w < WPB; ++w) s += part[w];
     pseudo_rms_finish(A, s, red_sh, A.E * NU);
   }
 }

@@ -289,7 +289,11 @@ __host__ __device__ constexpr int occupancy_tile(int bytes_el, int per_block, in
 
 // TD: tile divisor of a kernel variant (1: the default tile below; 2: half
 // of it, rounded to whole warps where possible), chosen per element type,
-// order and precision by the autotuner.
+// order and precision by the autotuner; 0: one warp's elements (FP64 fields,
+// see one_warp_better).
+__host__ __device__ constexpr int tile_of(int et0, int td, int ln) {
+  return td == 0 ? (ln <= 32 ? 32 / ln : 1) : td == 1 ? et0 : (et0 / td < 1 ? 1 : warp_tile(et0 / td, ln));
+}
 template <int DIM, int N, typename T, int MODE, int TD = 1>
 struct KBLayout {
   using S = TS<DIM, N>;
@@ -313,7 +317,7 @@ struct KBLayout {
   static constexpr bool OCC = MODE == 0 && DIM == 3;  // tile chosen for resident warps
   static constexpr int ET0 = OCC ? occupancy_tile(BYTES_EL, 16 * 13 + 2 * (int)sizeof(T) + 64, LN, ET_T)
                                  : warp_tile(ET_T < ET_S ? ET_T : ET_S, LN);
-  static constexpr int ET = TD == 1 ? ET0 : (ET0 / TD < 1 ? 1 : warp_tile(ET0 / TD, LN));
+  static constexpr int ET = tile_of(ET0, TD, LN);
   static constexpr int FS = FRP_FIELD_SPLIT ? NFLD : 1;  // fields split across threads
   static constexpr int LINES = ET * LN;
   static constexpr int THREADS = (LINES * FS + 31) / 32 * 32;  // whole warps; idle lanes inactive
@@ -424,6 +428,10 @@ __device__ __forceinline__ void kb_tensor_body(const KArgs& A, const int blk) {
   const T* vsf = reinterpret_cast<const T*>(A.vsf);
   if (LY::VT && A.vsu) tile_async(vu, vsu + e0 * DIM * NU, ne * DIM * NU * (int)sizeof(T));
   if (LY::VT && A.vsf) tile_async(vf, vsf + e0 * DIM * NF, ne * DIM * NF * (int)sizeof(T));
+  // FP64 fields keep the separable velocity tables of all elements (a sincospi
+  // in FP64 is some 60 instructions on a pipe of 2 lanes a clock)
+  const bool tabs = MODE == 0 && sizeof(T) == 8 && A.vtabd != nullptr;
+  if (tabs) tile_async(vtab, A.vtabd + e0 * DIM * NT * 2, ne * DIM * NT * 2 * (int)sizeof(T));
   if constexpr (DIM == 3) {
     if (lact) {
       const int fi = ll % N, fj = ll / N;
@@ -450,7 +458,7 @@ __device__ __forceinline__ void kb_tensor_body(const KArgs& A, const int blk) {
   // separable velocity: per-axis tables of the elements with a diagonal map
   // (read after the first axis pass's barrier)
   const bool sepk = MODE == 0 && vel_separable(BC.vel.kind);
-  if (sepk)
+  if (sepk && !tabs)
     for (int t = tid; t < ne * DIM * NT; t += blockDim.x) {
       const int el = t / (DIM * NT), r = t % (DIM * NT), c = r / NT, j = r % NT;
       if (mcs[el * kKbRec + 11] != (T)2) continue;
@@ -1065,7 +1073,7 @@ struct KALayout {
   static constexpr int ET_T = 256 / LN < 1 ? 1 : 256 / LN;
   static constexpr int ET_S = 45056 / BYTES_EL < 1 ? 1 : 45056 / BYTES_EL;
   static constexpr int ET0 = warp_tile(ET_T < ET_S ? ET_T : ET_S, LN);
-  static constexpr int ET = TD == 1 ? ET0 : (ET0 / TD < 1 ? 1 : warp_tile(ET0 / TD, LN));
+  static constexpr int ET = tile_of(ET0, TD, LN);
   static constexpr int FS = FRP_FIELD_SPLIT ? NFLD : 1;  // fields split across threads
   static constexpr int LINES = ET * LN;
   static constexpr int THREADS = (LINES * FS + 31) / 32 * 32;  // whole warps; idle lanes inactive
@@ -1413,6 +1421,21 @@ template <int DIM, typename T, int MODE>
 struct StageKA {
   static constexpr bool v = DIM == 3 && sizeof(T) == 4 && MODE == 0;
 };
+
+// The separable velocity tables (vel_tab_entry) of every element of an FP64
+// field, E x DIM x (N + 2) x 2; read for elements with a diagonal map.
+template <int DIM, int N>
+__global__ void k_vel_tab64(const KArgs A) {
+  constexpr int NT = N + 2, NC = TS<DIM, N>::NC;
+  const int64_t n = A.E * DIM * NT;
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t e = q / (DIM * NT);
+    const int r = (int)(q % (DIM * NT)), c = r / NT, j = r % NT;
+    const double* g = A.geo + e * TS<DIM, N>::NG + c * NC;
+    const double xi = j < N ? A.cd.ops.x[j] : (j == N ? -1.0 : 1.0);
+    vel_tab_entry<double>(A.cd.vel.kind, g[0] + g[1 + c] * xi, const_cast<double*>(A.vtabd) + q * 2);
+  }
+}
 
 // Spatial velocity factor v(x) (g = 1) at the solution and flux points of
 // every element, evaluated once in double and stored in the bulk type.
