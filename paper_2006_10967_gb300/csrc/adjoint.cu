@@ -65,15 +65,27 @@ void la(const AdjArgs& B, cudaStream_t s) {
   using LY = AdjLayout<DIM, N>;
   adj_a<DIM, N><<<(unsigned)((B.K.E + LY::ET - 1) / LY::ET), LY::THREADS, 0, s>>>(B);
 }
-template <int DIM, int N, int MODE>
-void lb(const AdjArgs& B, cudaStream_t s) {
-  using LY = AdjLayout<DIM, N>;
+template <int DIM, int N, int MODE, int TD>
+void lb_tile(const AdjArgs& B, cudaStream_t s) {
+  using LY = AdjLayout<DIM, N, TD>;
   static bool init = false;
   if (!init) {
-    cudaFuncSetAttribute(adj_b<DIM, N, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LY::SMEM);
+    cudaFuncSetAttribute(adj_b<DIM, N, MODE, TD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LY::SMEM);
     init = true;
   }
-  adj_b<DIM, N, MODE><<<(unsigned)((B.K.E + LY::ET - 1) / LY::ET), LY::THREADS, LY::SMEM, s>>>(B);
+  adj_b<DIM, N, MODE, TD><<<(unsigned)((B.K.E + LY::ET - 1) / LY::ET), LY::THREADS, LY::SMEM, s>>>(B);
+}
+// One-warp tiles where they leave fewer warps on the busiest SM, as the FP64
+// field kernels (4,096 quads p = 4: five instead of six).
+template <int DIM, int N, int MODE>
+void lb(const AdjArgs& B, cudaStream_t s) {
+  const auto busiest = [&](int et, int threads) {
+    return ((B.K.E + et - 1) / et + 151) / 152 * ((threads + 31) / 32);
+  };
+  using L1 = AdjLayout<DIM, N, 1>;
+  using L0 = AdjLayout<DIM, N, 0>;
+  if (busiest(L0::ET, L0::THREADS) < busiest(L1::ET, L1::THREADS)) lb_tile<DIM, N, MODE, 0>(B, s);
+  else lb_tile<DIM, N, MODE, 1>(B, s);
 }
 template <int DIM, int N>
 void lc(const AdjArgs& B, cudaStream_t s) {

@@ -1,5 +1,8 @@
 // Instantiation helpers for the tensor kernels (included by k_quad.cu, k_hex.cu).
 #pragma once
+#include <algorithm>
+#include <cmath>
+
 #include "kdispatch.hpp"
 #include "ktensor.cuh"
 
@@ -61,19 +64,31 @@ void launch_vel_tab64(const KArgs& A, cudaStream_t s) {
   k_vel_tab64<DIM, N><<<152 * 8, kThreads, 0, s>>>(A);
 }
 
-// FP64 fields are bound by the FP64 pipe of the busiest SM (16 clocks a warp
-// instruction whatever its active lanes), so by its number of warps: one-warp
-// tiles are taken where they leave fewer there, 8 % allowed for the per-block
-// time factor.  256 quads p = 3: residual and update kernels of 11 and 4 blocks
-// (three and eight warps on an SM) against 32 blocks of one warp; 13,824 hexes
-// p = 3: 52 against 46 warps on the busiest SM.
-template <typename Tile, typename One>
-bool one_warp_better(int64_t E) {
-  const auto busiest = [&](int et, int threads) {
-    const int64_t blocks = (E + et - 1) / et;
-    return (double)((blocks + 151) / 152 * (threads / 32));
-  };
-  return 1.08 * busiest(One::ET, One::THREADS) < busiest(Tile::ET, Tile::THREADS);
+// FP64 fields: the residual kernel's time in clocks with tile layout LY, as the
+// larger of the FP64 pipe's work on the busiest SM (16 clocks a warp
+// instruction whatever its active lanes) and one block's chain of dependent
+// instructions (about 90 clocks each with few warps on an SM).  A warp executes
+// about DIM 4 N (N + 4) FP64 instructions in the line passes, 90 a round of
+// points (in the line pass for odd N) and 110 a round of common-flux points.
+// 256 quads p = 3: 39.8 us with the default tile (11 blocks), 38.8 with one
+// warp's eight elements, 28.7 with four, 22.4 with one or two; 4,096 quads
+// p = 4: 67 us with the default tile (two blocks of three warps on an SM), 55
+// with one warp's.
+template <int DIM, int N, typename LY>
+double kb_clocks(int64_t E) {
+  using S = TS<DIM, N>;
+  constexpr int W = LY::THREADS / 32;
+  constexpr double line = DIM * 4.0 * N * (N + 4) + (N % 2 ? 90.0 * N : 0.0);
+  constexpr double pts = N % 2 ? 0.0 : 90.0, flux = 110.0;
+  const auto up = [](double a, double b) { return std::ceil(a / b); };
+  const double work = W * line + up(LY::ET * S::NU, 32) * pts + up(LY::ET * S::NF / 2.0, 32) * flux;
+  const double chain = line + up(LY::ET * S::NU, LY::THREADS) * pts + up(LY::ET * S::NF / 2.0, LY::THREADS) * flux;
+  return std::max(16.0 * up(up((double)E, LY::ET), 152) * work, 90.0 * chain);
+}
+// The update kernel has no rounds: the warps on the busiest SM decide.
+template <typename LY>
+int64_t ka_warps(int64_t E) {
+  return ((E + LY::ET - 1) / LY::ET + 151) / 152 * (LY::THREADS / 32);
 }
 
 // TB, TA: the tile divisors of the physical-step residual and update
@@ -93,9 +108,12 @@ void fill_tensor(int64_t E, KernelSet* ks) {
   ks->ka_rate_pseudo = ks->ka[1];
   if constexpr (sizeof(T) == 8) {
     ks->vtab64 = launch_vel_tab64<DIM, N>;
-    ks->prepared = ks->prepared && prepare_tensor<DIM, N, T, 0, 0>();
-    if (one_warp_better<KBLayout<DIM, N, T, 0, TB>, KBLayout<DIM, N, T, 0, 0>>(E)) ks->kb[0] = launch_kb_tensor<DIM, N, T, 0, 0>;
-    if (one_warp_better<KALayout<DIM, N, T, 0, TA>, KALayout<DIM, N, T, 0, 0>>(E)) {
+    ks->prepared = ks->prepared && prepare_tensor<DIM, N, T, 0, 0>() && prepare_tensor<DIM, N, T, 0, -1>();
+    const double t1 = kb_clocks<DIM, N, KBLayout<DIM, N, T, 0, TB>>(E), t0 = kb_clocks<DIM, N, KBLayout<DIM, N, T, 0, 0>>(E),
+                 tq = kb_clocks<DIM, N, KBLayout<DIM, N, T, 0, -1>>(E);
+    if (tq < t0 && tq < t1) ks->kb[0] = launch_kb_tensor<DIM, N, T, 0, -1>;
+    else if (t0 < t1) ks->kb[0] = launch_kb_tensor<DIM, N, T, 0, 0>;
+    if (ka_warps<KALayout<DIM, N, T, 0, 0>>(E) < ka_warps<KALayout<DIM, N, T, 0, TA>>(E)) {
       ks->ka[0] = launch_ka_tensor<DIM, N, T, 0, 0>;
       ks->ka_rate = ks->ka[0];
     }

@@ -53,7 +53,8 @@ struct AdjArgs {
   double* lam_psi0;     // preconditioning sweep: E x NU, += (dR_p/dpsi0)^T lam (adj_b<.., 1>)
 };
 
-template <int DIM, int N>
+// TD: 1 the default tile, 0 one warp's elements (see one_warp_better).
+template <int DIM, int N, int TD = 1>
 struct AdjLayout {
   using S = TS<DIM, N>;
   static constexpr int LN = S::NFP;
@@ -68,7 +69,7 @@ struct AdjLayout {
   static constexpr int BYTES_EL = PER_EL * 8 + S::NF;
   static constexpr int ET_T = 256 / LN < 1 ? 1 : 256 / LN;
   static constexpr int ET_S = 49152 / BYTES_EL < 1 ? 1 : 49152 / BYTES_EL;
-  static constexpr int ET = ET_T < ET_S ? ET_T : ET_S;
+  static constexpr int ET = tile_of(ET_T < ET_S ? ET_T : ET_S, TD, LN);
   static constexpr int THREADS = ET * LN;
   static constexpr size_t SMEM = (size_t)ET * BYTES_EL + 64;
 };
@@ -103,32 +104,41 @@ __global__ void k_coef_table(const KArgs A, double* cs) {
 //   dA_m += 2 pi g sum_p w_pm cos th_pm,  dB_m -= 2 pi g sum_p w_pm sin th_pm,
 //   w_pm = k_y,m lv0_p - k_x,m lv1_p,
 // over the points p of block b's share, to coefp[b][.] (no atomics).
-// Launch: blocks = the partial slots, 256 threads = 32 mode lanes x 8 groups.
+// Launch: blocks = the partial slots, 256 threads = 8 warps.  A warp takes as
+// many points at once as its lanes hold modes (a power of two): bound by the
+// FP64 pipe at 16 clocks a warp instruction whatever its active lanes, 16 modes
+// on 32 lanes left half of it unused (57 us a stage of 184,320 points).
 __global__ void k_coef_acc(const double* lv, const double* cs, int64_t npts, VelDescT<double> V, double g,
                            double* coefp) {
   const int M = V.n_modes, M2 = 2 * M;
-  const int m = threadIdx.x & 31, grp = threadIdx.x >> 5, ngrp = blockDim.x >> 5;
+  int mp = 1;
+  while (mp < M) mp *= 2;
+  const int lane = threadIdx.x & 31, m = lane & (mp - 1), sub = lane / mp, pw = 32 / mp;
+  const int grp = threadIdx.x >> 5, ngrp = blockDim.x >> 5;
   const int64_t per = (npts + gridDim.x - 1) / gridDim.x;
   const int64_t p0 = (int64_t)blockIdx.x * per, p1 = p0 + per < npts ? p0 + per : npts;
   double ac = 0.0, as = 0.0;
   if (m < M) {
     const double kx = V.kx[m], ky = V.ky[m];
-    for (int64_t p = p0 + grp; p < p1; p += ngrp) {
-      const double w = ky * lv[2 * p] - kx * lv[2 * p + 1];
-      ac += w * cs[(p * M + m) * 2 + 0];
-      as += w * cs[(p * M + m) * 2 + 1];
+    for (int64_t p = p0 + grp * pw + sub; p < p1; p += ngrp * pw) {
+      const double2 l = *reinterpret_cast<const double2*>(lv + 2 * p);
+      const double2 t = *reinterpret_cast<const double2*>(cs + (p * M + m) * 2);
+      const double w = ky * l.x - kx * l.y;
+      ac += w * t.x;
+      as += w * t.y;
     }
   }
   __shared__ double red[2][8][32];
-  red[0][grp][m] = ac;
-  red[1][grp][m] = as;
+  red[0][grp][lane] = ac;
+  red[1][grp][lane] = as;
   __syncthreads();
-  if (grp == 0 && m < M) {
+  if (grp == 0 && sub == 0 && m < M) {
     double sc = 0.0, ss = 0.0;
-    for (int q = 0; q < ngrp; ++q) {
-      sc += red[0][q][m];
-      ss += red[1][q][m];
-    }
+    for (int q = 0; q < ngrp; ++q)
+      for (int k = m; k < 32; k += mp) {
+        sc += red[0][q][k];
+        ss += red[1][q][k];
+      }
     const double f = 2.0 * M_PI * g;
     coefp[(int64_t)blockIdx.x * M2 + m] += f * sc;
     coefp[(int64_t)blockIdx.x * M2 + M + m] -= f * ss;
@@ -180,10 +190,10 @@ __global__ void __launch_bounds__(256) adj_a(const AdjArgs B) {
 }
 
 // ---------------------------------------------------------------------------
-template <int DIM, int N, int MODE = 0>
+template <int DIM, int N, int MODE = 0, int TD = 1>
 __global__ void __launch_bounds__(256) adj_b(const AdjArgs B) {
   using S = TS<DIM, N>;
-  using LY = AdjLayout<DIM, N>;
+  using LY = AdjLayout<DIM, N, TD>;
   constexpr int NU = S::NU, NF = S::NF, NG = S::NG, NFP = S::NFP, ET = LY::ET, LN = LY::LN;
   const KArgs& A = B.K;
   extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -289,10 +289,13 @@ __host__ __device__ constexpr int occupancy_tile(int bytes_el, int per_block, in
 
 // TD: tile divisor of a kernel variant (1: the default tile below; 2: half
 // of it, rounded to whole warps where possible), chosen per element type,
-// order and precision by the autotuner; 0: one warp's elements (FP64 fields,
-// see one_warp_better).
+// order and precision by the autotuner; 0: one warp's elements, -1: a quarter
+// of a warp's (FP64 fields, see kb_clocks).
 __host__ __device__ constexpr int tile_of(int et0, int td, int ln) {
-  return td == 0 ? (ln <= 32 ? 32 / ln : 1) : td == 1 ? et0 : (et0 / td < 1 ? 1 : warp_tile(et0 / td, ln));
+  return td == 0    ? (ln <= 32 ? 32 / ln : 1)
+         : td == -1 ? (32 / ln / 4 < 1 ? 1 : 32 / ln / 4)
+         : td == 1  ? et0
+                    : (et0 / td < 1 ? 1 : warp_tile(et0 / td, ln));
 }
 template <int DIM, int N, typename T, int MODE, int TD = 1>
 struct KBLayout {
