@@ -184,7 +184,7 @@ bool set_line_kernels(const fr_mesh& m, bool gen, bool tab, KernelSet* ks) {
 // Blocks of the largest launch (one reduction partial each): the block-wide
 // kernels', the element-wise kernels' or the line kernels'.
 int most_blocks(const fr_mesh& m, const KernelSet& ks, int elementwise) {
-  int64_t n = std::max(ks.max_blocks, elementwise);
+  int64_t n = std::max<int64_t>({ks.max_blocks, elementwise, std::min(m.E, kSmallTileElems)});
   if (m.etype == FR_TRI) n = std::max<int64_t>(n, (m.E + 31) / 32);  // a warp a block (ka_trir)
   if (m.etype != FR_TRI && m.nfp <= 32) {
     const int per = kPseudoWarps * (32 / m.nfp);

@@ -17,14 +17,14 @@ void launch_kb_line(const KArgs& A, cudaStream_t s) {
   constexpr int smem = KBLine<DIM, N, GEN, TAB>::F * 4 * kLineWarps;
   static_assert(smem <= 48 * 1024, "no shared-memory opt-in needed");
   const unsigned grid = line_grid<DIM, N>(A.E, kLineWarps);
-  if (A.cf.prm.nphi) kb_line<DIM, N, GEN, TAB, true, kLineWarps><<<grid, kLineWarps * 32, smem, s>>>(A);
-  else kb_line<DIM, N, GEN, TAB, false, kLineWarps><<<grid, kLineWarps * 32, smem, s>>>(A);
+  if (A.cf.prm.nphi) launch_pdl(kb_line<DIM, N, GEN, TAB, true, kLineWarps>, grid, kLineWarps * 32, smem, A, s);
+  else launch_pdl(kb_line<DIM, N, GEN, TAB, false, kLineWarps>, grid, kLineWarps * 32, smem, A, s);
 }
 
 template <int DIM, int N, bool GEN, int SF>
 void launch_ka_stage(const KArgs& A, cudaStream_t s) {
-  ka_line<DIM, N, GEN, kLineWarps, SF>
-      <<<line_grid<DIM, N>(A.E, kLineWarps), kLineWarps * 32, KALine<DIM, N, SF, GEN>::F * 4 * kLineWarps, s>>>(A);
+  launch_pdl(ka_line<DIM, N, GEN, kLineWarps, SF>, line_grid<DIM, N>(A.E, kLineWarps), kLineWarps * 32,
+             KALine<DIM, N, SF, GEN>::F * 4 * kLineWarps, A, s);
 }
 
 template <int DIM, int N, bool GEN>
@@ -66,7 +66,8 @@ bool fill_line(bool gen, bool tab, KernelSet* ks) {
 
 template <int DIM, int N, bool GEN>
 void launch_kb_pseudo(const KArgs& A, cudaStream_t s) {
-  kbp_line<DIM, N, GEN, kPseudoWarps><<<line_grid<DIM, N>(A.E, kPseudoWarps), kPseudoWarps * 32, KBPLine<DIM, N, GEN>::F * 4 * kPseudoWarps, s>>>(A);
+  kbp_line<DIM, N, GEN, kPseudoWarps>
+      <<<line_grid<DIM, N>(A.E, kPseudoWarps), kPseudoWarps * 32, KBPLine<DIM, N, GEN>::F * 4 * kPseudoWarps, s>>>(A);
 }
 
 template <int DIM, int N, bool GEN, int SF>

@@ -113,6 +113,19 @@ void fill_tensor(int64_t E, KernelSet* ks) {
                  tq = kb_clocks<DIM, N, KBLayout<DIM, N, T, 0, -1>>(E);
     if (tq < t0 && tq < t1) ks->kb[0] = launch_kb_tensor<DIM, N, T, 0, -1>;
     else if (t0 < t1) ks->kb[0] = launch_kb_tensor<DIM, N, T, 0, 0>;
+    // the preconditioning's reduction keeps a partial a block: small tiles only
+    // where they stay within the slots every field has
+    if (E <= kSmallTileElems) {
+      ks->prepared = ks->prepared && prepare_tensor<DIM, N, T, 1, 0>() && prepare_tensor<DIM, N, T, 1, -1>();
+      const double p1 = kb_clocks<DIM, N, KBLayout<DIM, N, T, 1>>(E), p0 = kb_clocks<DIM, N, KBLayout<DIM, N, T, 1, 0>>(E),
+                   pq = kb_clocks<DIM, N, KBLayout<DIM, N, T, 1, -1>>(E);
+      if (pq < p0 && pq < p1) ks->kb[1] = launch_kb_tensor<DIM, N, T, 1, -1>;
+      else if (p0 < p1) ks->kb[1] = launch_kb_tensor<DIM, N, T, 1, 0>;
+      if (ka_warps<KALayout<DIM, N, T, 1, 0>>(E) < ka_warps<KALayout<DIM, N, T, 1>>(E)) {
+        ks->ka[1] = launch_ka_tensor<DIM, N, T, 1, 0>;
+        ks->ka_rate_pseudo = ks->ka[1];
+      }
+    }
     if (ka_warps<KALayout<DIM, N, T, 0, 0>>(E) < ka_warps<KALayout<DIM, N, T, 0, TA>>(E)) {
       ks->ka[0] = launch_ka_tensor<DIM, N, T, 0, 0>;
       ks->ka_rate = ks->ka[0];

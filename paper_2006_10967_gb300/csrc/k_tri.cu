@@ -4,24 +4,24 @@
 
 namespace frp {
 
-template <int P, typename T, int MODE, bool TC>
+template <int P, typename T, int MODE, bool TC, int TD = 1>
 void launch_kb_tri(const KArgs& A, cudaStream_t s) {
-  using LY = KBTriLayout<P, T, MODE, TC>;
-  launch_kernel(kb_tri<P, T, MODE, TC>, LY::SMEM, LY::ET, A, s);
+  using LY = KBTriLayout<P, T, MODE, TC, TD>;
+  launch_kernel(kb_tri<P, T, MODE, TC, TD>, LY::SMEM, LY::ET, A, s);
 }
 
-template <int P, typename T, int MODE, bool TC>
+template <int P, typename T, int MODE, bool TC, int TD = 1>
 void launch_ka_tri(const KArgs& A, cudaStream_t s) {
-  using LY = KATriLayout<P, T, MODE, TC>;
-  launch_kernel(ka_tri<P, T, MODE, TC>, LY::SMEM, LY::ET, A, s);
+  using LY = KATriLayout<P, T, MODE, TC, TD>;
+  launch_kernel(ka_tri<P, T, MODE, TC, TD>, LY::SMEM, LY::ET, A, s);
 }
 
-template <int P, typename T, int MODE, bool TC>
+template <int P, typename T, int MODE, bool TC, int TD = 1>
 bool prepare_tri() {
-  return cudaFuncSetAttribute(kb_tri<P, T, MODE, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)KBTriLayout<P, T, MODE, TC>::SMEM) == cudaSuccess &&
-         cudaFuncSetAttribute(ka_tri<P, T, MODE, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)KATriLayout<P, T, MODE, TC>::SMEM) == cudaSuccess;
+  return cudaFuncSetAttribute(kb_tri<P, T, MODE, TC, TD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)KBTriLayout<P, T, MODE, TC, TD>::SMEM) == cudaSuccess &&
+         cudaFuncSetAttribute(ka_tri<P, T, MODE, TC, TD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)KATriLayout<P, T, MODE, TC, TD>::SMEM) == cudaSuccess;
 }
 
 template <int P, typename T>
@@ -39,6 +39,23 @@ void fill_tri(int64_t E, KernelSet* ks) {
   ks->ka_rate = ks->ka[0];
   ks->ka[1] = launch_ka_tri<P, T, 1, TC>;
   ks->ka_rate_pseudo = ks->ka[1];
+  if constexpr (sizeof(T) == 8) {
+    // an FP64 tile's Steps are rounds of its threads over the tile's points, each
+    // a chain of dependent FP64 instructions: quarter tiles while they leave at
+    // most two blocks an SM
+    if ((E + KBTriLayout<P, T, 0, TC, 4>::ET - 1) / KBTriLayout<P, T, 0, TC, 4>::ET <= 2 * 152) {
+      ks->prepared = ks->prepared && prepare_tri<P, T, 0, TC, 4>() && prepare_tri<P, T, 1, TC, 4>();
+      ks->kb[0] = launch_kb_tri<P, T, 0, TC, 4>;
+      ks->kb[1] = launch_kb_tri<P, T, 1, TC, 4>;
+    }
+    if ((E + KATriLayout<P, T, 0, TC, 4>::ET - 1) / KATriLayout<P, T, 0, TC, 4>::ET <= 2 * 152) {
+      ks->prepared = ks->prepared && prepare_tri<P, T, 0, TC, 4>() && prepare_tri<P, T, 1, TC, 4>();
+      ks->ka[0] = launch_ka_tri<P, T, 0, TC, 4>;
+      ks->ka[1] = launch_ka_tri<P, T, 1, TC, 4>;
+      ks->ka_rate = ks->ka[0];
+      ks->ka_rate_pseudo = ks->ka[1];
+    }
+  }
   int et = KBTriLayout<P, T, 0, TC>::ET;
   if (KATriLayout<P, T, 0, TC>::ET < et) et = KATriLayout<P, T, 0, TC>::ET;
   if (KBTriLayout<P, T, 1, TC>::ET < et) et = KBTriLayout<P, T, 1, TC>::ET;

@@ -26,6 +26,10 @@ bool kernels_quad(int order, int precision, int64_t E, int variant, KernelSet* k
 bool kernels_hex(int order, int precision, int64_t E, int variant, KernelSet* ks);
 bool kernels_tri(int order, int precision, int64_t E, int variant, KernelSet* ks);
 
+// Largest mesh whose FP64 preconditioning may take small tiles; every field has
+// a reduction slot an element up to that size.
+constexpr int64_t kSmallTileElems = 16384;
+
 // Replace the physical-step kernels of a mixed tensor field by the line kernels
 // (kline.cuh); false where they are not built (the set is then unchanged) or
 // could not be prepared.  gen, tab: see KBLine.
@@ -49,6 +53,29 @@ bool reg_kernels_tri(int order, bool physical, KernelSet* ks);
 constexpr int kLineWarps = 2, kPseudoWarps = 4;
 // Blocks of the preconditioning's stage 4 update: six of 128 threads on each SM.
 constexpr unsigned kPseudoBlocks = 152 * 6;
+
+// Launch with programmatic stream serialisation: the kernel's blocks may start
+// while the kernel before it on the stream drains (the kernel itself waits, see
+// pdl_wait in kline.cuh).  After a kernel that does not let its dependents
+// start early, it is an ordinary launch.  us a stage with and without: 128^2
+// quads p = 4 13.8 and 14.4, 200^2 p = 5 29.8 and 31.3, jittered 32^3 hexes p = 3
+// 70.0 and 72.0; past kEarlyBlocks there is little to hide and the early blocks
+// cost more (64^3 hexes p = 3: 354 and 351).
+constexpr unsigned kEarlyBlocks = 152 * 160;
+template <typename K>
+inline void launch_pdl(K kern, unsigned grid, int threads, size_t smem, const KArgs& A, cudaStream_t s) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = grid <= kEarlyBlocks ? 1 : 0;
+  cudaLaunchKernelEx(&c, kern, A);
+}
 
 template <typename K>
 inline void launch_kernel(K kern, size_t smem, int et, const KArgs& A, cudaStream_t s, int threads = kThreads) {

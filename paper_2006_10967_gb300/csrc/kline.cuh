@@ -197,6 +197,16 @@ __device__ __forceinline__ void tile_fetch(float* dst, const void* src, int ne, 
     for (int i = lane; i < ne * PER / 4; i += 32) cp_async_4(d + 4 * i, s + 4 * i);
   }
 }
+// Programmatic dependent launch: a kernel's blocks start while the kernel before
+// it drains, and read what that kernel wrote only after pdl_wait (its
+// completion).  pdl_launch follows pdl_wait in every kernel, so that when a
+// kernel's blocks run, all kernels but the one before it are complete: before
+// pdl_wait they read connectivity, metric, weights and velocity data (written
+// at set-up) and, in the update kernels, the solution, accumulator and flux
+// balances (written by the update before; between them the residual kernel
+// writes only rp and fc).  Every kernel waits before it returns.
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int LEFT>
 __device__ __forceinline__ void cp_async_wait_but() {
@@ -375,7 +385,7 @@ struct KBLine {
 
 // NPHI: the interface normal comes from phi (the unpreconditioned method).
 template <int DIM, int N, bool GEN, bool TAB, bool NPHI, int WPB>
-__global__ void __launch_bounds__(WPB * 32, (GEN ? 16 : 20) / WPB) kb_line(const KArgs A) {
+__global__ void __launch_bounds__(WPB * 32, (GEN || (DIM == 3 && N == 5) ? 16 : 20) / WPB) kb_line(const KArgs A) {
   using L = LL<DIM, N>;
   using K = KBLine<DIM, N, GEN, TAB>;
   constexpr int NU = L::NU, NF = L::NF, NFP = L::NFP, LN = L::LN, EPW = L::EPW, NP = L::NP, AS = L::AS;
@@ -394,68 +404,24 @@ __global__ void __launch_bounds__(WPB * 32, (GEN ? 16 : 20) / WPB) kb_line(const
   const LineOps& O = A.lo;
   const PrmT<float>& P = A.cf.prm;
 
-  // ---- loads: the line's state, connectivity, partner traces
-  float2 u[2][NP];
-  if constexpr (L::DIRECT) {
-#pragma unroll
-    for (int f = 0; f < 2; ++f)
-      grow_get<N>(reinterpret_cast<const float*>(A.ustg) + (e * 2 + f) * NU + l * N, u[f]);
-  } else {
-    float* in = wsm + K::O_IN;
-    const int ne = (int)max((int64_t)0, min((int64_t)EPW, A.E - e0));
-    tile_fetch<EPW, 2 * NU * 4>(in, reinterpret_cast<const float*>(A.ustg) + e0 * 2 * NU, ne, lane);
-    cp_async_commit();
-  }
+  // ---- loads that no kernel of the march writes: connectivity, mid-tile data, metric
+  const int ne = (int)max((int64_t)0, min((int64_t)EPW, A.E - e0));
   int fl[DIM][2];
-  float2 o[DIM][2];
-  [[maybe_unused]] int32_t w2[DIM][2];
-  if constexpr (DIM == 3) {
-    int2 fw[DIM][2];
+  [[maybe_unused]] int2 fw[DIM][2];     // hexes: face words
+  [[maybe_unused]] int32_t w2[DIM][2];  // quads: connectivity words
 #pragma unroll
-    for (int a = 0; a < DIM; ++a)
+  for (int a = 0; a < DIM; ++a)
 #pragma unroll
-      for (int sd = 0; sd < 2; ++sd) fw[a][sd] = __ldg(A.ffw + e * 6 + 2 * a + sd);
-    const int fi = l % N, fj = l / N;
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      float t[2][2];
-#pragma unroll
-      for (int sd = 0; sd < 2; ++sd) {
-        const int32_t po = face_link<N, NF>(A, fw[a][sd], e, 2 * a + sd, fi, fj, fl[a][sd]);
-        const bool nb = (fl[a][sd] & (kFwL | kFwWall)) == kFwL;
-        t[0][sd] = nb ? trA[po] : 0.f;
-        t[1][sd] = nb ? trA[po + NF] : 0.f;
-      }
-      o[a][0] = make_float2(t[0][0], t[0][1]);
-      o[a][1] = make_float2(t[1][0], t[1][1]);
+    for (int s = 0; s < 2; ++s) {
+      if constexpr (DIM == 3) fw[a][s] = __ldg(A.ffw + e * 6 + 2 * a + s);
+      else w2[a][s] = __ldg(A.fnbr + e * NF + (2 * a + s) * NFP + l);
     }
-  } else {
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      float t[2][2];
-#pragma unroll
-      for (int sd = 0; sd < 2; ++sd) {
-        const int k = (2 * a + sd) * NFP + l;
-        const int32_t og = (int32_t)(e * NF + k);
-        w2[a][sd] = A.fnbr[og];
-        t[0][sd] = trA[e * 2 * NF + k];
-        t[1][sd] = trA[e * 2 * NF + NF + k];
-        fl[a][sd] = (w2[a][sd] & 1) | ((w2[a][sd] >> 1) == og ? kFwWall : 0);
-      }
-      o[a][0] = make_float2(t[0][0], t[0][1]);
-      o[a][1] = make_float2(t[1][0], t[1][1]);
-    }
+  if (GEN ? A.vtab != nullptr : TAB) tile_fetch<EPW, DIM * NT * 8>(wsm + K::O_TAB, A.vtab + e0 * DIM * NT, ne, lane);
+  if constexpr (K::PTS) {
+    tile_fetch<EPW, DIM * NF * 4>(wsm + K::O_VF, reinterpret_cast<const float*>(A.vsf) + e0 * DIM * NF, ne, lane);
+    tile_fetch<EPW, DIM * NU * 4>(wsm + K::O_VU, reinterpret_cast<const float*>(A.vsu) + e0 * DIM * NU, ne, lane);
   }
-  {
-    const int ne = (int)max((int64_t)0, min((int64_t)EPW, A.E - e0));
-    if (GEN ? A.vtab != nullptr : TAB) tile_fetch<EPW, DIM * NT * 8>(wsm + K::O_TAB, A.vtab + e0 * DIM * NT, ne, lane);
-    if constexpr (K::PTS) {
-      tile_fetch<EPW, DIM * NF * 4>(wsm + K::O_VF, reinterpret_cast<const float*>(A.vsf) + e0 * DIM * NF, ne, lane);
-      tile_fetch<EPW, DIM * NU * 4>(wsm + K::O_VU, reinterpret_cast<const float*>(A.vsu) + e0 * DIM * NU, ne, lane);
-    }
-    if constexpr (GEN) tile_fetch<EPW, L::S::NG * 4>(wsm + K::O_GEO, A.geof + e0 * L::S::NG, ne, lane);
-    cp_async_commit();
-  }
+  if constexpr (GEN) tile_fetch<EPW, L::S::NG * 4>(wsm + K::O_GEO, A.geof + e0 * L::S::NG, ne, lane);
   const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
   const bool diag = !GEN || __ldg(mc + 11) == 2.f;
   const bool tab = GEN ? diag && A.vtab != nullptr : TAB;
@@ -463,6 +429,39 @@ __global__ void __launch_bounds__(WPB * 32, (GEN ? 16 : 20) / WPB) kb_line(const
 #pragma unroll
   for (int a = 0; a < DIM; ++a) sd[a] = __ldg(mc + a * 4);
   const float rdet = __ldg(mc + 10);
+  pdl_wait();
+  pdl_launch();
+  // ---- the line's state and the partner traces
+  float2 u[2][NP];
+  float2 o[DIM][2];
+  if constexpr (L::DIRECT) {
+#pragma unroll
+    for (int f = 0; f < 2; ++f)
+      grow_get<N>(reinterpret_cast<const float*>(A.ustg) + (e * 2 + f) * NU + l * N, u[f]);
+  } else {
+    tile_fetch<EPW, 2 * NU * 4>(wsm + K::O_IN, reinterpret_cast<const float*>(A.ustg) + e0 * 2 * NU, ne, lane);
+    cp_async_commit();
+  }
+#pragma unroll
+  for (int a = 0; a < DIM; ++a) {
+    float t[2][2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const int k = (2 * a + s) * NFP + l;
+      if constexpr (DIM == 3) {
+        const int32_t po = face_link<N, NF>(A, fw[a][s], e, 2 * a + s, l % N, l / N, fl[a][s]);
+        const bool nb = (fl[a][s] & (kFwL | kFwWall)) == kFwL;
+        t[0][s] = nb ? trA[po] : 0.f;
+        t[1][s] = nb ? trA[po + NF] : 0.f;
+      } else {
+        t[0][s] = trA[e * 2 * NF + k];
+        t[1][s] = trA[e * 2 * NF + NF + k];
+        fl[a][s] = (w2[a][s] & 1) | ((w2[a][s] >> 1) == (int32_t)(e * NF + k) ? kFwWall : 0);
+      }
+    }
+    o[a][0] = make_float2(t[0][0], t[0][1]);
+    o[a][1] = make_float2(t[1][0], t[1][1]);
+  }
 
   // time factor and eps (of the element in a batch), evaluated by every warp for
   // itself: three FP64 instructions a warp cost less than a block barrier
@@ -476,7 +475,7 @@ __global__ void __launch_bounds__(WPB * 32, (GEN ? 16 : 20) / WPB) kb_line(const
     eps = P.eps;
   }
   if constexpr (!L::DIRECT) {
-    cp_async_wait_but<1>();  // the state; the rest follows before the faces
+    cp_async_wait_all();
     __syncwarp();
     const float* in = wsm + K::O_IN;
 #pragma unroll
@@ -541,7 +540,7 @@ __global__ void __launch_bounds__(WPB * 32, (GEN ? 16 : 20) / WPB) kb_line(const
   // the other fields' faces need the axis-0 component of the field that gives the normal
   constexpr int kn = NPHI ? 0 : 1;
   if (lane_ok && diag) row_put<NP, L::V4>(Q + (kn * DIM) * FA + pline<DIM, N>(0, l), q[kn][0]);
-  cp_async_wait_all();
+  if constexpr (L::DIRECT) cp_async_wait_all();  // the mid-tile data
   __syncwarp();
 #pragma unroll
   for (int f = 0; f < 2; ++f)
@@ -870,7 +869,6 @@ __global__ void __launch_bounds__(WPB * 32, (GEN ? 16 : 20) / WPB) kb_line(const
   }
   if constexpr (!L::DIRECT) {
     __syncwarp();
-    const int ne = (int)min((int64_t)EPW, A.E - e0);
     if (ne > 0) warp_flush(rp + e0 * 2 * NU, wsm + K::O_IN, ne * 2 * NU, lane);
   }
 }
@@ -989,104 +987,88 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
   float2 y[2][NP];       // partial divergence, then the stage value
   float2 u[2][N];        // solution pairs (hi, lo)
   float ac[2][N];        // RK accumulator
-  if constexpr (L::DIRECT) {
-    const float* src = SF == 0 ? ustg : reinterpret_cast<const float*>(A.rp);
+  float aff = 1.f, rdet = 0.f;  // record: affine flag, 1 / det J
+  [[maybe_unused]] RKConstF rk;
+  double ta = 0.0;  // this thread's element balance so far (finished by the first threads of the block)
+  const int64_t gt = (int64_t)blockIdx.x * NEL * 2 + threadIdx.x;
+  float2 rW = make_float2(0.f, 0.f);  // stage 4: 1 / W
+  if constexpr (SF >= 1) {
+    const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
+    rdet = __ldg(mc + 10);
+    if (GEN) aff = DIM == 3 ? __ldg(mc + 11) : 0.f;
+    if constexpr (L::DIRECT) {
 #pragma unroll
-    for (int f = 0; f < 2; ++f) {
-      const int64_t r = (e * 2 + f) * NU + l * N;
-      grow_get<N>(src + r, y[f]);
-      if constexpr (SF >= 1) {
+      for (int f = 0; f < 2; ++f) {
+        const int64_t r = (e * 2 + f) * NU + l * N;
 #pragma unroll
         for (int j = 0; j < N; j += 2) {
           const float4 t = *reinterpret_cast<const float4*>(U + r + j);
           u[f][j] = make_float2(t.x, t.y);
           u[f][j + 1] = make_float2(t.z, t.w);
         }
+        if constexpr (SF >= 2) {
+          float2 t[NP];
+          grow_get<N>(acc + r, t);
+          unpair<N>(t, ac[f]);
+        }
       }
-      if constexpr (SF >= 2) {
-        float2 t[NP];
-        grow_get<N>(acc + r, t);
-        unpair<N>(t, ac[f]);
-      }
+    } else if (ne > 0) {
+      tile_fetch<EPW, 2 * NU * 8>(in + K::O_U, U + e0 * 2 * NU, ne, lane);
+      if constexpr (SF >= 2) tile_fetch<EPW, 2 * NU * 4>(in + K::O_A, acc + e0 * 2 * NU, ne, lane);
     }
-  } else if (ne > 0) {
-    const float* src = SF == 0 ? ustg : reinterpret_cast<const float*>(A.rp);
-    tile_fetch<EPW, 2 * NU * 4>(in, src + e0 * 2 * NU, ne, lane);
-    if constexpr (SF >= 1) tile_fetch<EPW, 2 * NU * 8>(in + K::O_U, U + e0 * 2 * NU, ne, lane);
-    if constexpr (SF >= 2) tile_fetch<EPW, 2 * NU * 4>(in + K::O_A, acc + e0 * 2 * NU, ne, lane);
-    cp_async_commit();
-  }
-  if constexpr (SF >= 1) {
     if (SF == 4 && cons && ne > 0) tile_fetch<EPW, NU * 8>(wsm + K::O_W, A.wdetf + e0 * NU, ne, lane);
     if (GEN && ne > 0) tile_fetch<EPW, L::S::NG * 4>(wsm + K::O_GEO, A.geof + e0 * L::S::NG, ne, lane);
-    cp_async_commit();
-  }
-  float aff = 1.f, rdet = 0.f;  // record: affine flag, 1 / det J
-  if constexpr (SF >= 1) {
-    const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
-    rdet = __ldg(mc + 10);
-    if (GEN) aff = DIM == 3 ? __ldg(mc + 11) : 0.f;
+    rk = A.ep ? A.ep[e].rk : A.rk;
+    if (SF >= 2 && cons && threadIdx.x < 2 * NEL && gt < 2 * A.E) {
+      ta = A.tacc[gt];
+      if (SF == 4) rW = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(A.mcg) + (gt / 2) * kMetricRec + 12);
+    }
   }
   int fl[DIM][2];
+  [[maybe_unused]] int2 fw[DIM][2];
   [[maybe_unused]] int32_t w2[DIM][2];
+#pragma unroll
+  for (int a = 0; a < DIM; ++a)
+#pragma unroll
+    for (int sd = 0; sd < 2; ++sd) {
+      if constexpr (DIM == 3) fw[a][sd] = __ldg(A.ffw + e * 6 + 2 * a + sd);
+      else w2[a][sd] = __ldg(A.fnbr + e * NF + (2 * a + sd) * NFP + l);
+    }
+  pdl_wait();
+  pdl_launch();
+  {
+    const float* src = SF == 0 ? ustg : reinterpret_cast<const float*>(A.rp);
+    if constexpr (L::DIRECT) {
+#pragma unroll
+      for (int f = 0; f < 2; ++f) grow_get<N>(src + (e * 2 + f) * NU + l * N, y[f]);
+    } else if (ne > 0) {
+      tile_fetch<EPW, 2 * NU * 4>(in, src + e0 * 2 * NU, ne, lane);
+    }
+  }
   float2 F[DIM][2];  // transformed common flux at the two ends: the own at L ends, the partner's at R ends
-  if constexpr (DIM == 3) {
-    int2 fw[DIM][2];
 #pragma unroll
-    for (int a = 0; a < DIM; ++a)
+  for (int a = 0; a < DIM; ++a) {
+    float t[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
-      for (int sd = 0; sd < 2; ++sd) fw[a][sd] = __ldg(A.ffw + e * 6 + 2 * a + sd);
-    const int fi = l % N, fj = l / N;
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      float t[2][2];
-#pragma unroll
-      for (int sd = 0; sd < 2; ++sd) {
-        const int32_t po = face_link<N, NF>(A, fw[a][sd], e, 2 * a + sd, fi, fj, fl[a][sd]);
-        if constexpr (SF >= 1) {
-          const int32_t own = (int32_t)(e * 2 * NF + (2 * a + sd) * NFP + l);
-          const int32_t s = (fl[a][sd] & kFwL) ? own : po;
-          t[0][sd] = fcA[s];
-          t[1][sd] = fcA[s + NF];
-        }
+    for (int sd = 0; sd < 2; ++sd) {
+      const int k = (2 * a + sd) * NFP + l;
+      int32_t at = (int32_t)(e * 2 * NF + k);
+      if constexpr (DIM == 3) {
+        const int32_t po = face_link<N, NF>(A, fw[a][sd], e, 2 * a + sd, l % N, l / N, fl[a][sd]);
+        if (!(fl[a][sd] & kFwL)) at = po;
+      } else {
+        fl[a][sd] = (w2[a][sd] & 1) | ((w2[a][sd] >> 1) == (int32_t)(e * NF + k) ? kFwWall : 0);
       }
       if constexpr (SF >= 1) {
-        F[a][0] = make_float2(t[0][0], t[0][1]);
-        F[a][1] = make_float2(t[1][0], t[1][1]);
+        t[0][sd] = fcA[at];
+        t[1][sd] = fcA[at + NF];
       }
     }
-  } else {
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      float t[2][2];
-#pragma unroll
-      for (int sd = 0; sd < 2; ++sd) {
-        const int k = (2 * a + sd) * NFP + l;
-        const int32_t og = (int32_t)(e * NF + k);
-        w2[a][sd] = A.fnbr[og];
-        fl[a][sd] = (w2[a][sd] & 1) | ((w2[a][sd] >> 1) == og ? kFwWall : 0);
-        if constexpr (SF >= 1) {
-          t[0][sd] = fcA[e * 2 * NF + k];
-          t[1][sd] = fcA[e * 2 * NF + NF + k];
-        }
-      }
-      if constexpr (SF >= 1) {
-        F[a][0] = make_float2(t[0][0], t[0][1]);
-        F[a][1] = make_float2(t[1][0], t[1][1]);
-      }
-    }
+    F[a][0] = make_float2(t[0][0], t[0][1]);
+    F[a][1] = make_float2(t[1][0], t[1][1]);
   }
-  double ta = 0.0;  // this thread's element balance so far (finished by the first threads of the block)
-  const int64_t gt = (int64_t)blockIdx.x * NEL * 2 + threadIdx.x;
-  float2 rW = make_float2(0.f, 0.f);  // stage 4: 1 / W
-  if (SF >= 2 && cons && threadIdx.x < 2 * NEL && gt < 2 * A.E) {
-    ta = A.tacc[gt];
-    if (SF == 4) rW = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(A.mcg) + (gt / 2) * kMetricRec + 12);
-  }
-  [[maybe_unused]] RKConstF rk;
-  if constexpr (SF >= 1) rk = A.ep ? A.ep[e].rk : A.rk;
   if constexpr (!L::DIRECT) {
-    cp_async_wait_but<(SF >= 1)>();
+    cp_async_wait_all();
     __syncwarp();
 #pragma unroll
     for (int f = 0; f < 2; ++f) {

@@ -97,7 +97,6 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
   using L = LL<DIM, N>;
   using K = KBPLine<DIM, N, GEN>;
   constexpr int NU = L::NU, NF = L::NF, NFP = L::NFP, LN = L::LN, EPW = L::EPW, NP = L::NP, AS = L::AS;
-  if (*(volatile int32_t*)&A.status[ST_PSEUDO_DONE]) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float* wsm = reinterpret_cast<float*>(smem_raw) + warp * K::F;
@@ -114,57 +113,28 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
   const PrmT<float>& P = A.cf.prm;
 
   // ---- loads
-  float2 u[NP];
-  const float* ug = reinterpret_cast<const float*>(A.ustg);
-  if constexpr (L::DIRECT) grow_get<N>(ug + (e * 2 + 1) * NU + l * N, u);
-  else rows_fetch<NU>(in, ug + (e0 * 2 + 1) * NU, 2 * NU, ne, lane);
-  cp_async_commit();
   if (GEN && ne > 0) tile_fetch<EPW, L::S::NG * 4>(wsm + K::O_GEO, A.geof + e0 * L::S::NG, ne, lane);
   int fl[DIM][2];
-  float2 o[DIM];
+  [[maybe_unused]] int2 fw[DIM][2];
   [[maybe_unused]] int32_t w2[DIM][2];
-  if constexpr (DIM == 3) {
-    int2 fw[DIM][2];
 #pragma unroll
-    for (int a = 0; a < DIM; ++a)
+  for (int a = 0; a < DIM; ++a)
 #pragma unroll
-      for (int sd = 0; sd < 2; ++sd) fw[a][sd] = __ldg(A.ffw + e * 6 + 2 * a + sd);
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      float t[2];
-#pragma unroll
-      for (int sd = 0; sd < 2; ++sd) {
-        const int32_t po = face_link<N, NF>(A, fw[a][sd], e, 2 * a + sd, l % N, l / N, fl[a][sd]);
-        t[sd] = (fl[a][sd] & (kFwL | kFwWall)) == kFwL ? trA[po + NF] : 0.f;
-      }
-      o[a] = make_float2(t[0], t[1]);
+    for (int s = 0; s < 2; ++s) {
+      if constexpr (DIM == 3) fw[a][s] = __ldg(A.ffw + e * 6 + 2 * a + s);
+      else w2[a][s] = __ldg(A.fnbr + e * NF + (2 * a + s) * NFP + l);
     }
-  } else {
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      float t[2];
-#pragma unroll
-      for (int sd = 0; sd < 2; ++sd) {
-        const int k = (2 * a + sd) * NFP + l;
-        const int32_t og = (int32_t)(e * NF + k);
-        w2[a][sd] = A.fnbr[og];
-        t[sd] = trA[e * 2 * NF + NF + k];
-        fl[a][sd] = (w2[a][sd] & 1) | ((w2[a][sd] >> 1) == og ? kFwWall : 0);
-      }
-      o[a] = make_float2(t[0], t[1]);
-    }
-  }
   float p0[N];
   if constexpr (N % 2 == 0) {
 #pragma unroll
     for (int j = 0; j < N; j += 2) {
-      const double2 t = __ldg(reinterpret_cast<const double2*>(A.psi0 + e * NU + l * N + j));
+      const double2 t = *reinterpret_cast<const double2*>(A.psi0 + e * NU + l * N + j);
       p0[j] = (float)t.x;
       p0[j + 1] = (float)t.y;
     }
   } else {
 #pragma unroll
-    for (int j = 0; j < N; ++j) p0[j] = (float)__ldg(A.psi0 + e * NU + l * N + j);
+    for (int j = 0; j < N; ++j) p0[j] = (float)A.psi0[e * NU + l * N + j];
   }
   const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
   const bool diag = !GEN || __ldg(mc + 11) == 2.f;
@@ -172,8 +142,29 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
 #pragma unroll
   for (int a = 0; a < DIM; ++a) sd[a] = __ldg(mc + a * 4);
   const float det = __ldg(mc + 9), rdet = __ldg(mc + 10);
+  if (*(volatile int32_t*)&A.status[ST_PSEUDO_DONE]) return;
+  float2 u[NP], o[DIM];
+  const float* ug = reinterpret_cast<const float*>(A.ustg);
+  if constexpr (L::DIRECT) grow_get<N>(ug + (e * 2 + 1) * NU + l * N, u);
+  else rows_fetch<NU>(in, ug + (e0 * 2 + 1) * NU, 2 * NU, ne, lane);
+#pragma unroll
+  for (int a = 0; a < DIM; ++a) {
+    float t[2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const int k = (2 * a + s) * NFP + l;
+      if constexpr (DIM == 3) {
+        const int32_t po = face_link<N, NF>(A, fw[a][s], e, 2 * a + s, l % N, l / N, fl[a][s]);
+        t[s] = (fl[a][s] & (kFwL | kFwWall)) == kFwL ? trA[po + NF] : 0.f;
+      } else {
+        t[s] = trA[e * 2 * NF + NF + k];
+        fl[a][s] = (w2[a][s] & 1) | ((w2[a][s] >> 1) == (int32_t)(e * NF + k) ? kFwWall : 0);
+      }
+    }
+    o[a] = make_float2(t[0], t[1]);
+  }
   if constexpr (!L::DIRECT) {
-    cp_async_wait_but<0>();
+    cp_async_wait_all();
     __syncwarp();
     grow_get<N>(in + es * NU + l * N, u);
   }

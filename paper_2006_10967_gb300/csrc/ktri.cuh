@@ -77,7 +77,9 @@ __device__ __forceinline__ void tri_metric(const T* g, TriMet<T>& m) {
 
 // TC: the float path's operator applies on tensor cores (mma_tf32.cuh);
 // otherwise scalar dot products (the only form of the FP64 path).
-template <int P, typename T, int MODE, bool TC = false>
+// TD: tile divisor; FP64 fields on small meshes take quarter tiles, so that
+// their few blocks spread over the SMs (see fill_tri).
+template <int P, typename T, int MODE, bool TC = false, int TD = 1>
 struct KBTriLayout {
   using S = TriS<P>;
   static constexpr int NFLD = MODE == 0 ? 2 : 1;
@@ -87,14 +89,15 @@ struct KBTriLayout {
                                   (MMA ? NFLD * 2 * S::NF : 0);
   static constexpr int BYTES_EL = PER_EL_T * (int)sizeof(T) + S::NF;
   static constexpr int ETr = 32768 / BYTES_EL;
-  static constexpr int ET = ETr < 1 ? 1 : (ETr > 64 ? 64 : ETr);
+  static constexpr int ET1 = ETr < 1 ? 1 : (ETr > 64 ? 64 : ETr);
+  static constexpr int ET = ET1 / TD < 1 ? 1 : ET1 / TD;
   static constexpr size_t SMEM = (size_t)ET * BYTES_EL + sizeof(TriOpsS<P, T>) + 64;
 };
 
-template <int P, typename T, int MODE, bool TC = false>
+template <int P, typename T, int MODE, bool TC = false, int TD = 1>
 __global__ void __launch_bounds__(kThreads) kb_tri(const KArgs A) {
   using S = TriS<P>;
-  using LY = KBTriLayout<P, T, MODE, TC>;
+  using LY = KBTriLayout<P, T, MODE, TC, TD>;
   constexpr int NU = S::NU, NF = S::NF, NG = S::NG, NFLD = LY::NFLD, ET = LY::ET, N = S::N;
   constexpr int F0 = MODE == 0 ? 0 : 1;
   constexpr bool kMMA = LY::MMA;
@@ -440,7 +443,7 @@ __global__ void __launch_bounds__(kThreads) kb_tri(const KArgs A) {
   (void)N;
 }
 
-template <int P, typename T, int MODE, bool TC = false>
+template <int P, typename T, int MODE, bool TC = false, int TD = 1>
 struct KATriLayout {
   using S = TriS<P>;
   static constexpr int NFLD = MODE == 0 ? 2 : 1;
@@ -453,14 +456,15 @@ struct KATriLayout {
                                   (CONS ? 2 * S::NU * 8 : 0);
   static constexpr int HEAD_EL = (NFLD * S::NU + NFLD * S::NF + S::NG + 1 + (FLT ? NFLD * S::NU : 0));  // T values before u2s
   static constexpr int ETr = 16384 / BYTES_EL;
-  static constexpr int ET = ETr < 1 ? 1 : (ETr > 128 ? 128 : ETr);
+  static constexpr int ET1 = ETr < 1 ? 1 : (ETr > 128 ? 128 : ETr);
+  static constexpr int ET = ET1 / TD < 1 ? 1 : ET1 / TD;
   static constexpr size_t SMEM = (size_t)ET * BYTES_EL + sizeof(TriOpsS<P, T>) + 64 + 16;  // + u2s alignment
 };
 
-template <int P, typename T, int MODE, bool TC = false>
+template <int P, typename T, int MODE, bool TC = false, int TD = 1>
 __global__ void __launch_bounds__(kThreads) ka_tri(const KArgs A) {
   using S = TriS<P>;
-  using LY = KATriLayout<P, T, MODE, TC>;
+  using LY = KATriLayout<P, T, MODE, TC, TD>;
   constexpr int NU = S::NU, NF = S::NF, NG = S::NG, NFLD = LY::NFLD, ET = LY::ET;
   constexpr int F0 = MODE == 0 ? 0 : 1;
   if (MODE == 1 && *(volatile int32_t*)&A.status[ST_PSEUDO_DONE]) return;
