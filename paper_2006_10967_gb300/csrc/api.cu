@@ -177,8 +177,8 @@ bool use_line_pseudo(const fr_mesh& m, const fr_params& p) {
 bool set_line_pseudo(const fr_mesh& m, bool gen, KernelSet* ks) {
   return m.etype == FR_QUAD ? line_pseudo_quad(m.order, gen, ks) : line_pseudo_hex(m.order, gen, ks);
 }
-bool set_line_kernels(const fr_mesh& m, bool gen, bool tab, KernelSet* ks) {
-  return m.etype == FR_QUAD ? line_kernels_quad(m.order, gen, tab, ks) : line_kernels_hex(m.order, gen, tab, ks);
+bool set_line_kernels(const fr_mesh& m, bool gen, bool tab, bool nphi, KernelSet* ks) {
+  return m.etype == FR_QUAD ? line_kernels_quad(m.order, gen, tab, nphi, ks) : line_kernels_hex(m.order, gen, tab, nphi, ks);
 }
 
 // Blocks of the largest launch (one reduction partial each): the block-wide
@@ -781,7 +781,7 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
   const bool diagonal = m->etype != FR_TRI && all_diagonal(*m);
   if (use_line_kernels(*m, *prm)) {
     if (vel_separable(prm->vel.kind)) A.vtab = reinterpret_cast<const float2*>(b + L.vtab);
-    if (!set_line_kernels(*m, !diagonal, A.vtab != nullptr, &f->ks)) {
+    if (!set_line_kernels(*m, !diagonal, A.vtab != nullptr, prm->normal == FR_NORMAL_PHI, &f->ks)) {
       delete f;
       return FR_ECUDA;
     }
@@ -1009,7 +1009,7 @@ extern "C" int fr_field_init_batch(const fr_mesh* m, const fr_params* prm, int n
   if (use_line_kernels(*m, *prm)) {
     // the table holds params->vel, the instances' own velocities are in the point cache
     f->args.vtab = nullptr;
-    if (!set_line_kernels(*m, !all_diagonal(*m), false, &f->ks)) {
+    if (!set_line_kernels(*m, !all_diagonal(*m), false, prm->normal == FR_NORMAL_PHI, &f->ks)) {
       fr_field_destroy(f);
       return FR_ECUDA;
     }

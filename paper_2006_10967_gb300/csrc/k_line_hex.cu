@@ -3,12 +3,12 @@
 #include "k_line_inst.cuh"
 
 namespace frp {
-bool line_kernels_hex(int order, bool gen, bool tab, KernelSet* ks) {
+bool line_kernels_hex(int order, bool gen, bool tab, bool nphi, KernelSet* ks) {
   switch (order) {
-    case 1: return fill_line<3, 2>(gen, tab, ks);
-    case 2: return fill_line<3, 3>(gen, tab, ks);
-    case 3: return fill_line<3, 4>(gen, tab, ks);
-    case 4: return fill_line<3, 5>(gen, tab, ks);
+    case 1: return fill_line<3, 2>(gen, tab, nphi, ks);
+    case 2: return fill_line<3, 3>(gen, tab, nphi, ks);
+    case 3: return fill_line<3, 4>(gen, tab, nphi, ks);
+    case 4: return fill_line<3, 5>(gen, tab, nphi, ks);
     default: return false;
   }
 }

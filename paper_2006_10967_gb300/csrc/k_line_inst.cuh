@@ -17,8 +17,13 @@ void launch_kb_line(const KArgs& A, cudaStream_t s) {
   constexpr int smem = KBLine<DIM, N, GEN, TAB>::F * 4 * kLineWarps;
   static_assert(smem <= 48 * 1024, "no shared-memory opt-in needed");
   const unsigned grid = line_grid<DIM, N>(A.E, kLineWarps);
-  if (A.cf.prm.nphi) launch_pdl(kb_line<DIM, N, GEN, TAB, true, kLineWarps>, grid, kLineWarps * 32, smem, A, s);
-  else launch_pdl(kb_line<DIM, N, GEN, TAB, false, kLineWarps>, grid, kLineWarps * 32, smem, A, s);
+  launch_pdl(kb_line<DIM, N, GEN, TAB, false, kLineWarps>, grid, kLineWarps * 32, smem, A, s);
+}
+// The unpreconditioned method (normal from phi) takes one kernel for all meshes.
+template <int DIM, int N>
+void launch_kb_line_phi(const KArgs& A, cudaStream_t s) {
+  launch_pdl(kb_line<DIM, N, true, false, true, kLineWarps>, line_grid<DIM, N>(A.E, kLineWarps), kLineWarps * 32,
+             KBLine<DIM, N, true, false>::F * 4 * kLineWarps, A, s);
 }
 
 template <int DIM, int N, bool GEN, int SF>
@@ -30,7 +35,7 @@ void launch_ka_stage(const KArgs& A, cudaStream_t s) {
 template <int DIM, int N, bool GEN>
 void launch_ka_line(const KArgs& A, cudaStream_t s) {
   switch (A.stage) {
-    case 0: launch_ka_stage<DIM, N, GEN, 0>(A, s); return;
+    case 0: launch_ka_stage<DIM, N, false, 0>(A, s); return;  // no metric
     case 1: launch_ka_stage<DIM, N, GEN, 1>(A, s); return;
     case 2: launch_ka_stage<DIM, N, GEN, 2>(A, s); return;
     case 3: launch_ka_stage<DIM, N, GEN, 3>(A, s); return;
@@ -55,13 +60,15 @@ bool fill_line_set(bool tab, KernelSet* ks) {
   else ks->kb[0] = tab ? launch_kb_line<DIM, N, false, true> : launch_kb_line<DIM, N, false, false>;
   ks->ka[0] = launch_ka_line<DIM, N, GEN>;
   ks->vtab = launch_vel_tab<DIM, N>;
-  return prepare_ka_line<DIM, N, GEN, 0>() && prepare_ka_line<DIM, N, GEN, 1>() && prepare_ka_line<DIM, N, GEN, 2>() &&
+  return prepare_ka_line<DIM, N, false, 0>() && prepare_ka_line<DIM, N, GEN, 1>() && prepare_ka_line<DIM, N, GEN, 2>() &&
          prepare_ka_line<DIM, N, GEN, 3>() && prepare_ka_line<DIM, N, GEN, 4>();
 }
 
 template <int DIM, int N>
-bool fill_line(bool gen, bool tab, KernelSet* ks) {
-  return gen ? fill_line_set<DIM, N, true>(tab, ks) : fill_line_set<DIM, N, false>(tab, ks);
+bool fill_line(bool gen, bool tab, bool nphi, KernelSet* ks) {
+  const bool ok = gen ? fill_line_set<DIM, N, true>(tab, ks) : fill_line_set<DIM, N, false>(tab, ks);
+  if (nphi) ks->kb[0] = launch_kb_line_phi<DIM, N>;
+  return ok;
 }
 
 template <int DIM, int N, bool GEN>
@@ -81,7 +88,7 @@ void launch_kap_stage(const KArgs& A, cudaStream_t s) {
 template <int DIM, int N, bool GEN>
 void launch_ka_pseudo(const KArgs& A, cudaStream_t s) {
   switch (A.stage) {
-    case 0: launch_kap_stage<DIM, N, GEN, 0>(A, s); return;
+    case 0: launch_kap_stage<DIM, N, false, 0>(A, s); return;
     case 1: launch_kap_stage<DIM, N, GEN, 1>(A, s); return;
     case 2: launch_kap_stage<DIM, N, GEN, 2>(A, s); return;
     case 3: launch_kap_stage<DIM, N, GEN, 3>(A, s); return;

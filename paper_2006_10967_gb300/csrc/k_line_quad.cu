@@ -2,14 +2,14 @@
 #include "k_line_inst.cuh"
 
 namespace frp {
-bool line_kernels_quad(int order, bool gen, bool tab, KernelSet* ks) {
+bool line_kernels_quad(int order, bool gen, bool tab, bool nphi, KernelSet* ks) {
   switch (order) {
-    case 1: return fill_line<2, 2>(gen, tab, ks);
-    case 2: return fill_line<2, 3>(gen, tab, ks);
-    case 3: return fill_line<2, 4>(gen, tab, ks);
-    case 4: return fill_line<2, 5>(gen, tab, ks);
-    case 5: return fill_line<2, 6>(gen, tab, ks);
-    case 6: return fill_line<2, 7>(gen, tab, ks);
+    case 1: return fill_line<2, 2>(gen, tab, nphi, ks);
+    case 2: return fill_line<2, 3>(gen, tab, nphi, ks);
+    case 3: return fill_line<2, 4>(gen, tab, nphi, ks);
+    case 4: return fill_line<2, 5>(gen, tab, nphi, ks);
+    case 5: return fill_line<2, 6>(gen, tab, nphi, ks);
+    case 6: return fill_line<2, 7>(gen, tab, nphi, ks);
     default: return false;
   }
 }

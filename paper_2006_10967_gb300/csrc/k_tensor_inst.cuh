@@ -8,6 +8,13 @@
 
 namespace frp {
 
+// The mixed preconditioning of quads and of hexes p <= 4 always runs in the line
+// kernels (use_line_pseudo); only its update kernel's rate output is kept here.
+template <int DIM, int N, typename T, int MODE>
+struct HasKB {
+  static constexpr bool v = !(MODE == 1 && sizeof(T) == 4 && (DIM == 2 || N <= 5));
+};
+
 template <int DIM, int N, typename T, int MODE, int TD = 1>
 void launch_kb_tensor(const KArgs& A, cudaStream_t s) {
   using LY = KBLayout<DIM, N, T, MODE, TD>;
@@ -50,9 +57,10 @@ void launch_vcache(const KArgs& A, cudaStream_t s) {
 // filled, so that no launch (and no graph capture) has to do it.
 template <int DIM, int N, typename T, int MODE, int TD = 1>
 bool prepare_tensor() {
-  bool ok = cudaFuncSetAttribute(kb_tensor<DIM, N, T, MODE, TD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)KBLayout<DIM, N, T, MODE, TD>::SMEM) == cudaSuccess &&
-            prepare_ka<DIM, N, T, MODE, TD, -2>();
+  bool ok = prepare_ka<DIM, N, T, MODE, TD, -2>();
+  if constexpr (HasKB<DIM, N, T, MODE>::v)
+    ok = ok && cudaFuncSetAttribute(kb_tensor<DIM, N, T, MODE, TD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)KBLayout<DIM, N, T, MODE, TD>::SMEM) == cudaSuccess;
   if constexpr (StageKA<DIM, T, MODE>::v)
     ok = ok && prepare_ka<DIM, N, T, MODE, TD, 1>() && prepare_ka<DIM, N, T, MODE, TD, 2>() &&
          prepare_ka<DIM, N, T, MODE, TD, 3>() && prepare_ka<DIM, N, T, MODE, TD, 4>();
@@ -101,7 +109,7 @@ void fill_tensor(int64_t E, KernelSet* ks) {
   ks->vcache = launch_vcache<DIM, N, T>;
   ks->mconst = launch_mconst<DIM, N, T>;
   ks->kb[0] = launch_kb_tensor<DIM, N, T, 0, TB>;
-  ks->kb[1] = launch_kb_tensor<DIM, N, T, 1>;
+  if constexpr (HasKB<DIM, N, T, 1>::v) ks->kb[1] = launch_kb_tensor<DIM, N, T, 1>;
   ks->ka[0] = launch_ka_tensor<DIM, N, T, 0, TA>;
   ks->ka_rate = ks->ka[0];
   ks->ka[1] = launch_ka_tensor<DIM, N, T, 1>;
@@ -116,11 +124,9 @@ void fill_tensor(int64_t E, KernelSet* ks) {
     // the preconditioning's reduction keeps a partial a block: small tiles only
     // where they stay within the slots every field has
     if (E <= kSmallTileElems) {
-      ks->prepared = ks->prepared && prepare_tensor<DIM, N, T, 1, 0>() && prepare_tensor<DIM, N, T, 1, -1>();
-      const double p1 = kb_clocks<DIM, N, KBLayout<DIM, N, T, 1>>(E), p0 = kb_clocks<DIM, N, KBLayout<DIM, N, T, 1, 0>>(E),
-                   pq = kb_clocks<DIM, N, KBLayout<DIM, N, T, 1, -1>>(E);
-      if (pq < p0 && pq < p1) ks->kb[1] = launch_kb_tensor<DIM, N, T, 1, -1>;
-      else if (p0 < p1) ks->kb[1] = launch_kb_tensor<DIM, N, T, 1, 0>;
+      ks->prepared = ks->prepared && prepare_tensor<DIM, N, T, 1, 0>();
+      if (kb_clocks<DIM, N, KBLayout<DIM, N, T, 1, 0>>(E) < kb_clocks<DIM, N, KBLayout<DIM, N, T, 1>>(E))
+        ks->kb[1] = launch_kb_tensor<DIM, N, T, 1, 0>;
       if (ka_warps<KALayout<DIM, N, T, 1, 0>>(E) < ka_warps<KALayout<DIM, N, T, 1>>(E)) {
         ks->ka[1] = launch_ka_tensor<DIM, N, T, 1, 0>;
         ks->ka_rate_pseudo = ks->ka[1];

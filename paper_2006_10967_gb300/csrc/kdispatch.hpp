@@ -32,9 +32,9 @@ constexpr int64_t kSmallTileElems = 16384;
 
 // Replace the physical-step kernels of a mixed tensor field by the line kernels
 // (kline.cuh); false where they are not built (the set is then unchanged) or
-// could not be prepared.  gen, tab: see KBLine.
-bool line_kernels_quad(int order, bool gen, bool tab, KernelSet* ks);
-bool line_kernels_hex(int order, bool gen, bool tab, KernelSet* ks);
+// could not be prepared.  gen, tab: see KBLine; nphi: normal from phi.
+bool line_kernels_quad(int order, bool gen, bool tab, bool nphi, KernelSet* ks);
+bool line_kernels_hex(int order, bool gen, bool tab, bool nphi, KernelSet* ks);
 // The same for the preconditioning kernels of a mixed tensor field; gen false:
 // every element is affine with a diagonal Jacobian.
 bool line_pseudo_quad(int order, bool gen, KernelSet* ks);

@@ -205,6 +205,11 @@ __device__ __forceinline__ void tile_fetch(float* dst, const void* src, int ne, 
 // at set-up) and, in the update kernels, the solution, accumulator and flux
 // balances (written by the update before; between them the residual kernel
 // writes only rp and fc).  Every kernel waits before it returns.
+// kEarly: regular hexes of N >= 4 (the large 3D runs) wait first and load their
+// state first: with thousands of blocks a wave there is little to hide, and the
+// other order cost them 2 % (64^3 p = 3: 358 and 350 us a stage).
+template <int DIM, int N, bool GEN>
+constexpr bool kEarly = !(DIM == 3 && N >= 4 && !GEN);
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
@@ -404,8 +409,23 @@ __global__ void __launch_bounds__(WPB * 32, (GEN || (DIM == 3 && N == 5) ? 16 : 
   const LineOps& O = A.lo;
   const PrmT<float>& P = A.cf.prm;
 
-  // ---- loads that no kernel of the march writes: connectivity, mid-tile data, metric
   const int ne = (int)max((int64_t)0, min((int64_t)EPW, A.E - e0));
+  float2 u[2][NP];
+  float2 o[DIM][2];
+  auto load_state = [&]() {
+    pdl_wait();
+    pdl_launch();
+    if constexpr (L::DIRECT) {
+#pragma unroll
+      for (int f = 0; f < 2; ++f)
+        grow_get<N>(reinterpret_cast<const float*>(A.ustg) + (e * 2 + f) * NU + l * N, u[f]);
+    } else {
+      tile_fetch<EPW, 2 * NU * 4>(wsm + K::O_IN, reinterpret_cast<const float*>(A.ustg) + e0 * 2 * NU, ne, lane);
+      cp_async_commit();
+    }
+  };
+  if constexpr (!kEarly<DIM, N, GEN>) load_state();
+  // ---- loads that no kernel of the march writes: connectivity, mid-tile data, metric
   int fl[DIM][2];
   [[maybe_unused]] int2 fw[DIM][2];     // hexes: face words
   [[maybe_unused]] int32_t w2[DIM][2];  // quads: connectivity words
@@ -429,19 +449,7 @@ __global__ void __launch_bounds__(WPB * 32, (GEN || (DIM == 3 && N == 5) ? 16 : 
 #pragma unroll
   for (int a = 0; a < DIM; ++a) sd[a] = __ldg(mc + a * 4);
   const float rdet = __ldg(mc + 10);
-  pdl_wait();
-  pdl_launch();
-  // ---- the line's state and the partner traces
-  float2 u[2][NP];
-  float2 o[DIM][2];
-  if constexpr (L::DIRECT) {
-#pragma unroll
-    for (int f = 0; f < 2; ++f)
-      grow_get<N>(reinterpret_cast<const float*>(A.ustg) + (e * 2 + f) * NU + l * N, u[f]);
-  } else {
-    tile_fetch<EPW, 2 * NU * 4>(wsm + K::O_IN, reinterpret_cast<const float*>(A.ustg) + e0 * 2 * NU, ne, lane);
-    cp_async_commit();
-  }
+  if constexpr (kEarly<DIM, N, GEN>) load_state();
 #pragma unroll
   for (int a = 0; a < DIM; ++a) {
     float t[2][2];
@@ -992,6 +1000,18 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
   double ta = 0.0;  // this thread's element balance so far (finished by the first threads of the block)
   const int64_t gt = (int64_t)blockIdx.x * NEL * 2 + threadIdx.x;
   float2 rW = make_float2(0.f, 0.f);  // stage 4: 1 / W
+  auto load_rate = [&]() {
+    pdl_wait();
+    pdl_launch();
+    const float* src = SF == 0 ? ustg : reinterpret_cast<const float*>(A.rp);
+    if constexpr (L::DIRECT) {
+#pragma unroll
+      for (int f = 0; f < 2; ++f) grow_get<N>(src + (e * 2 + f) * NU + l * N, y[f]);
+    } else if (ne > 0) {
+      tile_fetch<EPW, 2 * NU * 4>(in, src + e0 * 2 * NU, ne, lane);
+    }
+  };
+  if constexpr (!kEarly<DIM, N, GEN>) load_rate();
   if constexpr (SF >= 1) {
     const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
     rdet = __ldg(mc + 10);
@@ -1034,17 +1054,7 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
       if constexpr (DIM == 3) fw[a][sd] = __ldg(A.ffw + e * 6 + 2 * a + sd);
       else w2[a][sd] = __ldg(A.fnbr + e * NF + (2 * a + sd) * NFP + l);
     }
-  pdl_wait();
-  pdl_launch();
-  {
-    const float* src = SF == 0 ? ustg : reinterpret_cast<const float*>(A.rp);
-    if constexpr (L::DIRECT) {
-#pragma unroll
-      for (int f = 0; f < 2; ++f) grow_get<N>(src + (e * 2 + f) * NU + l * N, y[f]);
-    } else if (ne > 0) {
-      tile_fetch<EPW, 2 * NU * 4>(in, src + e0 * 2 * NU, ne, lane);
-    }
-  }
+  if constexpr (kEarly<DIM, N, GEN>) load_rate();
   float2 F[DIM][2];  // transformed common flux at the two ends: the own at L ends, the partner's at R ends
 #pragma unroll
   for (int a = 0; a < DIM; ++a) {
