@@ -14,7 +14,8 @@ void launch_kb_trir(const KArgs& A, cudaStream_t s) {
 }
 template <int P, int MODE, int SF>
 void launch_ka_stage(const KArgs& A, cudaStream_t s) {
-  ka_trir<P, MODE, SF><<<tri_grid<P>(A.E), TriReg<P>::TB, TriReg<P>::KA_SMEM, s>>>(A);
+  constexpr int per = TriReg<P>::TB / 32 * TriReg<P>::ka_elems(MODE);
+  ka_trir<P, MODE, SF><<<(unsigned)((A.E + per - 1) / per), TriReg<P>::TB, TriReg<P>::ka_smem(MODE), s>>>(A);
 }
 template <int P, int MODE>
 void launch_ka_trir(const KArgs& A, cudaStream_t s) {
@@ -28,7 +29,7 @@ void launch_ka_trir(const KArgs& A, cudaStream_t s) {
 }
 template <int P>
 bool fill_trir(bool physical, KernelSet* ks) {
-  static_assert(TriReg<P>::KB_SMEM <= 48 * 1024 && TriReg<P>::KA_SMEM <= 48 * 1024, "no shared-memory opt-in needed");
+  static_assert(TriReg<P>::KB_SMEM <= 48 * 1024 && TriReg<P>::ka_smem(1) <= 48 * 1024, "no shared-memory opt-in needed");
   if (physical) {
     ks->kb[0] = launch_kb_trir<P, 0>;
     ks->ka[0] = launch_ka_trir<P, 0>;

@@ -10,7 +10,8 @@
 //
 // The block-wide kernels computed each output as a dot product of two
 // shared-memory vectors (two loads a multiply-add, with a barrier a Step) and
-// were latency bound: 30.3 + 20.8 us a stage on 29,768 triangles of order 3.
+// were latency bound: 30.3 + 20.8 us a stage on 29,768 triangles of order 3, now
+// 7.8 + 8.3.
 #pragma once
 #include "kline_pseudo.cuh"
 #include "ktri.cuh"
@@ -58,7 +59,8 @@ struct TriReg {
   // weights (then traces), w det J pairs
   static constexpr int KA_F = 2 * NU + 4 * NU + 2 * NU + 2 * NF + 2 * NU;
   static_assert(SIZE % 4 == 0 && O_D % 4 == 0 && O_LIFT % 4 == 0 && O_V % 4 == 0, "16-byte boundaries");
-  static constexpr size_t KA_SMEM = ((size_t)SIZE + TB * KA_F) * 4;
+  __host__ __device__ static constexpr int ka_elems(int mode) { return mode == 0 ? 16 : 32; }  // elements a warp of the update kernel
+  static constexpr size_t ka_smem(int mode) { return ((size_t)SIZE + TB / 32 * ka_elems(mode) * KA_F) * 4; }
 };
 
 // edge ed of element e: flags, partner's first flux point (of the edge's first point; the partner's points run
@@ -391,23 +393,29 @@ __global__ void __launch_bounds__(TriReg<P>::TB) kb_trir(const __grid_constant__
 }
 
 // ---- update kernel: SF 1..4, or 0 for the traces of ustg alone -----------------
+// The fields are independent here, so a thread takes one field of one element
+// in the physical step (16 elements a warp, twice the warps of a thread an
+// element: 10.0 -> 8.3 us a stage on 29,768 triangles of order 3), psi of one
+// element in the preconditioning (32 a warp, rows of both fields in the buffers).
 template <int P, int MODE, int SF>
 __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__ KArgs A) {
   using R = TriReg<P>;
-  constexpr int N = R::N, NU = R::NU, NF = R::NF, NPE = R::NPE, NPU = R::NPU, NFLD = MODE == 0 ? 2 : 1, F0 = 2 - NFLD;
+  constexpr int N = R::N, NU = R::NU, NF = R::NF, NPE = R::NPE, NPU = R::NPU;
+  constexpr int EW = R::ka_elems(MODE);  // elements a warp
   if (MODE == 1 && *(volatile int32_t*)&A.status[ST_PSEUDO_DONE]) return;
   extern __shared__ __align__(16) float smem_f[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int el = MODE == 0 ? lane >> 1 : lane, f = MODE == 0 ? lane & 1 : 1;  // the thread's element and field
   float* ops = smem_f;
-  float* yb = ops + R::SIZE + warp * 32 * R::KA_F;
-  float* sb = yb + 32 * 2 * NU;   // solution pairs
-  float* ab = sb + 32 * 4 * NU;   // accumulator
-  float* tb = ab + 32 * 2 * NU;   // face weights, later the traces
-  float* wb = tb + 32 * 2 * NF;   // w det J pairs (stage 4)
-  const int64_t e0 = ((int64_t)blockIdx.x * R::TB) + warp * 32;
-  const int ne = (int)max((int64_t)0, min((int64_t)32, A.E - e0));
-  const bool act = lane < ne;
-  const int64_t e = min(e0 + lane, A.E - 1);
+  float* yb = ops + R::SIZE + warp * EW * R::KA_F;
+  float* sb = yb + EW * 2 * NU;   // solution pairs
+  float* ab = sb + EW * 4 * NU;   // accumulator
+  float* tb = ab + EW * 2 * NU;   // face weights, later the traces
+  float* wb = tb + EW * 2 * NF;   // w det J pairs (stage 4)
+  const int64_t e0 = ((int64_t)blockIdx.x * (R::TB / 32) + warp) * EW;
+  const int ne = (int)max((int64_t)0, min((int64_t)EW, A.E - e0));
+  const bool act = el < ne;
+  const int64_t e = min(e0 + el, A.E - 1);
   const float2* Lt = reinterpret_cast<const float2*>(ops + R::O_L);
   const float2* Lf = reinterpret_cast<const float2*>(ops + R::O_LIFT);
   const float* fcA = reinterpret_cast<const float*>(A.fc);
@@ -415,20 +423,20 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
   const bool cons = MODE == 0 && SF >= 1 && A.tacc && A.wphys;
 
   // ---- loads (whole rows of both fields)
-  tile_fetch<32, 2 * NU * 4>(yb, (SF == 0 ? ustg : reinterpret_cast<const float*>(A.rp)) + e0 * 2 * NU, ne, lane);
-  if (SF >= 1) tile_fetch<32, 2 * NU * 8>(sb, reinterpret_cast<const float2*>(A.u) + e0 * 2 * NU, ne, lane);
+  tile_fetch<EW, 2 * NU * 4>(yb, (SF == 0 ? ustg : reinterpret_cast<const float*>(A.rp)) + e0 * 2 * NU, ne, lane);
+  if (SF >= 1) tile_fetch<EW, 2 * NU * 8>(sb, reinterpret_cast<const float2*>(A.u) + e0 * 2 * NU, ne, lane);
   // acc: at stage 1 only the other field's half of a preconditioning row is kept
-  if (SF >= 2 || (SF == 1 && MODE == 1)) tile_fetch<32, 2 * NU * 4>(ab, reinterpret_cast<const float*>(A.acc) + e0 * 2 * NU, ne, lane);
+  if (SF >= 2 || (SF == 1 && MODE == 1)) tile_fetch<EW, 2 * NU * 4>(ab, reinterpret_cast<const float*>(A.acc) + e0 * 2 * NU, ne, lane);
   if (cons) {
-    tile_fetch<32, NF * 8>(tb, A.wphys + e0 * NF, ne, lane);
-    if (SF == 4) tile_fetch<32, NU * 8>(wb, A.wdetf + e0 * NU, ne, lane);
+    tile_fetch<EW, NF * 8>(tb, A.wphys + e0 * NF, ne, lane);
+    if (SF == 4) tile_fetch<EW, NU * 8>(wb, A.wdetf + e0 * NU, ne, lane);
   }
   float phi_keep[MODE == 1 ? NU : 1];  // preconditioning: phi's stage value
   if (MODE == 1 && SF >= 1)
 #pragma unroll
     for (int j = 0; j < NU; ++j) phi_keep[j] = ustg[e * 2 * NU + j];
   tri_ops(A, ops, R::SIZE);
-  float F[NFLD][3][N];
+  float F[3][N];
   int fl[3];
   float pm[3] = {0.f, 0.f, 0.f}, rdj = 0.f;
   if constexpr (SF >= 1) {
@@ -448,168 +456,125 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
       fl[ed] = tri_edge<P>(A, e, ed, off);
       const bool isl = fl[ed] & kFwL;
       // the own flux at L points, the partner's at R points (points backwards)
-      const int64_t b = isl ? e * 2 * NF + ed * N : off;
+      const float* b = fcA + (isl ? e * 2 * NF + ed * N : off) + f * NF;
       const int st = isl ? 1 : -1;
 #pragma unroll
-      for (int f = 0; f < NFLD; ++f)
-#pragma unroll
-        for (int k = 0; k < N; ++k) F[f][ed][k] = (NFLD == 2 || !isl) ? fcA[b + (F0 + f) * NF + k * st] : 0.f;
+      for (int k = 0; k < N; ++k) F[ed][k] = (MODE == 0 || !isl) ? b[k * st] : 0.f;
     }
   }
-  double ta[2] = {0.0, 0.0};
-  if (SF >= 2 && cons) {
-    const double2 t = *reinterpret_cast<const double2*>(A.tacc + e * 2);
-    ta[0] = t.x;
-    ta[1] = t.y;
-  }
+  double ta = 0.0;
+  if (SF >= 2 && cons) ta = A.tacc[e * 2 + f];
   cp_async_wait_all();
   __syncthreads();
-  float* yr = yb + lane * 2 * NU;
-  float2 y[NFLD][NPU];
+  float* yr = yb + (el * 2 + f) * NU;
+  float2 y[NPU];
 #pragma unroll
-  for (int f = 0; f < NFLD; ++f)
-#pragma unroll
-    for (int i = 0; i < NPU; ++i)
-      y[f][i] = make_float2(2 * i < NU ? yr[(F0 + f) * NU + (2 * i < NU ? 2 * i : 0)] : 0.f,
-                            2 * i + 1 < NU ? yr[(F0 + f) * NU + (2 * i + 1 < NU ? 2 * i + 1 : 0)] : 0.f);
+  for (int i = 0; i < NPU; ++i)
+    y[i] = make_float2(2 * i < NU ? yr[2 * i < NU ? 2 * i : 0] : 0.f, 2 * i + 1 < NU ? yr[2 * i + 1 < NU ? 2 * i + 1 : 0] : 0.f);
   [[maybe_unused]] float2 sh = make_float2(0.f, 0.f);  // MODE 1 stage 4: squared changes
   if constexpr (SF >= 1) {
     // ---- lift of minus the partner's flux at R points; flux balance
-    float2 bal[NFLD];
-#pragma unroll
-    for (int f = 0; f < NFLD; ++f) bal[f] = make_float2(0.f, 0.f);
+    float2 bal = make_float2(0.f, 0.f);
 #pragma unroll
     for (int ed = 0; ed < 3; ++ed) {
       const bool isl = fl[ed] & kFwL;
 #pragma unroll
       for (int k = 0; k < N; ++k) {
         if (cons) {
-          const float2 w = reinterpret_cast<const float2*>(tb)[lane * NF + ed * N + k];
-#pragma unroll
-          for (int f = 0; f < NFLD; ++f) bal[f] = ff_add(bal[f], ff_mul(w, isl ? F[f][ed][k] : -F[f][ed][k]));
+          const float2 w = reinterpret_cast<const float2*>(tb)[el * NF + ed * N + k];
+          bal = ff_add(bal, ff_mul(w, isl ? F[ed][k] : -F[ed][k]));
         }
         tri_fence();
-#pragma unroll
-        for (int f = 0; f < NFLD; ++f)
-          tri_acc<NPU>(Lf + (ed * N + k) * NPU, isl ? 0.f : -pm[ed] * F[f][ed][k], y[f]);
+        tri_acc<NPU>(Lf + (ed * N + k) * NPU, isl ? 0.f : -pm[ed] * F[ed][k], y);
       }
     }
     if (cons && SF < 4 && act) {
-      double2 t;
-      t.x = -((double)bal[0].x + (double)bal[0].y);
-      t.y = -((double)bal[NFLD - 1].x + (double)bal[NFLD - 1].y);
-      if (SF >= 2) {
-        t.x = ta[0] + 2.0 * t.x;
-        t.y = ta[1] + 2.0 * t.y;
-      }
-      *reinterpret_cast<double2*>(A.tacc + e * 2) = t;
+      const double Te = -((double)bal.x + (double)bal.y);
+      A.tacc[e * 2 + f] = SF == 1 ? Te : ta + 2.0 * Te;
     }
-    float2* sr = reinterpret_cast<float2*>(sb) + lane * 2 * NU;
-    float* ar = ab + lane * 2 * NU;
-    float2 dl[NFLD];
-#pragma unroll
-    for (int f = 0; f < NFLD; ++f) dl[f] = make_float2(0.f, 0.f);
+    float2* sr = reinterpret_cast<float2*>(sb) + (el * 2 + f) * NU;
+    float* ar = ab + (el * 2 + f) * NU;
     float bad = 0.f;
-    float2 Ssum[NFLD], W = make_float2(0.f, 0.f);
-#pragma unroll
-    for (int f = 0; f < NFLD; ++f) Ssum[f] = make_float2(0.f, 0.f);
+    float2 Ssum = make_float2(0.f, 0.f), W = Ssum;
 #pragma unroll
     for (int j = 0; j < NU; ++j) {
-      float2 wd = make_float2(0.f, 0.f);
-      if (SF == 4 && cons) {
-        wd = reinterpret_cast<const float2*>(wb)[lane * NU + j];
-        W = ff_add(W, wd);
-      }
-#pragma unroll
-      for (int f = 0; f < NFLD; ++f) {
-        const float Rj = -pair_at(y[f], j) * rdj;
-        const int i = (F0 + f) * NU + j;
-        const float2 uu = sr[i];
-        float yn;
-        if constexpr (SF == 1) {
-          ar[i] = Rj;
-          yn = uu.x + __fmaf_rn(A.rk.half_dt, Rj, uu.y);
-        } else if constexpr (SF == 2 || SF == 3) {
-          ar[i] = __fmaf_rn(2.f, Rj, ar[i]);
-          yn = uu.x + __fmaf_rn(SF == 2 ? A.rk.half_dt : A.rk.dt, Rj, uu.y);
-        } else {
-          const float inc = A.rk.dt6 * (ar[i] + Rj);
-          const float s2 = uu.x + inc;
-          const float e2 = two_sum_lo(uu.x, inc, s2) + uu.y;
-          yn = s2 + e2;
-          const float lo = e2 - (yn - s2);
-          sr[i] = make_float2(yn, lo);
-          if constexpr (MODE == 0) {
-            if (cons) Ssum[f] = ff_add(Ssum[f], ff_mul(wd, inc));
-          } else {
-            const float h = yn - uu.x, l = two_sum_lo(yn, -uu.x, h) + (lo - uu.y);
-            const float sq = __fmul_rn(h, h);
-            sh = ff_add(sh, make_float2(sq, __fmaf_rn(2.f * h, l, __fmaf_rn(h, h, -sq))));
+      const float Rj = -pair_at(y, j) * rdj;
+      const float2 uu = sr[j];
+      float yn;
+      if constexpr (SF == 1) {
+        ar[j] = Rj;
+        yn = uu.x + __fmaf_rn(A.rk.half_dt, Rj, uu.y);
+      } else if constexpr (SF == 2 || SF == 3) {
+        ar[j] = __fmaf_rn(2.f, Rj, ar[j]);
+        yn = uu.x + __fmaf_rn(SF == 2 ? A.rk.half_dt : A.rk.dt, Rj, uu.y);
+      } else {
+        const float inc = A.rk.dt6 * (ar[j] + Rj);
+        const float s2 = uu.x + inc;
+        const float e2 = two_sum_lo(uu.x, inc, s2) + uu.y;
+        yn = s2 + e2;
+        const float lo = e2 - (yn - s2);
+        sr[j] = make_float2(yn, lo);
+        if constexpr (MODE == 0) {
+          if (cons) {
+            const float2 wd = reinterpret_cast<const float2*>(wb)[el * NU + j];
+            W = ff_add(W, wd);
+            Ssum = ff_add(Ssum, ff_mul(wd, inc));
           }
+        } else {
+          const float h = yn - uu.x, l = two_sum_lo(yn, -uu.x, h) + (lo - uu.y);
+          const float sq = __fmul_rn(h, h);
+          sh = ff_add(sh, make_float2(sq, __fmaf_rn(2.f * h, l, __fmaf_rn(h, h, -sq))));
         }
-        bad = __fmaf_rn(yn, 0.f, bad);
-        if (j & 1) y[f][j / 2].y = yn;
-        else y[f][j / 2].x = yn;
       }
+      bad = __fmaf_rn(yn, 0.f, bad);
+      if (j & 1) y[j / 2].y = yn;
+      else y[j / 2].x = yn;
     }
     if constexpr (SF == 4 && MODE == 0) {
       if (cons) {
+        const double Te = -((double)bal.x + (double)bal.y);
+        const double tgt = A.rk.ddt6 * (ta + Te);
+        const double d = (tgt - ((double)Ssum.x + (double)Ssum.y)) / ((double)W.x + (double)W.y);
+        const float dh = (float)d, dl = (float)(d - (double)dh);
 #pragma unroll
-        for (int f = 0; f < NFLD; ++f) {
-          const double Te = -((double)bal[f].x + (double)bal[f].y);
-          const double tgt = A.rk.ddt6 * (ta[f] + Te);
-          const double d = (tgt - ((double)Ssum[f].x + (double)Ssum[f].y)) / ((double)W.x + (double)W.y);
-          dl[f].x = (float)d;
-          dl[f].y = (float)(d - (double)dl[f].x);
+        for (int j = 0; j < NU; ++j) {
+          const float2 uu = sr[j];
+          const float s2 = uu.x + dh;
+          const float e2 = two_sum_lo(uu.x, dh, s2) + (uu.y + dl);
+          const float hi = s2 + e2;
+          sr[j] = make_float2(hi, e2 - (hi - s2));
+          bad = __fmaf_rn(hi, 0.f, bad);
+          if (j & 1) y[j / 2].y = hi;
+          else y[j / 2].x = hi;
         }
-#pragma unroll
-        for (int j = 0; j < NU; ++j)
-#pragma unroll
-          for (int f = 0; f < NFLD; ++f) {
-            const float2 uu = sr[(F0 + f) * NU + j];
-            const float s2 = uu.x + dl[f].x;
-            const float e2 = two_sum_lo(uu.x, dl[f].x, s2) + (uu.y + dl[f].y);
-            const float hi = s2 + e2;
-            sr[(F0 + f) * NU + j] = make_float2(hi, e2 - (hi - s2));
-            bad = __fmaf_rn(hi, 0.f, bad);
-            if (j & 1) y[f][j / 2].y = hi;
-            else y[f][j / 2].x = hi;
-          }
       }
     }
     if (act && bad != 0.f) atomicExch(&A.status[ST_STATUS], -4);
 #pragma unroll
-    for (int f = 0; f < NFLD; ++f)
-#pragma unroll
-      for (int j = 0; j < NU; ++j) yr[(F0 + f) * NU + j] = pair_at(y[f], j);
+    for (int j = 0; j < NU; ++j) yr[j] = pair_at(y, j);
     if (MODE == 1)
 #pragma unroll
-      for (int j = 0; j < NU; ++j) yr[j] = phi_keep[j];
+      for (int j = 0; j < NU; ++j) yr[j - NU] = phi_keep[j];
   }
-  // ---- traces of the new stage value (psi's alone are packed across the lanes' weights)
-  if (NFLD == 1) __syncwarp();
-  float* trr = tb + lane * NFLD * NF;
+  // ---- traces of the new stage value, in the weights' place (rows of the warp's threads)
+  __syncwarp();
+  float* trr = tb + lane * NF;
 #pragma unroll
   for (int ed = 0; ed < 3; ++ed) {
-    float2 t[NFLD][NPE];
+    float2 t[NPE];
 #pragma unroll
-    for (int f = 0; f < NFLD; ++f)
-#pragma unroll
-      for (int i = 0; i < NPE; ++i) t[f][i] = dup2(0.f);
+    for (int i = 0; i < NPE; ++i) t[i] = dup2(0.f);
 #pragma unroll
     for (int j = 0; j < NU; ++j) {
       tri_fence();
-#pragma unroll
-      for (int f = 0; f < NFLD; ++f) tri_acc<NPE>(Lt + (ed * NU + j) * NPE, pair_at(y[f], j), t[f]);
+      tri_acc<NPE>(Lt + (ed * NU + j) * NPE, pair_at(y, j), t);
     }
 #pragma unroll
-    for (int f = 0; f < NFLD; ++f)
-#pragma unroll
-      for (int k = 0; k < N; ++k) trr[f * NF + ed * N + k] = pair_at(t[f], k);
+    for (int k = 0; k < N; ++k) trr[ed * N + k] = pair_at(t, k);
   }
   __syncwarp();
   float* tr = reinterpret_cast<float*>(A.tr);
-  if constexpr (NFLD == 2) tri_flush<2 * NF * 4>(tr + e0 * 2 * NF, tb, ne, lane);
+  if constexpr (MODE == 0) tri_flush<2 * NF * 4>(tr + e0 * 2 * NF, tb, ne, lane);
   else rows_flush<NF>(tr + (e0 * 2 + 1) * NF, tb, 2 * NF, ne, lane);
   if constexpr (SF >= 1) {
     tri_flush<2 * NU * 4>(ustg + e0 * 2 * NU, yb, ne, lane);
