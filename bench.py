@@ -188,7 +188,8 @@ def source_sha():
     h = hashlib.sha256()
     # the tensor kernels, their launch table and the field set-up that lays
     # out the arrays they read
-    for fn in ("ktensor.cuh", "kcommon.cuh", "geom.cuh", "k_tensor_inst.cuh", "api.cu"):
+    for fn in ("kline.cuh", "k_line_inst.cuh", "kdispatch.hpp", "ktensor.cuh", "kcommon.cuh", "geom.cuh",
+               "k_tensor_inst.cuh", "api.cu"):
         h.update(open(os.path.join(ROOT, "paper_2006_10967_gb300", "csrc", fn), "rb").read())
     return h.hexdigest()[:16]
 
@@ -401,7 +402,7 @@ def run_ensemble(G, S, K, W, world, flush, precision="mixed", n_inst=256, rk_ste
     peak = pk.get("hbm_gbs") or 6800.0
     roof = {"bound": "hbm", "kernel": ("RK stage of all orders: kb_group + ka_group (one launch each)"
                                        if group is not None else
-                                       "RK stage of every order group (kb_tensor + ka_tensor per order, 4 streams)"),
+                                       "RK stage of every order group (kb_line + ka_line per order, 4 streams)"),
             "achieved": b_stage / stage_s / 1e9, "peak": peak, "unit": "GB/s",
             "frac": b_stage / stage_s / 1e9 / peak, "traffic": None,
             "alg_bytes_per_stage": b_stage, "stage_us": stage_s * 1e6,
@@ -819,8 +820,9 @@ def roofline(out, etype, p, precision, workload):
         if v[1]:
             stage_kern[k]["share_of_step"] = v[0] / tot
     traffic_dof = load_traffic(f"stage_{workload}_{etype}_p{p}_{precision}")
-    return {"bound": "hbm", "kernel": "RK stage: kb_tensor + ka_tensor" if etype != "tri" else
-            "RK stage: kb_tri + ka_tri",
+    kname = {"mixed": {"tri": "trir"}, "fp64": {"tri": "tri"}}[precision].get(
+        etype, "line" if precision == "mixed" else "tensor")
+    return {"bound": "hbm", "kernel": f"RK stage: kb_{kname} + ka_{kname}",
             "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": traffic_dof * ndof if traffic_dof else None,
             "alg_bytes_per_dof_stage": b_alg, "stage_us": stage_s * 1e6,

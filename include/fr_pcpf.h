@@ -158,10 +158,12 @@ typedef struct fr_params {
   int32_t variant;       /* implementation of the residual and update kernels, all giving the
                             same result to round-off: 0 the default; fr_kernel_variants gives
                             the count for a mesh and precision (FR_MIXED: triangles 0 scalar
-                            dot products, 1 the operator applies on tensor cores, mma.sync
+                            arithmetic, 1 the operator applies on tensor cores, mma.sync
                             m16n8k8 in three-term TF32 with FP32 accumulation; quads and hexes
-                            the element tiles of the physical-step residual and update kernels:
-                            0 default/default, 1 half/half, 2 default/half, 3 half/default).
+                            the element tiles of the block-wide physical-step residual and
+                            update kernels: 0 default/default, 1 half/half, 2 default/half,
+                            3 half/default; fields with a velocity cache on quads and on hexes
+                            of order <= 4 run warp-per-element kernels under every number).
                             An autotuner picks among them by measurement.  Out of range:
                             FR_EUNSUPPORTED from fr_field_init, negative: FR_EINVAL */
 } fr_params;

@@ -47,9 +47,9 @@ bool reg_kernels_tri(int order, bool physical, KernelSet* ks);
 
 // Warps a block of the line kernels.  Their warps are independent, so small
 // blocks spread best (64^3 hexes p = 3, residual + update: 185 + 183 us with
-// four, 183 + 178 with two); the preconditioning's stage 4 leaves one partial a
-// block for the last block to add up and takes four (stage 4 of 64^3: with two
-// warps a block the update kernel's mean goes from 122 to 151 us).
+// four, 183 + 178 with two).  The preconditioning's stage 4 leaves one partial
+// a block for the last block to add up, on a grid of a fixed number of blocks:
+// four warps each, half the partials of two.
 constexpr int kLineWarps = 2, kPseudoWarps = 4;
 // Blocks of the preconditioning's stage 4 update: six of 128 threads on each SM.
 constexpr unsigned kPseudoBlocks = 152 * 6;

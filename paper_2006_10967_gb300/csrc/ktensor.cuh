@@ -21,6 +21,10 @@
 // MODE 0 is the physical system u = [phi, psi]; MODE 1 the preconditioning
 // system for psi alone (Eq. pseudotimesystem) with element viscosity nu_s
 // from the resolution indicator (Eqs. resolutionIndicator, nu_s).
+//
+// They serve the FP64 path, the adjoint's recomputation, the ensemble's one
+// launch, and mixed fields that keep no velocity cache or are hexes of order 5;
+// the other mixed fields run on kline.cuh.
 #pragma once
 #include <type_traits>
 

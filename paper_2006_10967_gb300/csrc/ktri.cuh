@@ -12,7 +12,8 @@
 //   Step 6      div~ f~        = Dr f~_0 + Ds f~_1 + LIFT (F~ - f~perp)   ([Dr | Ds | LIFT], NU x (2 NU + NF))
 //   ka          R-side lift LIFT c and the next stage's traces L y
 // The FP64 path keeps scalar dot products (FP64 tensor throughput is far
-// below the FP64 FMA pipe's on this GPU).
+// below the FP64 FMA pipe's on this GPU).  Mixed fields of variant 0 and order
+// up to 4 run on ktri_reg.cuh (their physical step where the velocity is cached).
 #pragma once
 #include <type_traits>
 
