@@ -48,9 +48,10 @@ __device__ __forceinline__ float2 ff_div(float2 a, float2 b) {
 // (1 + sin(pi (log10 r - s0) / (2 kappa))) / 2 is sin^2 z.  The logarithm is the
 // series 2 (t + t^3 / 3 + ...) of the significand m in [1/sqrt 2, sqrt 2),
 // t = (m - 1) / (m + 1), and the sine its Taylor series up to pi / 4, both with
-// the leading term in float-float, so that nu_s is good to a float rounding as
-// the FP64 evaluation was (log10 and sin in FP64 took a warp 3000 cycles of the
-// FP64 pipe wherever one of its elements lies in the ramp).
+// the leading terms in float-float, so that nu_s is the rounded exact value to
+// 5.956e-8 (the FP64 evaluation too; 99.99 % of the results are the same).
+// log10 and sin in FP64 took a warp 3000 cycles of the FP64 pipe wherever one of
+// its elements lies in the ramp.
 __device__ __forceinline__ float sensor_nu(const PhysPrm& P, float2 lo, float2 hi, float2 nu_max) {
   const float tot = lo.x + hi.x;
   if (!(tot > 0.f) || !(hi.x > 0.f)) return 0.f;
@@ -66,12 +67,14 @@ __device__ __forceinline__ float sensor_nu(const PhysPrm& P, float2 lo, float2 h
   const float sc = mh / r.x;  // a power of two
   const float2 m = make_float2(mh, r.y * sc);
   const float2 t = ff_div(ff_add(m, make_float2(-1.f, 0.f)), ff_add(m, make_float2(1.f, 0.f)));
+  const float2 t3 = ff_mul2(ff_mul2(t, t), t);
   const float t2 = t.x * t.x;
-  float ps = __fmaf_rn(t2, 1.f / 11.f, 1.f / 9.f);
+  float ps = __fmaf_rn(t2, 1.f / 13.f, 1.f / 11.f);
+  ps = __fmaf_rn(t2, ps, 1.f / 9.f);
   ps = __fmaf_rn(t2, ps, 1.f / 7.f);
   ps = __fmaf_rn(t2, ps, 1.f / 5.f);
-  ps = __fmaf_rn(t2, ps, 1.f / 3.f);
-  const float2 half_log = ff_add(t, make_float2(t.x * t2 * ps, 0.f));
+  const float2 third = make_float2(0.333333343f, -9.93410776e-9f);
+  const float2 half_log = ff_add(t, ff_add(ff_mul2(t3, third), make_float2(t3.x * t2 * ps, 0.f)));
   // z = C0 + k C1 + half_log C2
   float2 z = ff_add(ff_mul2(make_float2(P.ramp_c1h, P.ramp_c1l), make_float2((float)k, 0.f)),
                     ff_mul2(make_float2(P.ramp_c2h, P.ramp_c2l), half_log));
@@ -81,11 +84,12 @@ __device__ __forceinline__ float sensor_nu(const PhysPrm& P, float2 lo, float2 h
   if (z.x >= hpi.x) return nu_max.x;
   const bool up = z.x > 0.785398163f;
   if (up) z = ff_add(hpi, make_float2(-z.x, -z.y));  // sin^2 z = 1 - sin^2(pi/2 - z)
-  const float z2 = z.x * z.x;
-  float s = __fmaf_rn(z2, 1.f / 362880.f, -1.f / 5040.f);
-  s = __fmaf_rn(z2, s, 1.f / 120.f);
-  s = __fmaf_rn(z2, s, -1.f / 6.f);
-  float2 v = ff_add(z, make_float2(z.x * z2 * s, 0.f));
+  const float2 z2 = ff_mul2(z, z), z3 = ff_mul2(z2, z);
+  float s = __fmaf_rn(z2.x, -1.f / 39916800.f, 1.f / 362880.f);
+  s = __fmaf_rn(z2.x, s, -1.f / 5040.f);
+  const float2 sixth = make_float2(-0.166666672f, 4.96705388e-9f), c5 = make_float2(0.00833333377f, -4.34617203e-10f);
+  const float2 z35 = ff_add(sixth, ff_add(ff_mul2(z2, c5), make_float2(z2.x * z2.x * s, 0.f)));
+  float2 v = ff_add(z, ff_mul2(z3, z35));
   v = ff_mul2(v, v);
   if (up) v = ff_add(make_float2(1.f, 0.f), make_float2(-v.x, -v.y));
   v = ff_mul2(v, nu_max);
