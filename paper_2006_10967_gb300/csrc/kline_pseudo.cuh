@@ -252,9 +252,9 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
   //      lane's line holds modes (its two indices, 0..N-1)) and at it
   float nu;
   {
-    // scaled by 2^40 (exact) so that the squares of small coefficients keep their low parts
+    // scaled by 2^20 (exact): squares of coefficients from 1e-18 to 1e12 neither overflow nor lose their low parts
 #pragma unroll
-    for (int m = 0; m < N; ++m) cm[m] *= 0x1p40f;
+    for (int m = 0; m < N; ++m) cm[m] *= 0x1p20f;
     const bool top = DIM == 3 ? (l % N == N - 1 || l / N == N - 1) : l == N - 1;
     float2 b = make_float2(0.f, 0.f), t;
 #pragma unroll

@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(TriReg<P>::TB) kb_trir(const __grid_constant__
     for (int i = 0; i <= P; ++i)
 #pragma unroll
       for (int j = 0; j <= P - i; ++j, ++m) {
-        const float v = pair_at(c, m) * 0x1p40f;  // as in kbp_line
+        const float v = pair_at(c, m) * 0x1p20f;  // as in kbp_line
         const float s = __fmul_rn(v, v);
         float2& t = i + j == P ? hi : lo;
         t = ff_add(t, make_float2(s, __fmaf_rn(v, v, -s)));
