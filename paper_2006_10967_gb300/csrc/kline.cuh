@@ -200,13 +200,12 @@ __device__ __forceinline__ void tile_fetch(float* dst, const void* src, int ne, 
   }
 }
 // Programmatic dependent launch: a kernel's blocks start while the kernel before
-// it drains, and read what that kernel wrote only after pdl_wait (its
-// completion).  pdl_launch follows pdl_wait in every kernel, so that when a
-// kernel's blocks run, all kernels but the one before it are complete: before
-// pdl_wait they read connectivity, metric, weights and velocity data (written
-// at set-up) and, in the update kernels, the solution, accumulator and flux
-// balances (written by the update before; between them the residual kernel
-// writes only rp and fc).  Every kernel waits before it returns.
+// it drains.  Only pdl_wait makes another kernel's writes visible, so before it
+// they read nothing that a kernel of the march writes: connectivity, metric,
+// weights, parameters and velocity data, all written at set-up.  The solution,
+// accumulator and flux balances of the update kernels come from the update two
+// kernels before, which is complete by then, but they are read after pdl_wait
+// like the rest.  Every kernel waits before it returns.
 // kEarly: regular hexes of N >= 4 (the large 3D runs) wait first and load their
 // state first: with thousands of blocks a wave there is little to hide, and the
 // other order cost them 2 % (64^3 p = 3: 358 and 350 us a stage).
@@ -1002,31 +1001,24 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
   double ta = 0.0;  // this thread's element balance so far (finished by the first threads of the block)
   const int64_t gt = (int64_t)blockIdx.x * NEL * 2 + threadIdx.x;
   float2 rW = make_float2(0.f, 0.f);  // stage 4: 1 / W
-  auto load_rate = [&]() {
+  // what the march writes: the rate, the solution, the accumulator and the flux
+  // balances, all after pdl_wait
+  auto load_state = [&]() {
     pdl_wait();
     pdl_launch();
     const float* src = SF == 0 ? ustg : reinterpret_cast<const float*>(A.rp);
     if constexpr (L::DIRECT) {
 #pragma unroll
-      for (int f = 0; f < 2; ++f) grow_get<N>(src + (e * 2 + f) * NU + l * N, y[f]);
-    } else if (ne > 0) {
-      tile_fetch<EPW, 2 * NU * 4>(in, src + e0 * 2 * NU, ne, lane);
-    }
-  };
-  if constexpr (!kEarly<DIM, N, GEN>) load_rate();
-  if constexpr (SF >= 1) {
-    const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
-    rdet = __ldg(mc + 10);
-    if (GEN) aff = DIM == 3 ? __ldg(mc + 11) : 0.f;
-    if constexpr (L::DIRECT) {
-#pragma unroll
       for (int f = 0; f < 2; ++f) {
         const int64_t r = (e * 2 + f) * NU + l * N;
+        grow_get<N>(src + r, y[f]);
+        if constexpr (SF >= 1) {
 #pragma unroll
-        for (int j = 0; j < N; j += 2) {
-          const float4 t = *reinterpret_cast<const float4*>(U + r + j);
-          u[f][j] = make_float2(t.x, t.y);
-          u[f][j + 1] = make_float2(t.z, t.w);
+          for (int j = 0; j < N; j += 2) {
+            const float4 t = *reinterpret_cast<const float4*>(U + r + j);
+            u[f][j] = make_float2(t.x, t.y);
+            u[f][j + 1] = make_float2(t.z, t.w);
+          }
         }
         if constexpr (SF >= 2) {
           float2 t[NP];
@@ -1035,16 +1027,23 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
         }
       }
     } else if (ne > 0) {
-      tile_fetch<EPW, 2 * NU * 8>(in + K::O_U, U + e0 * 2 * NU, ne, lane);
+      tile_fetch<EPW, 2 * NU * 4>(in, src + e0 * 2 * NU, ne, lane);
+      if constexpr (SF >= 1) tile_fetch<EPW, 2 * NU * 8>(in + K::O_U, U + e0 * 2 * NU, ne, lane);
       if constexpr (SF >= 2) tile_fetch<EPW, 2 * NU * 4>(in + K::O_A, acc + e0 * 2 * NU, ne, lane);
     }
+    if constexpr (SF >= 2)
+      if (cons && threadIdx.x < 2 * NEL && gt < 2 * A.E) ta = A.tacc[gt];
+  };
+  if constexpr (!kEarly<DIM, N, GEN>) load_state();
+  if constexpr (SF >= 1) {
+    const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
+    rdet = __ldg(mc + 10);
+    if (GEN) aff = DIM == 3 ? __ldg(mc + 11) : 0.f;
     if (SF == 4 && cons && ne > 0) tile_fetch<EPW, NU * 8>(wsm + K::O_W, A.wdetf + e0 * NU, ne, lane);
     if (GEN && ne > 0) tile_fetch<EPW, L::S::NG * 4>(wsm + K::O_GEO, A.geof + e0 * L::S::NG, ne, lane);
     rk = A.ep ? A.ep[e].rk : A.rk;
-    if (SF >= 2 && cons && threadIdx.x < 2 * NEL && gt < 2 * A.E) {
-      ta = A.tacc[gt];
-      if (SF == 4) rW = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(A.mcg) + (gt / 2) * kMetricRec + 12);
-    }
+    if (SF == 4 && cons && threadIdx.x < 2 * NEL && gt < 2 * A.E)
+      rW = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(A.mcg) + (gt / 2) * kMetricRec + 12);
   }
   int fl[DIM][2];
   [[maybe_unused]] int2 fw[DIM][2];
@@ -1056,7 +1055,7 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
       if constexpr (DIM == 3) fw[a][sd] = __ldg(A.ffw + e * 6 + 2 * a + sd);
       else w2[a][sd] = __ldg(A.fnbr + e * NF + (2 * a + sd) * NFP + l);
     }
-  if constexpr (kEarly<DIM, N, GEN>) load_rate();
+  if constexpr (kEarly<DIM, N, GEN>) load_state();
   float2 F[DIM][2];  // transformed common flux at the two ends: the own at L ends, the partner's at R ends
 #pragma unroll
   for (int a = 0; a < DIM; ++a) {

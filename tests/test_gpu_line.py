@@ -158,3 +158,25 @@ def test_triangle_thread_kernels_agree_with_the_block_wide_ones(G, order, mk, ve
         assert _rel(F.get(which), B.get(which)) < 2e-5
     if not walls:
         assert abs(F.mass(0) - m0) < 1e-13
+
+
+@pytest.mark.parametrize("etype,order,ns,jitter,vel", [("quad", 3, (180, 150), 0.0, "rider_kothe"),
+                                                       ("quad", 4, (160, 150), 0.1, "stream"),
+                                                       ("hex", 2, (24, 23, 22), 0.1, "leveque"),
+                                                       ("hex", 3, (22, 20, 19), 0.0, "leveque")])
+def test_early_launched_kernels_march_as_serialised_ones(G, etype, order, ns, jitter, vel):
+    """On meshes of several waves, where an element's block runs on another SM
+    each time, the graph's launches (each kernel's blocks start while the one
+    before it drains) give the bits of launches with an event between them."""
+    w, mesh = _workload(etype, order, ns, jitter, vel, False)
+    M = G.Mesh.from_synthetic(mesh, order)
+    P = G.make_params(w, "mixed", pseudo_fixed=True, n_precond=1000)
+    F, R = [G.Field(M, P, ic=w.circle) for _ in range(2)]
+    R.profile(True)
+    for f in (F, R):
+        f.step(19)
+        assert f.sync() == 0
+    assert R.profile_read()["ka_phys"][1] == 4 * 19
+    for which in (0, 1):
+        assert np.array_equal(F.get(which), R.get(which))
+    assert F.mass(0) == R.mass(0)
