@@ -146,7 +146,10 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
 #pragma unroll
   for (int a = 0; a < DIM; ++a) sd[a] = __ldg(mc + a * 4);
   const float det = __ldg(mc + 9), rdet = __ldg(mc + 10);
-  if (*(volatile int32_t*)&A.status[ST_PSEUDO_DONE]) return;
+  if (*(volatile int32_t*)&A.status[ST_PSEUDO_DONE]) {
+    if (GEN) cp_async_wait_all();  // no copy in flight outlives its block
+    return;
+  }
   float2 u[NP], o[DIM];
   const float* ug = reinterpret_cast<const float*>(A.ustg);
   if constexpr (L::DIRECT) grow_get<N>(ug + (e * 2 + 1) * NU + l * N, u);

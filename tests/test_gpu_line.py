@@ -180,3 +180,32 @@ def test_early_launched_kernels_march_as_serialised_ones(G, etype, order, ns, ji
     for which in (0, 1):
         assert np.array_equal(F.get(which), R.get(which))
     assert F.mass(0) == R.mass(0)
+
+
+@pytest.mark.parametrize("etype,order,ns,jitter", [("quad", 3, (9, 7), 0.1), ("quad", 4, (8, 5), 0.0),
+                                                   ("hex", 2, (4, 3, 3), 0.1), ("hex", 3, (4, 3, 3), 0.1),
+                                                   ("tri", 3, (7, 5), 0.0)])
+def test_preconditioning_after_its_stop_rule_does_nothing(G, etype, order, ns, jitter):
+    """The launches that follow the iteration at which the stop rule holds
+    return at once: the state is that of the iterations up to it, bit for bit."""
+    w, mesh = _workload("quad" if etype == "tri" else etype, order, ns, jitter, "uniform", True)
+    if etype == "tri":
+        mesh = S.tri_split(*ns, periodic=(False, False))
+    M = G.Mesh.from_synthetic(mesh, order)
+    rms = []
+    for k in (1, 2, 3):
+        w.pseudo_kmax = k
+        rms.append(G.Field(M, G.make_params(w, "mixed", pseudo_fixed=True), ic=w.circle).stats()["last_pseudo_rms"])
+    assert rms[0] > rms[1] > rms[2] > 0
+    w.pseudo_kmax, w.pseudo_tol = 12, rms[1]
+    F = G.Field(M, G.make_params(w, "mixed"), ic=w.circle)
+    w.pseudo_kmax = 2
+    R = G.Field(M, G.make_params(w, "mixed", pseudo_fixed=True), ic=w.circle)
+    assert F.stats()["last_pseudo_iters"] == R.stats()["last_pseudo_iters"] == 2
+    assert F.stats()["last_pseudo_rms"] == R.stats()["last_pseudo_rms"]
+    for which in (0, 1):
+        assert np.array_equal(F.get(which), R.get(which))
+    for f in (F, R):
+        f.step(2)
+        assert f.sync() == 0
+    assert np.array_equal(F.get(0), R.get(0))
