@@ -181,6 +181,21 @@ bool set_line_kernels(const fr_mesh& m, bool gen, bool tab, bool nphi, KernelSet
   return m.etype == FR_QUAD ? line_kernels_quad(m.order, gen, tab, nphi, ks) : line_kernels_hex(m.order, gen, tab, nphi, ks);
 }
 
+// Whether every edge's partner points are one edge's, last to first, as on any
+// mesh whose triangles do not overlap (all are oriented alike).  The
+// thread-per-element kernels take an edge's partner from its first point; the
+// block-wide ones, which follow each point's own word, keep other meshes.
+bool tri_edges_backwards(const fr_mesh& m) {
+  const int n = m.n;
+  for (int64_t b = 0; b < m.E * m.nf; b += n) {
+    const int64_t w = m.fnbr[b], p = w >> 1;
+    for (int k = 0; k < n; ++k)
+      if (m.fnbr[b + k] != (p == b ? ((b + k) << 1 | 1) : ((p - k) << 1 | (w & 1)))) return false;
+    if (p != b && p % n != n - 1) return false;
+  }
+  return true;
+}
+
 // Blocks of the largest launch (one reduction partial each): the block-wide
 // kernels', the element-wise kernels' or the line kernels'.
 int most_blocks(const fr_mesh& m, const KernelSet& ks, int elementwise) {
@@ -854,7 +869,8 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
     A.tripack = reinterpret_cast<const float*>(b + L.tri_pack);
     // variant 0 of the mixed path at p <= 4 (variant 1: tensor cores; p = 5 has
     // more values an element than a thread's registers)
-    if (prm->precision == FR_MIXED && prm->variant == 0 && m->order <= 4) reg_kernels_tri(m->order, prm->vel_cache, &f->ks);
+    if (prm->precision == FR_MIXED && prm->variant == 0 && m->order <= 4 && tri_edges_backwards(*m))
+      reg_kernels_tri(m->order, prm->vel_cache, &f->ks);
     const uint8_t* hi = reinterpret_cast<const uint8_t*>(b + L.tri_high);
     A.trid = tri_pointers<double>(m->tri, reinterpret_cast<const double*>(b + L.tri_d), hi);
     A.trif = tri_pointers<float>(m->tri, reinterpret_cast<const float*>(b + L.tri_f), hi);

@@ -209,3 +209,21 @@ def test_preconditioning_after_its_stop_rule_does_nothing(G, etype, order, ns, j
         f.step(2)
         assert f.sync() == 0
     assert np.array_equal(F.get(0), R.get(0))
+
+
+@pytest.mark.parametrize("order", [1, 2, 3, 4])
+def test_triangles_on_the_same_side_of_their_edge(G, order):
+    """Two triangles that overlap: the points of the edge they share run alike
+    in both, not backwards.  The march follows FP64's as on any other mesh."""
+    w, _ = _workload("quad", order, (2, 2), 0.0, "uniform", True)
+    mesh = S.meshes.Mesh("tri", np.array([[0.0, 0.0], [1.0, 0.0], [0.3, 1.0], [0.6, 0.8]]),
+                         np.array([[0, 1, 2], [0, 1, 3]]), (False, False), (1.0, 1.0), "folded")
+    M = G.Mesh.from_synthetic(mesh, order)
+    F, D = [G.Field(M, G.make_params(w, p, pseudo_fixed=True), ic=w.circle) for p in ("mixed", "fp64")]
+    assert _rel(F.rhs_pseudo().cpu().numpy(), D.rhs_pseudo().cpu().numpy()) < 1e-4
+    assert _rel(F.rhs(0.3).cpu().numpy(), D.rhs(0.3).cpu().numpy()) < 1e-4
+    for f in (F, D):
+        f.step(2)
+        assert f.sync() == 0
+    for which in (0, 1):
+        assert _rel(F.get(which), D.get(which)) < 1e-5
