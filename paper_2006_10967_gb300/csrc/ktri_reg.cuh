@@ -64,13 +64,27 @@ struct TriReg {
 };
 
 // edge ed of element e: flags, partner's first flux point (of the edge's first point; the partner's points run
-// backwards) as an offset into an E x 2 x NF array (field 0)
+// backwards, which a field that takes these kernels has of every edge, see tri_edges_backwards) as an offset into an
+// E x 2 x NF array (field 0).  The checked build looks at all words of the edge; an edge that is not whole becomes a wall.
 template <int P>
 __device__ __forceinline__ int tri_edge(const KArgs& A, int64_t e, int ed, int64_t& off) {
   constexpr int NF = TriS<P>::NF, N = P + 1;
   const int32_t own = (int32_t)(e * NF + ed * N);
   const int32_t w = __ldg(A.fnbr + own);
-  const int32_t p = partner<NF>(A, w, own);
+  const int32_t p = w >> 1;
+#ifdef FR_BOUNDS_CHECK
+  for (int k = 0; k < N; ++k) {
+    const int32_t wk = __ldg(A.fnbr + own + k);
+    const bool whole = p == own ? wk == (int32_t)(((own + k) << 1) | 1)
+                                : p >= 0 && p < A.E * NF && p % N == N - 1 && wk == (int32_t)(((p - k) << 1) | (w & 1));
+    if (!whole) {
+      atomicExch(&A.status[ST_STATUS], kStatusBounds);
+      atomicExch(&A.status[ST_BAD_INDEX], wk);
+      off = (int64_t)e * 2 * NF + ed * N;
+      return kFwL | kFwWall;
+    }
+  }
+#endif
   off = (int64_t)(p / NF) * 2 * NF + p % NF;
   return (w & 1) | (p == own ? kFwWall : 0);
 }
