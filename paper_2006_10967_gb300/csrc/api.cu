@@ -1090,6 +1090,20 @@ extern "C" int fr_mass_integral(fr_field* f, int which, double* out_host, void* 
 }
 
 namespace {
+// Whether a kernel may use p as an array of doubles: memory of the current
+// device on a boundary of 8 bytes.  A copy takes more (any byte boundary, the
+// memory of a device without peer access).
+bool kernel_may_use(const void* p) {
+  cudaPointerAttributes at{};
+  int dev = -1;
+  if (reinterpret_cast<uintptr_t>(p) % sizeof(double) != 0) return false;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == dev;
+}
+
 int copy_field(fr_field* f, int which, void* dst, const void* src, bool to_state, cudaMemcpyKind kind,
                cudaStream_t s) {
   const size_t NU = f->nu, E = f->E;
@@ -1098,8 +1112,9 @@ int copy_field(fr_field* f, int which, void* dst, const void* src, bool to_state
     else CK(cudaMemcpyAsync(dst, f->args.psi0, E * NU * 8, kind, s));
     return FR_OK;
   }
-  if (kind == cudaMemcpyDeviceToDevice) {
-    // one pass between the state and the caller's device array
+  if (kind == cudaMemcpyDeviceToDevice && kernel_may_use(to_state ? src : dst)) {
+    // one pass between the state and the caller's device array; other pointers
+    // go through copies below
     int grid;
     launch_elementwise_grid(f->E * f->nu, &grid);
     const int mixed = f->precision == FR_MIXED;

@@ -227,3 +227,38 @@ def test_triangles_on_the_same_side_of_their_edge(G, order):
         assert f.sync() == 0
     for which in (0, 1):
         assert _rel(F.get(which), D.get(which)) < 1e-5
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+@pytest.mark.parametrize("etype,order,ns", [("quad", 3, (7, 5)), ("hex", 2, (3, 4, 3))])
+def test_device_copies_take_any_byte_boundary(G, precision, etype, order, ns):
+    """get_device and set_device on arrays off a boundary of 8 bytes (only
+    copies can serve them) move what they move on a boundary; a captured
+    get_device replays."""
+    import ctypes as C
+
+    import torch
+    w, mesh = _workload(etype, order, ns, 0.0, "uniform", True)
+    M = G.Mesh.from_synthetic(mesh, order)
+    F, R = [G.Field(M, G.make_params(w, precision), ic=w.circle) for _ in range(2)]
+    F.step(1)
+    n = M.info.n_elems * M.info.nu
+    raw = torch.zeros(n * 8 + 16, dtype=torch.uint8, device="cuda")
+    L, s = G.lib(), C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    for off in (0, 4, 1):
+        for which in (0, 1, 2):
+            p = C.c_void_p(raw.data_ptr() + off)
+            assert L.fr_field_get_device(F.handle, which, p, s) == 0
+            got = raw[off:off + n * 8].cpu().numpy().tobytes()
+            assert got == F.get(which).tobytes()
+            R.set(which, np.zeros(M.shape))
+            assert L.fr_field_set_device(R.handle, which, p, s) == 0
+            assert R.get(which).tobytes() == got
+    out = torch.empty(M.shape, dtype=torch.float64, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        F.get_device(0, out)
+    F.step(1)
+    g.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(out.cpu().numpy(), F.get(0))
