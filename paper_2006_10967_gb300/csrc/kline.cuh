@@ -348,7 +348,9 @@ __global__ void k_vel_tab(const KArgs A) {
     const double xi = j < N ? A.cd.ops.x[j] : (j == N ? -1.0 : 1.0);
     const double x = k[0] + k[1 + b] * xi;
     double a = 1.0, f = 1.0;
-    if (kind == 1 || kind == 2) {  // Rider-Kothe (in 3D constant along axis 2), LeVeque
+    if (kind == 2 && DIM == 2) {  // LeVeque's field is a 3D one: zero in 2D, as in velocity()
+      a = f = 0.0;
+    } else if (kind == 1 || kind == 2) {  // Rider-Kothe (in 3D constant along axis 2), LeVeque
       if (kind == 2 || b < 2) {
         double s, c;
         sincospi(x, &s, &c);

@@ -262,3 +262,18 @@ def test_device_copies_take_any_byte_boundary(G, precision, etype, order, ns):
     g.replay()
     torch.cuda.synchronize()
     assert np.array_equal(out.cpu().numpy(), F.get(0))
+
+
+@pytest.mark.parametrize("kind", ["uniform", "rider_kothe", "leveque", "rotation"])
+@pytest.mark.parametrize("etype,order,ns", [("quad", 3, (6, 5)), ("quad", 4, (6, 5)), ("hex", 2, (3, 4, 3))])
+@pytest.mark.parametrize("jitter", [0.0, 0.1])
+def test_every_velocity_on_every_mesh_matches_fp64(G, kind, etype, order, ns, jitter):
+    """The velocity factors of axis-aligned elements give the FP64 path's
+    velocity for each kind in 2D and in 3D (LeVeque's field is zero in 2D)."""
+    w = _workload(etype, order, ns, jitter, "uniform", True)[0].with_(velocity=S.Velocity(
+        kind, a=(0.6, 0.4, 0.3) if kind == "uniform" else (0.5, 0.5, 0.0), T=3.0 if kind != "rotation" else 0.0))
+    M = G.Mesh.from_synthetic(w.mesh(), order)
+    a, b = [G.Field(M, G.make_params(w, p, pseudo_fixed=True), ic=w.circle).rhs(0.3).cpu().numpy()
+            for p in ("mixed", "fp64")]
+    for f in (0, 1):
+        assert np.abs(a[f] - b[f]).max() <= 1e-4 * np.abs(b).max()
