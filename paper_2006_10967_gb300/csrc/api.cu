@@ -1022,9 +1022,10 @@ extern "C" int fr_field_init_batch(const fr_mesh* m, const fr_params* prm, int n
     return FR_ECUDA;
   }
   f->args.ep = f->ep_region;
+  // the tables hold params->vel, the instances' own velocities are in the point cache
+  f->args.vtab = nullptr;
+  f->args.vtabd = nullptr;
   if (use_line_kernels(*m, *prm)) {
-    // the table holds params->vel, the instances' own velocities are in the point cache
-    f->args.vtab = nullptr;
     if (!set_line_kernels(*m, !all_diagonal(*m), false, prm->normal == FR_NORMAL_PHI, &f->ks)) {
       fr_field_destroy(f);
       return FR_ECUDA;

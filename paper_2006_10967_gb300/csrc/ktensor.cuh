@@ -463,8 +463,9 @@ __device__ __forceinline__ void kb_tensor_body(const KArgs& A, const int blk) {
   __syncthreads();
   const T gfac = gfac_s;
   // separable velocity: per-axis tables of the elements with a diagonal map
-  // (read after the first axis pass's barrier)
-  const bool sepk = MODE == 0 && vel_separable(BC.vel.kind);
+  // (read after the first axis pass's barrier); a batch's instances have their
+  // own velocities, in the point cache alone
+  const bool sepk = MODE == 0 && !A.ep && vel_separable(BC.vel.kind);
   if (sepk && !tabs)
     for (int t = tid; t < ne * DIM * NT; t += blockDim.x) {
       const int el = t / (DIM * NT), r = t % (DIM * NT), c = r / NT, j = r % NT;

@@ -142,3 +142,51 @@ def test_group_rejects_unsupported_fields(G):
     b = G.batch_from_workloads(ws[1:], precision="mixed")[0][1]
     with pytest.raises(G.FRError):
         G.Group([a, b])          # two fields of one order
+
+
+def _regular_instances(etype, p, kinds):
+    """Instances on axis-aligned meshes, each with its own steady velocity."""
+    dim = 3 if etype == "hex" else 2
+    out = []
+    for i, kind in enumerate(kinds):
+        n = 3 + i
+        h = 1.0 / n
+        mesh = (lambda n=n: S.hex_grid(n, n, n)) if dim == 3 else (lambda n=n: S.quad_grid(n, n))
+        vel = S.Velocity(kind, a=((0.6, 0.4, 0.3), (-0.3, 0.5, 0.2), (0.5, 0.4, 0.0))[i])
+        w = S.Workload(f"r{i}", mesh, p, vel, S.Circle((0.45, 0.5, 0.55)[:dim], 0.25, 3 * p / (4 * h)), t_end=1.0, h=h)
+        w.eps, w.nu_max = 0.06 * h / p, 0.15 * h / p
+        w.pseudo_dtau = 0.1 * h / (p + 1)
+        w.dt = 0.05 * h / (p + 1)
+        w.n_precond, w.pseudo_kmax = 3, 2
+        out.append(w)
+    return out
+
+
+@pytest.mark.parametrize("kinds", [("uniform", "uniform", "rotation"), ("rotation", "rider_kothe", "uniform")])
+@pytest.mark.parametrize("etype,p,precision", [("quad", 2, "fp64"), ("quad", 3, "mixed"), ("quad", 4, "fp64"),
+                                               ("hex", 2, "fp64"), ("hex", 3, "mixed"), ("hex", 5, "mixed")])
+def test_batch_instances_on_regular_meshes_keep_their_velocities(G, etype, p, precision, kinds):
+    ws = _regular_instances(etype, p, kinds)
+    (_, F, ranges), = G.batch_from_workloads(ws, precision=precision, pseudo_fixed=True)
+    F.step(4)
+    assert F.sync() == 0
+    for w, (b, e) in zip(ws, ranges):
+        R = G.Field(G.Mesh.from_synthetic(w.mesh(), p), G.make_params(w, precision, pseudo_fixed=True), ic=w.circle)
+        R.step(4)
+        for which in (0, 1):
+            ref = R.get(which)
+            assert np.abs(F.get(which)[b:e] - ref).max() < (1e-12 if precision == "fp64" else 2e-5) * np.abs(ref).max()
+
+
+def test_group_launch_keeps_the_instances_velocities(G):
+    ws = _regular_instances("quad", 2, ("uniform", "rotation", "uniform")) + \
+        _regular_instances("quad", 3, ("rotation", "uniform", "uniform"))
+    fa = G.batch_from_workloads(ws, precision="mixed", pseudo_fixed=True)
+    fb = G.batch_from_workloads(ws, precision="mixed", pseudo_fixed=True)
+    G.Group([F for _, F, _ in fa]).step(5)
+    for (_, Fa, _), (_, Fb, _) in zip(fa, fb):
+        Fb.step(5)
+        assert Fa.sync() == 0 and Fb.sync() == 0
+        for which in (0, 1):
+            a, b = Fa.get(which), Fb.get(which)
+            assert np.abs(a - b).max() <= 2e-6 * np.abs(b).max()
