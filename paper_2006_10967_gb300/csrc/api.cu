@@ -830,7 +830,7 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
     l = (float)(v - (double)h);
   };
   A.prm.ramp_lo = (float)(std::pow(10.0, prm->s0 - prm->kappa) * (1.0 - 1e-5));
-  const double rs = M_PI / (4.0 * prm->kappa);
+  const double rs = M_PI / (4.0 * std::max(prm->kappa, 1e-30));  // narrower ramps are a step already
   split(-rs * (prm->s0 - prm->kappa), A.prm.ramp_c0h, A.prm.ramp_c0l);
   split(rs * std::log10(2.0), A.prm.ramp_c1h, A.prm.ramp_c1l);
   split(rs * 2.0 * std::log10(std::exp(1.0)), A.prm.ramp_c2h, A.prm.ramp_c2l);

@@ -42,6 +42,32 @@ __device__ __forceinline__ float2 ff_div(float2 a, float2 b) {
   return make_float2(h, l - (h - q));
 }
 
+// The power of two that brings the largest magnitude of an element's modal
+// coefficients (given by its bits) to [1, 4): the ratio of the energies does not
+// depend on it, the scaling is exact, and no square of a coefficient of any
+// size overflows or is lost beside the largest one's.
+__device__ __forceinline__ float energy_scale(unsigned bits) {
+  return __int_as_float((int)(254u - min(bits >> 23, 253u)) << 23);
+}
+__device__ __forceinline__ unsigned abs_bits(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+// Maximum over the LN lanes of an element; every lane gets it.  first: the element's first lane.
+template <int LN>
+__device__ __forceinline__ unsigned line_max(unsigned v, int l, int first) {
+  if constexpr ((LN & (LN - 1)) == 0) {
+#pragma unroll
+    for (int o = LN / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+  } else {
+    constexpr int TOP = LN > 16 ? 16 : LN > 8 ? 8 : LN > 4 ? 4 : LN > 2 ? 2 : 1;
+#pragma unroll
+    for (int o = TOP; o > 0; o >>= 1) {
+      const unsigned t = __shfl_down_sync(0xffffffffu, v, o);
+      if (l + o < LN) v = max(v, t);
+    }
+    return __shfl_sync(0xffffffffu, v, first);
+  }
+}
+
 // nu_s of Eqs. resolutionIndicator, nu_s from the energies of the modes below
 // and at the top degree, evaluated in float-float.  With r = hi / (lo + hi) and
 // z = (pi / 2) (log10 r - (s0 - kappa)) / (2 kappa), the ramp
@@ -56,7 +82,8 @@ __device__ __forceinline__ float sensor_nu(const PhysPrm& P, float2 lo, float2 h
   const float tot = lo.x + hi.x;
   if (!(tot > 0.f) || !(hi.x > 0.f)) return 0.f;
   if (hi.x < P.ramp_lo * tot) return 0.f;  // most elements: flat or resolved
-  const float2 r = ff_div(hi, ff_add(lo, hi));
+  float2 r = ff_div(hi, ff_add(lo, hi));
+  if (r.x < 0x1p-126f) r = make_float2(0x1p-126f, 0.f);  // a ramp that reaches below the floats
   // r = m 2^k
   int k = (__float_as_int(r.x) >> 23) - 127;
   float mh = __int_as_float((__float_as_int(r.x) & 0x007fffff) | 0x3f800000);
@@ -255,9 +282,13 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
   //      lane's line holds modes (its two indices, 0..N-1)) and at it
   float nu;
   {
-    // scaled by 2^20 (exact): squares of coefficients from 1e-18 to 1e12 neither overflow nor lose their low parts
+    const int src = L::FULL ? es * LN : min(es * LN, 31);
+    unsigned big = 0;
 #pragma unroll
-    for (int m = 0; m < N; ++m) cm[m] *= 0x1p20f;
+    for (int m = 0; m < N; ++m) big = max(big, abs_bits(cm[m]));
+    const float unit = energy_scale(line_max<LN>(big, l, src));
+#pragma unroll
+    for (int m = 0; m < N; ++m) cm[m] *= unit;
     const bool top = DIM == 3 ? (l % N == N - 1 || l / N == N - 1) : l == N - 1;
     float2 b = make_float2(0.f, 0.f), t;
 #pragma unroll
@@ -272,7 +303,6 @@ __global__ void __launch_bounds__(WPB * 32, (!GEN ? 24 : DIM == 3 ? 16 : 20) / W
     float2 hi = top ? ff_add(t, b) : t, lo = top ? make_float2(0.f, 0.f) : b;
     if (!lane_ok) hi = lo = make_float2(0.f, 0.f);
     line_tree<LN>(lo, hi, l);
-    const int src = L::FULL ? es * LN : min(es * LN, 31);
     const float2 h0 = make_float2(__shfl_sync(0xffffffffu, hi.x, src + LineTree<LN>::LB),
                                   __shfl_sync(0xffffffffu, hi.y, src + LineTree<LN>::LB));
     nu = 0.f;

@@ -230,13 +230,17 @@ __global__ void __launch_bounds__(TriReg<P>::TB) kb_trir(const __grid_constant__
       tri_fence();
       tri_acc<NPU>(Vt + j * NPU, u[0][j], c);
     }
+    unsigned big = 0;
+#pragma unroll
+    for (int i = 0; i < NU; ++i) big = max(big, abs_bits(pair_at(c, i)));
+    const float unit = energy_scale(big);
     float2 lo = make_float2(0.f, 0.f), hi = lo;
     int m = 0;
 #pragma unroll
     for (int i = 0; i <= P; ++i)
 #pragma unroll
       for (int j = 0; j <= P - i; ++j, ++m) {
-        const float v = pair_at(c, m) * 0x1p20f;  // as in kbp_line
+        const float v = pair_at(c, m) * unit;
         const float s = __fmul_rn(v, v);
         float2& t = i + j == P ? hi : lo;
         t = ff_add(t, make_float2(s, __fmaf_rn(v, v, -s)));

@@ -277,3 +277,29 @@ def test_every_velocity_on_every_mesh_matches_fp64(G, kind, etype, order, ns, ji
             for p in ("mixed", "fp64")]
     for f in (0, 1):
         assert np.abs(a[f] - b[f]).max() <= 1e-4 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("scale", [1e-25, 1e-18, 1.0, 1e13, 1e16])
+@pytest.mark.parametrize("etype,order,ns,jitter", [("quad", 3, (6, 5), 0.0), ("quad", 4, (6, 5), 0.1), ("quad", 1, (6, 5), 0.0),
+                                                   ("hex", 2, (3, 4, 3), 0.1), ("hex", 3, (3, 4, 3), 0.0),
+                                                   ("hex", 4, (3, 2, 2), 0.0), ("tri", 2, (6, 5), 0.0), ("tri", 4, (4, 5), 0.0)])
+def test_viscosity_does_not_depend_on_the_size_of_psi(G, etype, order, ns, jitter, scale):
+    """The resolution indicator is a ratio of energies: the preconditioning's
+    rate with psi0 = 0 (no source) follows FP64 for psi of any size whose
+    squared gradient is a float."""
+    w, mesh = _workload("quad" if etype == "tri" else etype, order, ns, jitter, "uniform", True)
+    if etype == "tri":
+        mesh = S.tri_split(*ns, periodic=(False, False))
+    M = G.Mesh.from_synthetic(mesh, order)
+    x = M.solution_points()
+    psi = scale * np.sin(9 * x[..., 0] + 1) * np.cos(11 * x[..., 1])
+
+    def rate(precision, nu_max):
+        F = G.Field(M, G.make_params(w, precision, pseudo_fixed=True, nu_max=nu_max), ic=w.circle, precondition=False)
+        F.set(1, psi)
+        F.set(2, np.zeros(M.shape))
+        return F.rhs_pseudo().cpu().numpy()
+
+    ref = rate("fp64", w.nu_max)
+    assert _rel(rate("fp64", 2 * w.nu_max), ref) > 1e-3  # the viscosity's share of the rate
+    assert _rel(rate("mixed", w.nu_max), ref) < 1e-4
