@@ -334,13 +334,6 @@ int check_params(const fr_params* p) {
   } while (0)
 
 // ---- small kernels ---------------------------------------------------------
-// float -> double by moving the bits: exact, and on the integer units, where
-// the conversion instruction takes the FP64 pipe (2 lanes a clock).
-__device__ __forceinline__ double widen(float x) {
-  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu, e = m >> 23;
-  if (e - 1u < 254u) return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
-  return m == 0 ? __hiloint2double((int)u, 0) : (double)x;  // zero; subnormal, infinite, NaN
-}
 // The solution u is double in the FP64 path and a float-float pair
 // (hi, lo) in the mixed path; these helpers read and write one value.
 __device__ __forceinline__ double u_get(const KArgs& A, int mixed, int64_t g) {

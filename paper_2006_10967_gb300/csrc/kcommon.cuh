@@ -96,7 +96,6 @@ constexpr int kMetricRec = 16;
 
 struct RKConstF {
   float half_dt, dt, dt6;
-  float r2h, r2l;  // 1 / dt^2 as a float-float pair
   double rdt, ddt, ddt6;
 };
 
@@ -108,8 +107,6 @@ __host__ __device__ __forceinline__ RKConstF rk_const(double dt) {
   c.rdt = 1.0 / dt;
   c.ddt = dt;
   c.ddt6 = dt / 6.0;
-  c.r2h = (float)(c.rdt * c.rdt);
-  c.r2l = (float)(c.rdt * c.rdt - (double)c.r2h);
   return c;
 }
 
@@ -431,6 +428,13 @@ __device__ __forceinline__ float2 ff_add(float2 a, float2 b) {
   const float hi = s + e;
   return make_float2(hi, e - (hi - s));
 }
+// float -> double by moving the bits: exact, and on the integer units, where
+// the conversion instruction takes the FP64 pipe (2 lanes a clock).
+__device__ __forceinline__ double widen(float x) {
+  const unsigned u = __float_as_uint(x), m = u & 0x7fffffffu, e = m >> 23;
+  if (e - 1u < 254u) return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
+  return m == 0 ? __hiloint2double((int)u, 0) : (double)x;  // zero; subnormal, infinite, NaN
+}
 // (pair) x (float), exact product of the high parts by FMA
 __device__ __forceinline__ float2 ff_mul(float2 a, float b) {
   const float p = a.x * b;
@@ -571,7 +575,8 @@ __device__ __forceinline__ void pseudo_rms_finish(const KArgs& A, double partial
   __threadfence();
   double s = 0.0;
   // sixteen loads in flight a thread: with one at a time the last block spent
-  // 48 us on the 8,000 partials of 64,000 hexahedra
+  // 48 us on 8,000 partials (64,000 hexahedra, a partial a block of eight; the
+  // line kernels' resident grid leaves 912)
   int b = threadIdx.x;
   for (; b + 15 * (int)blockDim.x < (int)gridDim.x; b += 16 * blockDim.x) {
     double v[16];

@@ -5,8 +5,10 @@
 // The block-wide kernels spent most of their time in FP64: the modal energies
 // of the resolution indicator as one thread's serial sum per element, and nine
 // instructions a point for the pseudo-time residual, on a pipe of 2 lanes a
-// clock.  Here both are float-float sums over the lanes, and the indicator's
-// logarithm and sine are evaluated in float-float too (sensor_nu).
+// clock.  Here the energies are float-float sums over the lanes, the indicator's
+// logarithm and sine are evaluated in float-float (sensor_nu), and of the
+// residual only the sum of squares is FP64, two instructions a point: in
+// float-float its squares would leave the floats' range with psi.
 #pragma once
 #include "kline.cuh"
 
@@ -523,7 +525,7 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
   float2* U = reinterpret_cast<float2*>(A.u);
   const float* fcA = reinterpret_cast<const float*>(A.fc);
   const LineOps& O = A.lo;
-  [[maybe_unused]] float2 sum = make_float2(0.f, 0.f);  // stage 4: squared residuals
+  [[maybe_unused]] double sum = 0.0;  // stage 4: squared residuals
 
 #pragma unroll 1
   for (int64_t e0 = ((int64_t)blockIdx.x * WPB + warp) * EPW; e0 < A.E;
@@ -614,7 +616,7 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
       for (int j = 0; j < N; ++j) u[j] = reinterpret_cast<const float2*>(in + 2 * K::C)[rl + j];
   }
 
-  [[maybe_unused]] float2 sh = dup2(0.f), sl = dup2(0.f);  // stage 4: sum of the squared changes
+  [[maybe_unused]] double sq = 0.0;  // stage 4: sum of the squared changes
   if constexpr (SF >= 1) {
     const RKConstF& rk = A.ep ? A.ep[e].rkp : A.rk;
     const int lc1 = DIM == 3 ? l % N : l, lc2 = DIM == 3 ? l / N : 0;
@@ -654,7 +656,6 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
         rdj = rcp2(metric_all<DIM>(R0 + K::O_GEO + es * L::S::NG, xi, Sm));
       }
       const float2 R = mul2(make_float2(-y[p].x, -y[p].y), rdj);
-      float dh[2] = {0.f, 0.f}, dl[2] = {0.f, 0.f};
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
         const int j = 2 * p + i;
@@ -677,22 +678,15 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
           const float e2 = two_sum_lo(uu.x, inc, s2) + uu.y;
           yn = s2 + e2;
           const float lo = e2 - (yn - s2);
-          // the change as a float-float value
+          // the change as a float-float value, squared in FP64
           const float ch = yn - uu.x;
-          dl[i] = two_sum_lo(yn, -uu.x, ch) + (lo - uu.y);
-          dh[i] = ch;
+          const double d = widen(ch) + widen(two_sum_lo(yn, -uu.x, ch) + (lo - uu.y));
+          sq = fma(d, d, sq);
           u[j] = make_float2(yn, lo);
         }
         bad = __fmaf_rn(yn, 0.f, bad);
         if (i) y[p].y = yn;
         else y[p].x = yn;
-      }
-      if constexpr (SF == 4) {
-        // (dh + dl)^2, error-free in the leading product
-        const float2 h = make_float2(dh[0], dh[1]), lo = make_float2(dl[0], dl[1]);
-        const float2 sq = mul2(h, h);
-        sl = add2(sl, fma2(mul2(dup2(2.f), h), lo, fma2(h, h, make_float2(-sq.x, -sq.y))));
-        sum_add(sh, sl, sq);
       }
     }
     if (act && bad != 0.f) atomicExch(&A.status[ST_STATUS], -4);
@@ -760,23 +754,18 @@ __global__ void __launch_bounds__(WPB * 32, 24 / WPB) kap_line(const KArgs A) {
   if constexpr (SF == 4) {
     // 1 / dtau^2 times the lane's squared changes
     const RKConstF& rk = A.ep ? A.ep[e].rkp : A.rk;
-    if (act) sum = ff_add(sum, ff_mul2(ff_add(make_float2(sh.x, sl.x), make_float2(sh.y, sl.y)), make_float2(rk.r2h, rk.r2l)));
+    if (act) sum = fma(sq, rk.rdt * rk.rdt, sum);
     __syncwarp();  // the tile's buffers are read
   }
   }  // tiles
 
   if constexpr (SF == 4) {
-    // RMS of the pseudo-time residual: float-float to the warp's sum, FP64 over the block
+    // RMS of the pseudo-time residual
     __shared__ double part[WPB];
     __shared__ double red_sh[32];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      float2 t;
-      t.x = __shfl_xor_sync(0xffffffffu, sum.x, o);
-      t.y = __shfl_xor_sync(0xffffffffu, sum.y, o);
-      sum = ff_add(sum, t);
-    }
-    if (lane == 0) part[warp] = (double)sum.x + (double)sum.y;
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) part[warp] = sum;
     __syncthreads();
     double s = 0.0;
     if (threadIdx.x == 0)

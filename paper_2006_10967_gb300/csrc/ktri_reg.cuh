@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
 #pragma unroll
   for (int i = 0; i < NPU; ++i)
     y[i] = make_float2(2 * i < NU ? yr[2 * i < NU ? 2 * i : 0] : 0.f, 2 * i + 1 < NU ? yr[2 * i + 1 < NU ? 2 * i + 1 : 0] : 0.f);
-  [[maybe_unused]] float2 sh = make_float2(0.f, 0.f);  // MODE 1 stage 4: squared changes
+  [[maybe_unused]] double sq = 0.0;  // MODE 1 stage 4: squared changes
   if constexpr (SF >= 1) {
     // ---- lift of minus the partner's flux at R points; flux balance
     float2 bal = make_float2(0.f, 0.f);
@@ -539,9 +539,9 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
             Ssum = ff_add(Ssum, ff_mul(wd, inc));
           }
         } else {
-          const float h = yn - uu.x, l = two_sum_lo(yn, -uu.x, h) + (lo - uu.y);
-          const float sq = __fmul_rn(h, h);
-          sh = ff_add(sh, make_float2(sq, __fmaf_rn(2.f * h, l, __fmaf_rn(h, h, -sq))));
+          const float h = yn - uu.x;
+          const double d = widen(h) + widen(two_sum_lo(yn, -uu.x, h) + (lo - uu.y));
+          sq = fma(d, d, sq);
         }
       }
       bad = __fmaf_rn(yn, 0.f, bad);
@@ -604,16 +604,10 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
   if constexpr (MODE == 1 && SF == 4) {
     __shared__ double part[TriReg<P>::TB / 32];
     __shared__ double red_sh[32];
-    float2 v = ff_mul2(sh, make_float2(A.rk.r2h, A.rk.r2l));
-    if (!act) v = make_float2(0.f, 0.f);
+    double v = act ? sq * (A.rk.rdt * A.rk.rdt) : 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      float2 t;
-      t.x = __shfl_xor_sync(0xffffffffu, v.x, o);
-      t.y = __shfl_xor_sync(0xffffffffu, v.y, o);
-      v = ff_add(v, t);
-    }
-    if (lane == 0) part[warp] = (double)v.x + (double)v.y;
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) part[warp] = v;
     __syncthreads();
     double s = 0.0;
     for (int w = 0; w < TriReg<P>::TB / 32; ++w) s += part[w];

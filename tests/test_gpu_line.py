@@ -303,3 +303,42 @@ def test_viscosity_does_not_depend_on_the_size_of_psi(G, etype, order, ns, jitte
     ref = rate("fp64", w.nu_max)
     assert _rel(rate("fp64", 2 * w.nu_max), ref) > 1e-3  # the viscosity's share of the rate
     assert _rel(rate("mixed", w.nu_max), ref) < 1e-4
+
+
+@pytest.mark.parametrize("scale", [1e-25, 1.0, 1e16])
+@pytest.mark.parametrize("etype,order,ns,jitter", [("quad", 3, (6, 5), 0.0), ("quad", 4, (6, 5), 0.1),
+                                                   ("hex", 2, (3, 4, 3), 0.1), ("hex", 3, (3, 4, 3), 0.0),
+                                                   ("tri", 3, (6, 5), 0.0)])
+def test_pseudo_residual_does_not_depend_on_the_size_of_psi(G, etype, order, ns, jitter, scale):
+    w, mesh = _workload("quad" if etype == "tri" else etype, order, ns, jitter, "uniform", True)
+    if etype == "tri":
+        mesh = S.tri_split(*ns, periodic=(False, False))
+    M = G.Mesh.from_synthetic(mesh, order)
+    x = M.solution_points()
+    rms = []
+    for p in ("mixed", "fp64"):
+        F = G.Field(M, G.make_params(w, p, pseudo_fixed=True), ic=w.circle, precondition=False)
+        F.pseudo_begin()
+        F.set(1, scale * np.sin(9 * x[..., 0] + 1) * np.cos(11 * x[..., 1]))
+        F.set(2, np.zeros(M.shape))
+        for s in (1, 2, 3, 4):
+            F.pseudo_stage(s)
+        assert F.sync() == 0
+        rms.append(F.stats()["last_pseudo_rms"])
+    assert rms[1] > 0 and abs(rms[0] / rms[1] - 1) < 1e-4
+
+
+@pytest.mark.parametrize("etype,order,ns,jitter", [("hex", 3, (21, 19, 19), 0.0), ("hex", 2, (23, 22, 22), 0.1),
+                                                   ("quad", 4, (149, 148), 0.1), ("tri", 2, (96, 90), 0.0)])
+def test_preconditioning_of_meshes_past_one_grid(G, etype, order, ns, jitter):
+    """Just past the resident grid of the last stage's update a warp takes a
+    second, partly empty tile; triangles leave the reduction more partials than
+    sixteen rounds of a block's loads."""
+    w, mesh = _workload("quad" if etype == "tri" else etype, order, ns, jitter, "uniform", True)
+    if etype == "tri":
+        mesh = S.tri_split(*ns, periodic=(False, False))
+    M = G.Mesh.from_synthetic(mesh, order)
+    F, D = [G.Field(M, G.make_params(w, p, pseudo_fixed=True), ic=w.circle) for p in ("mixed", "fp64")]
+    assert F.stats()["last_pseudo_iters"] == D.stats()["last_pseudo_iters"] == 3
+    assert abs(F.stats()["last_pseudo_rms"] / D.stats()["last_pseudo_rms"] - 1) < 1e-4
+    assert _rel(F.get(1), D.get(1)) < 1e-5
