@@ -22,6 +22,7 @@ struct Layout {
   size_t status, dstate, red, geo, geof, fnbr, wdet, ustg, u, acc, rp, tr, fc, psi0, xfer, vsu, vsf, tacc, wdetf, ep, mcg;
   size_t tri_d, tri_f, tri_high;  // dense triangle operators (double, float), mode mask
   size_t tri_pack;                // their packed form (TriPack)
+  size_t triw;                    // triangles: quadrature areas (KArgs.triw)
   size_t wphys;                   // triangles: physical edge quadrature weight per flux point (float-float)
   size_t ffw;                     // hexahedra: face words (KArgs.ffw)
   size_t vtab64;                  // FP64 tensor fields with a separable velocity: its tables (KArgs.vtabd)
@@ -252,6 +253,7 @@ Layout make_layout(const fr_mesh& m, const fr_params& prm, int max_blocks) {
     L.tri_f = take(nops * sizeof(float));
     L.tri_high = take(NU);
     L.tri_pack = take(TriPack(m.order).size * sizeof(float));
+    L.triw = take(E * sizeof(double));
     L.wphys = take(E * NF * 2 * sizeof(float));
   }
   L.total = off;
@@ -851,7 +853,15 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
   up(L.geof, geof.data(), geof.size() * sizeof(float));
   std::vector<double> trid;
   std::vector<float> trif, tripack;
+  std::vector<double> triw;
+  A.triw = nullptr;
   if (m->etype == FR_TRI) {
+    triw.assign(m->E, 0.0);
+    for (int64_t e = 0; e < m->E; ++e)
+      for (int i = 0; i < m->nu; ++i)
+        triw[e] += (double)wdetf[2 * (e * m->nu + i)] + (double)wdetf[2 * (e * m->nu + i) + 1];
+    up(L.triw, triw.data(), triw.size() * sizeof(double));
+    A.triw = reinterpret_cast<const double*>(b + L.triw);
     pack_tri(m->tri, trid);
     pack_tri(m->tri, trif);
     up(L.tri_d, trid.data(), trid.size() * sizeof(double));

@@ -480,8 +480,9 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
       for (int k = 0; k < N; ++k) F[ed][k] = (MODE == 0 || !isl) ? b[k * st] : 0.f;
     }
   }
-  double ta = 0.0;
+  double ta = 0.0, W = 1.0;
   if (SF >= 2 && cons) ta = A.tacc[e * 2 + f];
+  if (SF == 4 && cons) W = __ldg(A.triw + e);
   cp_async_wait_all();
   __syncthreads();
   float* yr = yb + (el * 2 + f) * NU;
@@ -513,7 +514,7 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
     float2* sr = reinterpret_cast<float2*>(sb) + (el * 2 + f) * NU;
     float* ar = ab + (el * 2 + f) * NU;
     float bad = 0.f;
-    float2 Ssum = make_float2(0.f, 0.f), W = Ssum;
+    float2 Ssum = make_float2(0.f, 0.f);
 #pragma unroll
     for (int j = 0; j < NU; ++j) {
       const float Rj = -pair_at(y, j) * rdj;
@@ -535,7 +536,6 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
         if constexpr (MODE == 0) {
           if (cons) {
             const float2 wd = reinterpret_cast<const float2*>(wb)[el * NU + j];
-            W = ff_add(W, wd);
             Ssum = ff_add(Ssum, ff_mul(wd, inc));
           }
         } else {
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
       if (cons) {
         const double Te = -((double)bal.x + (double)bal.y);
         const double tgt = A.rk.ddt6 * (ta + Te);
-        const double d = (tgt - ((double)Ssum.x + (double)Ssum.y)) / ((double)W.x + (double)W.y);
+        const double d = (tgt - ((double)Ssum.x + (double)Ssum.y)) / W;
         const float dh = (float)d, dl = (float)(d - (double)dh);
 #pragma unroll
         for (int j = 0; j < NU; ++j) {
