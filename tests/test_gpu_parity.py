@@ -500,6 +500,43 @@ def test_tile_variants_march_with_the_oracle(G, case, variant):
         assert _rel(F.get(fld), F0.get(fld)) < 1e-6
 
 
+@pytest.mark.parametrize("case", ["quad_periodic_jitter_p3", "quad_walls_jitter_p4", "hex_periodic_jitter_p3",
+                                  "hex_rotated_walls_p3"])
+@pytest.mark.parametrize("variant", [1, 2, 3])
+def test_block_wide_tile_variants_march_with_the_oracle(G, case, variant):
+    """The same without the velocity cache, where the fields run on the
+    block-wide kernels that the variants' tiles belong to (with the cache,
+    quads and hexes of p <= 4 take the line kernels under every number)."""
+    w = CASES[case]()
+    sol, F = _pair(G, w, precision="mixed", variant=variant, vel_cache=False)
+    _, F1 = _pair(G, w, precision="mixed", variant=variant, vel_cache=False)
+    _, F0 = _pair(G, w, precision="mixed", variant=0, vel_cache=False)
+    for f in (F, F1, F0):
+        f.step(6)
+    sol.step(6)
+    assert F.sync() == 0
+    assert _rel(F.get(0), sol.phi.numpy()) < 1e-5
+    assert np.array_equal(F.get(0), F1.get(0)) and np.array_equal(F.get(1), F1.get(1))
+    for fld in (0, 1):
+        assert _rel(F.get(fld), F0.get(fld)) < 1e-6
+
+
+@pytest.mark.parametrize("variant", [1, 2, 3])
+@pytest.mark.parametrize("vel_cache", [True, False])
+def test_block_wide_tile_variants_of_hexes_of_order_5(G, variant, vel_cache):
+    w = _workload(lambda: S.hex_grid(3, periodic=(True, True, True), jitter=0.1, seed=5, shuffle_seed=3), 5,
+                  S.Velocity("leveque", T=3.0), S.Circle((0.45, 0.5, 0.4), 0.3, 3 * 5 / (4 / 3)), 1 / 3)
+    sol, F = _pair(G, w, precision="mixed", variant=variant, vel_cache=vel_cache)
+    _, F0 = _pair(G, w, precision="mixed", variant=0, vel_cache=vel_cache)
+    for f in (F, F0):
+        f.step(3)
+    sol.step(3)
+    assert F.sync() == 0
+    assert _rel(F.get(0), sol.phi.numpy()) < 1e-5
+    for fld in (0, 1):
+        assert _rel(F.get(fld), F0.get(fld)) < 1e-6
+
+
 def test_autotuner_measures_every_variant(G):
     from paper_2006_10967_gb300 import tune
     w = CASES["tri_delaunay_p3"]()
