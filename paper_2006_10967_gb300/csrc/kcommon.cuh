@@ -184,6 +184,23 @@ __device__ __forceinline__ int32_t partner(const KArgs& A, int32_t w, int32_t ow
   return p;
 }
 
+// A triangle edge of N points (connectivity words own .. own + N - 1 of n) is
+// whole if it is a wall (every point its own partner, on the L side) or all its
+// words lead, last to first, to the points of one edge with one L flag; its
+// partner's points are then p, p - 1, .. p - N + 1 with p from the first word.
+// Returns the first word that breaks the edge, -1 for a whole one.
+template <int N>
+__host__ __device__ inline int tri_edge_broken(const int32_t* fnbr, int64_t n, int32_t own) {
+  const int32_t w = fnbr[own], p = w >> 1;
+  for (int k = 0; k < N; ++k) {
+    const bool whole = p == own ? fnbr[own + k] == (int32_t)((uint32_t)(own + k) << 1 | 1)
+                                : p >= 0 && p < n && p % N == N - 1 &&
+                                      fnbr[own + k] == (int32_t)((uint32_t)(p - k) << 1 | (uint32_t)(w & 1));
+    if (!whole) return k;
+  }
+  return -1;
+}
+
 // Hexahedra carry one word pair per face (KArgs.ffw) in place of one
 // connectivity word per flux point.  Face point (i, j) (the line index
 // i + N j of the two other axes, lowest fastest) meets the partner's face

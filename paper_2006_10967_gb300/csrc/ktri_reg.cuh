@@ -73,16 +73,11 @@ __device__ __forceinline__ int tri_edge(const KArgs& A, int64_t e, int ed, int64
   const int32_t w = __ldg(A.fnbr + own);
   const int32_t p = w >> 1;
 #ifdef FR_BOUNDS_CHECK
-  for (int k = 0; k < N; ++k) {
-    const int32_t wk = __ldg(A.fnbr + own + k);
-    const bool whole = p == own ? wk == (int32_t)(((own + k) << 1) | 1)
-                                : p >= 0 && p < A.E * NF && p % N == N - 1 && wk == (int32_t)(((p - k) << 1) | (w & 1));
-    if (!whole) {
-      atomicExch(&A.status[ST_STATUS], kStatusBounds);
-      atomicExch(&A.status[ST_BAD_INDEX], wk);
-      off = (int64_t)e * 2 * NF + ed * N;
-      return kFwL | kFwWall;
-    }
+  if (const int k = tri_edge_broken<N>(A.fnbr, A.E * NF, own); k >= 0) {
+    atomicExch(&A.status[ST_STATUS], kStatusBounds);
+    atomicExch(&A.status[ST_BAD_INDEX], A.fnbr[own + k]);
+    off = (int64_t)e * 2 * NF + ed * N;
+    return kFwL | kFwWall;
   }
 #endif
   off = (int64_t)(p / NF) * 2 * NF + p % NF;

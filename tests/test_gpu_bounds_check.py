@@ -36,46 +36,3 @@ def test_parity_suites_pass_on_the_bounds_checked_build(suite, select):
     tail = "\n".join(r.stdout.splitlines()[-15:])
     assert r.returncode == 0, tail
     assert " passed" in tail and "failed" not in tail, tail
-
-
-_BAD_EDGE = """
-import numpy as np
-import synthetic as S
-import paper_2006_10967_gb300 as G
-from paper_2006_10967_gb300 import _capi
-N = {order} + 1
-w = S.workload("c2t")
-w.order, w.n_precond, w.pseudo_kmax = {order}, 1, 2
-M = G.Mesh.from_synthetic(S.tri_split(1, 1, periodic=(False, False)), w.order)
-n = 2 * 3 * N
-for case in ("before the array", "unread word", "wall off its L side"):
-    F = G.Field(M, G.make_params(w, "mixed", pseudo_fixed=True), ic=w.circle)
-    assert F.sync() == 0
-    words = F._ws[F._base - F._ws.data_ptr():][:F.workspace_bytes // 4 * 4].view(F.torch.int32)
-    v = words.cpu().numpy()
-    at = [i for i in range(0, len(v) - n, 64) if (v[i:i + n] >= 0).all() and (v[i:i + n] < 2 * n).all()
-          and (np.sort(v[i:i + n] >> 1) == np.arange(n)).all()]
-    assert len(at) == 1, at
-    c = v[at[0]:at[0] + n]
-    shared = int(np.flatnonzero(c & 1 == 0)[0])     # first point of the shared edge on its R side
-    where, word = {{"before the array": (shared, 0 << 1), "unread word": (shared + 1, (1 << 30) - 2),
-                   "wall off its L side": (0 if c[0] == 1 else N, None)}}[case]
-    words[at[0] + where] = int(c[where]) - 1 if word is None else word
-    F.step(1)
-    F.precondition()
-    assert F.sync() == _capi.FR_EBOUNDS, case
-print("checked")
-"""
-
-
-@pytest.mark.gpu
-@pytest.mark.parametrize("order", [1, 4])
-def test_checked_build_reports_a_broken_triangle_edge(order):
-    """A triangle edge whose words do not lead to one whole partner edge ends
-    the run of the thread-per-element kernels with FR_EBOUNDS: a partner at the
-    array's start, a word beyond the edge's first, a wall marked as an R side."""
-    from paper_2006_10967_gb300 import build
-    build.build(checked=True)
-    r = subprocess.run([sys.executable, "-c", _BAD_EDGE.format(order=order)], cwd=ROOT, capture_output=True, text=True,
-                       env=dict(os.environ, FRP_BOUNDS_CHECK="1"), timeout=300)
-    assert r.returncode == 0 and r.stdout.strip() == "checked", r.stdout + r.stderr
