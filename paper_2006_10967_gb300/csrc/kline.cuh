@@ -660,7 +660,7 @@ __global__ void __launch_bounds__(WPB * 32, (GEN || (DIM == 3 && N == 5) ? 16 : 
       const float2 nvis = fma2(sh, qn, mul2(dup2(-eps), qe[a][0]));  // minus the viscous flux over M
       const float saa = sd[a], pm = fabsf(saa);
       const float2 sg = make_float2(-saa, saa);
-      Fp = fma2(dup2(__fmul_rn(pm, P.tau)), dp, mul2(sg, fma2(M, nvis, mul2(ap, va))));
+      Fp = fma2(dup2(__fmul_rn(pm, P.tau)), dp, mul2(sg, fma2(ap, va, mul2(M, nvis))));
       Fs = fma2(dup2(__fmul_rn(pm, P.tau_psi)), ds, mul2(sg, mul2(as, va)));
     } else if (GEN) {
       float2 qf[2][DIM];
@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(WPB * 32, (GEN || (DIM == 3 && N == 5) ? 16 : 
       const float2 M = flux_mult(v2, P.gamma);
       const float2 sh = sharp2(pL, g2, P.gamma, P.rdelta);
       const float2 nvis = fma2(sh, qs, mul2(dup2(-eps), qp));
-      Fp = fma2(mul2(pm, dup2(P.tau)), dp, fma2(M, nvis, mul2(ap, vn)));
+      Fp = fma2(mul2(pm, dup2(P.tau)), dp, fma2(ap, vn, mul2(M, nvis)));
       Fs = fma2(mul2(pm, dup2(P.tau_psi)), ds, mul2(as, vn));
     }
     // R ends carry no flux here (ka lifts minus the partner's); no-flux walls none at all
@@ -800,7 +800,7 @@ __global__ void __launch_bounds__(WPB * 32, (GEN || (DIM == 3 && N == 5) ? 16 : 
 #pragma unroll
       for (int c = 0; c < DIM; ++c) {
         const float2 t = fma2(sh, qs[c], mul2(dup2(-eps), q[0][c][p]));
-        f0[c] = fma2(M, t, mul2(u[0][p], v[c]));
+        f0[c] = fma2(u[0][p], v[c], mul2(M, t));
         f1[c] = mul2(u[1][p], v[c]);
       }
 #pragma unroll
