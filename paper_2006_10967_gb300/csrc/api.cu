@@ -23,6 +23,7 @@ struct Layout {
   size_t tri_d, tri_f, tri_high;  // dense triangle operators (double, float), mode mask
   size_t tri_pack;                // their packed form (TriPack)
   size_t triw;                    // triangles: quadrature areas (KArgs.triw)
+  size_t trig;                    // triangles: metric records (KArgs.trig)
   size_t wphys;                   // triangles: physical edge quadrature weight per flux point (float-float)
   size_t ffw;                     // hexahedra: face words (KArgs.ffw)
   size_t vtab64;                  // FP64 tensor fields with a separable velocity: its tables (KArgs.vtabd)
@@ -254,6 +255,7 @@ Layout make_layout(const fr_mesh& m, const fr_params& prm, int max_blocks) {
     L.tri_high = take(NU);
     L.tri_pack = take(TriPack(m.order).size * sizeof(float));
     L.triw = take(E * sizeof(double));
+    L.trig = take(E * 3 * sizeof(float4));
     L.wphys = take(E * NF * 2 * sizeof(float));
   }
   L.total = off;
@@ -854,7 +856,9 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
   std::vector<double> trid;
   std::vector<float> trif, tripack;
   std::vector<double> triw;
+  std::vector<float4> trig;
   A.triw = nullptr;
+  A.trig = nullptr;
   if (m->etype == FR_TRI) {
     triw.assign(m->E, 0.0);
     for (int64_t e = 0; e < m->E; ++e)
@@ -862,6 +866,24 @@ extern "C" int fr_field_init(const fr_mesh* m, const fr_params* prm, const fr_ic
         triw[e] += (double)wdetf[2 * (e * m->nu + i)] + (double)wdetf[2 * (e * m->nu + i) + 1];
     up(L.triw, triw.data(), triw.size() * sizeof(double));
     A.triw = reinterpret_cast<const double*>(b + L.triw);
+    trig.resize(m->E * 3);
+    for (int64_t e = 0; e < m->E; ++e) {
+      const double* g = &m->geo[e * 6];
+      const double S00 = g[5], S01 = -g[2], S10 = -g[4], S11 = g[1], det = g[1] * g[5] - g[2] * g[4];
+      const double n0[3] = {-S10, S00 + S10, -S00}, n1[3] = {-S11, S01 + S11, -S01};
+      const double l[3] = {std::hypot(n0[0], n1[0]), std::hypot(n0[1], n1[1]), std::hypot(n0[2], n1[2])};
+      float* r = reinterpret_cast<float*>(&trig[3 * e]);
+      r[0] = (float)(1.0 / det);
+      for (int k = 0; k < 3; ++k) {
+        r[1 + k] = (float)(l[k] / (k == 1 ? std::sqrt(2.0) : 1.0));
+        r[4 + 2 * k] = (float)(n0[k] / l[k]);
+        r[5 + 2 * k] = (float)(n1[k] / l[k]);
+      }
+      r[10] = (float)det;
+      r[11] = 0.f;
+    }
+    up(L.trig, trig.data(), trig.size() * sizeof(float4));
+    A.trig = reinterpret_cast<const float4*>(b + L.trig);
     pack_tri(m->tri, trid);
     pack_tri(m->tri, trif);
     up(L.tri_d, trid.data(), trid.size() * sizeof(double));

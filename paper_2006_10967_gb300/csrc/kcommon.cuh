@@ -147,6 +147,7 @@ struct KArgs {
   const double* vtabd;   // FP64 tensor fields: E x dim x (n + 2) x 2 separable velocity tables, or nullptr
   const float2* wphys;   // triangles: E x nf physical flux-point weights (float-float), equal on both sides
   const double* triw;    // triangles: E quadrature areas (sum of w det J)
+  const float4* trig;    // triangles: E x 3 metric records: 1 / det J and the edges' |S^T n~|; their unit normals; det J
   int stage;             // 1..4 RK stage, -1: write the rate into out
   int use_dev_time;      // KB: t = dstate[DS_TIME] + c_s dt
   double t;              // KB: stage time when !use_dev_time

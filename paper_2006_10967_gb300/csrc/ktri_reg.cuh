@@ -141,10 +141,9 @@ __global__ void __launch_bounds__(TriReg<P>::TB) kb_trir(const __grid_constant__
   for (int i = 0; i < 6; ++i) g[i] = __ldg(A.geof + e * 6 + i);
   // affine map: S = det J J^{-1}
   const float S00 = g[5], S01 = -g[2], S10 = -g[4], S11 = g[1];
-  const float dj = g[1] * g[5] - g[2] * g[4], rdj = 1.f / dj;
-  // transformed normals n~ S of the edges (0, -1), (1, 1) / sqrt 2, (-1, 0)
+  const float4 rec = __ldg(A.trig + 3 * e), nrm = __ldg(A.trig + 3 * e + 1), nr2 = __ldg(A.trig + 3 * e + 2);
+  const float rdj = rec.x, dj = nr2.z;
   constexpr float r2 = 0.70710678f;
-  const float pn[3][2] = {{-S10, -S11}, {r2 * (S00 + S10), r2 * (S01 + S11)}, {-S00, -S01}};
   float gfac = 0.f;
   if (MODE == 0) gfac = time_factor_t<float>(A, A.use_dev_time ? A.dstate[DS_TIME] + rk_c(A.stage) * A.dt : A.t);
   cp_async_wait_all();
@@ -263,9 +262,8 @@ __global__ void __launch_bounds__(TriReg<P>::TB) kb_trir(const __grid_constant__
 #pragma unroll
         for (int c = 0; c < 2; ++c) tri_acc<NPE>(Lt + (ed * NU + j) * NPE, pair_at(q[f][c], j), qf[f][c]);
     }
-    const float pm = sqrtf(pn[ed][0] * pn[ed][0] + pn[ed][1] * pn[ed][1]);
-    const float rpm = 1.f / pm;
-    const float n0 = pn[ed][0] * rpm, n1 = pn[ed][1] * rpm;
+    const float pm = ed == 0 ? rec.y : ed == 1 ? rec.z : rec.w;
+    const float n0 = ed == 0 ? nrm.x : ed == 1 ? nrm.z : nr2.x, n1 = ed == 0 ? nrm.y : ed == 1 ? nrm.w : nr2.y;
     const bool isl = fl[ed] & kFwL, shut = Pm.noflux && (fl[ed] & kFwWall);
     float Fv[NFLD][2 * NPE];
 #pragma unroll
@@ -324,8 +322,8 @@ __global__ void __launch_bounds__(TriReg<P>::TB) kb_trir(const __grid_constant__
       const float2 M = flux_mult(fma2(v1, v1, mul2(v0, v0)), Pm.gamma);
       const float2 ph = make_float2(u[0][i0], u[0][i1]), ps = make_float2(u[NFLD - 1][i0], u[NFLD - 1][i1]);
       const float2 sh = sharp2(ph, fma2(qs1, qs1, mul2(qs0, qs0)), Pm.gamma, Pm.rdelta);
-      const float2 f00 = fma2(M, fma2(sh, qs0, mul2(dup2(-Pm.eps), q[0][0][i])), mul2(ph, v0));
-      const float2 f01 = fma2(M, fma2(sh, qs1, mul2(dup2(-Pm.eps), q[0][1][i])), mul2(ph, v1));
+      const float2 f00 = fma2(ph, v0, mul2(M, fma2(sh, qs0, mul2(dup2(-Pm.eps), q[0][0][i]))));
+      const float2 f01 = fma2(ph, v1, mul2(M, fma2(sh, qs1, mul2(dup2(-Pm.eps), q[0][1][i]))));
       const float2 f10 = mul2(ps, v0), f11 = mul2(ps, v1);
       q[0][0][i] = fma2(dup2(S01), f01, mul2(dup2(S00), f00));
       q[0][1][i] = fma2(dup2(S11), f01, mul2(dup2(S10), f00));
@@ -453,16 +451,11 @@ __global__ void __launch_bounds__(TriReg<P>::TB) ka_trir(const __grid_constant__
   int fl[3];
   float pm[3] = {0.f, 0.f, 0.f}, rdj = 0.f;
   if constexpr (SF >= 1) {
-    float g[6];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) g[i] = __ldg(A.geof + e * 6 + i);
-    rdj = 1.f / (g[1] * g[5] - g[2] * g[4]);
-    constexpr float r2 = 0.70710678f;
-    const float S00 = g[5], S01 = -g[2], S10 = -g[4], S11 = g[1];
-    const float a0 = r2 * (S00 + S10), a1 = r2 * (S01 + S11);
-    pm[0] = sqrtf(S10 * S10 + S11 * S11);
-    pm[1] = sqrtf(a0 * a0 + a1 * a1);
-    pm[2] = sqrtf(S00 * S00 + S01 * S01);
+    const float4 rec = __ldg(A.trig + 3 * e);
+    rdj = rec.x;
+    pm[0] = rec.y;
+    pm[1] = rec.z;
+    pm[2] = rec.w;
 #pragma unroll
     for (int ed = 0; ed < 3; ++ed) {
       int64_t off;

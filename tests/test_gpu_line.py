@@ -358,7 +358,8 @@ def test_mixed_preconditioning_is_as_close_as_the_block_wide_kernels(G, n, block
 
 
 @pytest.mark.parametrize("etype,orders,sizes", [("hex", (2, 3, 4), ((10,) * 3, (13,) * 3, (16,) * 3, (19, 14, 11))),
-                                                ("quad", (2, 3, 4), ((30, 30), (32, 32), (41, 37), (50, 50)))])
+                                                ("quad", (2, 3, 4), ((30, 30), (32, 32), (41, 37), (50, 50))),
+                                                ("tri", (1, 2, 3), ((20, 20), (25, 25), (31, 31), (40, 40)))])
 def test_rounding_is_no_worse_than_the_block_wide_kernels(G, etype, orders, sizes):
     """Distances from FP64 of the rate and of four steps from one state, over
     the block-wide kernels' (the same field without a cache, under a velocity
