@@ -5,7 +5,9 @@ the residual and update kernels (fr_params.variant; fr_kernel_variants gives
 the count), all equal to round-off.  measure() times each variant on a field
 of the caller's workload with CUDA events around a window of RK4 steps (after
 warm-up steps), and tune() keeps the fastest per (element type, order,
-precision) in tuning.json beside this file.  Fields built with
+precision) in tuning.json beside this file.  The tile variants of quads and of
+hexes of order <= 4 are those of the fields without a velocity cache (with it
+the line kernels run under every number), so they are measured without it.  Fields built with
 variant="auto" (the binding's default) take the table's entry, else 0.
 """
 import json
@@ -38,13 +40,15 @@ def lookup(etype, order, precision):
 def measure(workload, precision="mixed", steps=400, warmup=100, mesh=None):
     """Microseconds per RK stage of every kernel variant on the workload's field."""
     import torch
-    from . import Field, Mesh, kernel_variants, make_params
+    from . import FR_HEX, FR_TRI, Field, Mesh, kernel_variants, make_params
     m = mesh if mesh is not None else workload.mesh()
     M = Mesh.from_synthetic(m, workload.order)
+    # whether the variants differ with the velocity cache
+    cache = M.info.etype == FR_TRI or (M.info.etype == FR_HEX and M.info.order > 4)
     out = {}
     stream = torch.cuda.current_stream()
     for v in range(kernel_variants(M, precision)):
-        F = Field(M, make_params(workload, precision, variant=v), ic=workload.circle, precondition=True)
+        F = Field(M, make_params(workload, precision, variant=v, vel_cache=cache), ic=workload.circle, precondition=True)
         F.step(warmup)
         torch.cuda.synchronize()
         e0 = torch.cuda.Event(enable_timing=True)
