@@ -68,12 +68,13 @@ extern "C" {
 #define FR_HEX 2
 
 #define FR_FP64 0  /* every array and operation in double precision */
-#define FR_MIXED 1 /* float stage values/fluxes/traces; double solution,
-                      RK accumulator, psi0 and mass integral */
+#define FR_MIXED 1 /* float stage values, fluxes, traces and RK accumulator; the
+                      solution as a float-float pair (48 bits); double psi0,
+                      time, pseudo-time residual and mass integral */
 
 #define FR_VEL_UNIFORM 0     /* u = a g(t) */
 #define FR_VEL_RIDER_KOTHE 1 /* Section 4.2 field times g(t) */
-#define FR_VEL_LEVEQUE 2     /* Section 4.3 field times g(t) */
+#define FR_VEL_LEVEQUE 2     /* Section 4.3 field times g(t) (3D; zero on 2D meshes) */
 #define FR_VEL_STREAM 3      /* u = dPsi/dy, v = -dPsi/dx,
                                 Psi = g(t) sum_m A_m sin(2 pi k_m.x) + B_m cos(2 pi k_m.x) */
 #define FR_VEL_ROTATION 4    /* solid-body rotation about (a[0], a[1]): (a[1] - y, x - a[0]),
@@ -304,7 +305,10 @@ int fr_mass_integral_noalloc(const double* dev_u, const double* dev_w, int64_t n
  * flux-point traces. */
 int fr_field_get(fr_field* field, int which, double* host, void* stream);
 int fr_field_set(fr_field* field, int which, const double* host, void* stream);
-/* Device-pointer variants (asynchronous on `stream`), n_dof doubles. */
+/* Device-pointer variants (asynchronous on `stream`), n_dof doubles; any
+ * device pointer that cudaMemcpyAsync takes (memory of the current device on
+ * a boundary of 8 bytes is converted in one pass, other memory through a
+ * staging copy). */
 int fr_field_get_device(fr_field* field, int which, double* dev, void* stream);
 int fr_field_set_device(fr_field* field, int which, const double* dev, void* stream);
 

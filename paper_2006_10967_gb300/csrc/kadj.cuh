@@ -53,7 +53,7 @@ struct AdjArgs {
   double* lam_psi0;     // preconditioning sweep: E x NU, += (dR_p/dpsi0)^T lam (adj_b<.., 1>)
 };
 
-// TD: 1 the default tile, 0 one warp's elements (see one_warp_better).
+// TD: 1 the default tile, 0 one warp's elements (chosen in lb(), adjoint.cu).
 template <int DIM, int N, int TD = 1>
 struct AdjLayout {
   using S = TS<DIM, N>;

@@ -35,7 +35,7 @@ struct PrmT {
   int nphi;    // 1: the sharpening normal comes from phi's gradient (unpreconditioned CPF)
   int noflux;  // 1: zero common normal flux of the physical system at wall flux points
   R rdelta;    // 1 / delta
-  // separable velocity fields (vel_factors): v_c = vs[c] g prod_b T_cb with g = 1 unless vel_g
+  // separable velocity fields (k_vel_tab in kline.cuh): v_c = vs[c] g prod_b T_cb with g = 1 unless vel_g
   R vs[3];
   int vel_g;
 };

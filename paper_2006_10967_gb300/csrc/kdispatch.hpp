@@ -58,9 +58,10 @@ constexpr unsigned kPseudoBlocks = 152 * 6;
 // while the kernel before it on the stream drains (the kernel itself waits, see
 // pdl_wait in kline.cuh).  After a kernel that does not let its dependents
 // start early, it is an ordinary launch.  us a stage with and without: 128^2
-// quads p = 4 13.8 and 14.4, 200^2 p = 5 29.8 and 31.3, jittered 32^3 hexes p = 3
-// 70.0 and 72.0; past kEarlyBlocks there is little to hide and the early blocks
-// cost more (64^3 hexes p = 3: 354 and 351).
+// quads p = 4 11.93 and 12.04, 200^2 p = 5 29.2 and 29.5, jittered 211 x 187 p = 3
+// 17.5 and 18.2, jittered hexes 27 x 22 x 19 p = 2 21.0 and 21.8, 32^3 p = 3 71.8
+// and 72.8, regular 32^3 p = 4 the same (123.6 and 123.5); past kEarlyBlocks there
+// is little to hide and the early blocks cost more (64^3 hexes p = 3: 354 and 351).
 constexpr unsigned kEarlyBlocks = 152 * 160;
 template <typename K>
 inline void launch_pdl(K kern, unsigned grid, int threads, size_t smem, const KArgs& A, cudaStream_t s) {

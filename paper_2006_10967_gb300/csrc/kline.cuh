@@ -22,7 +22,7 @@
 // block-wide kb_tensor executed 796 a point and stage, at 67 % of the issue
 // slots; here 271 on hexes p = 3, at 61 to 66 %), the update kernel (ka_line)
 // moves memory.  Per stage on 64^3 hexes p = 3 (16.8 M points): residual 483 ->
-// 172 us, update 228 -> 180 us (61 bytes of DRAM traffic a point: 5.7 TB/s).
+// 177 us, update 228 -> 175 us (61 bytes of DRAM traffic a point: 5.8 TB/s).
 #pragma once
 #include "ktensor.cuh"
 
@@ -207,8 +207,9 @@ __device__ __forceinline__ void tile_fetch(float* dst, const void* src, int ne, 
 // kernels before, which is complete by then, but they are read after pdl_wait
 // like the rest.  Every kernel waits before it returns.
 // kEarly: regular hexes of N >= 4 (the large 3D runs) wait first and load their
-// state first: with thousands of blocks a wave there is little to hide, and the
-// other order cost them 2 % (64^3 p = 3: 358 and 350 us a stage).
+// state first: with thousands of blocks a wave there is little to hide (the
+// other order: 64^3 p = 3 360 and 359 us a stage, 32^3 p = 4 124 and 125; it cost
+// p = 3 2 % while the solution too was read before the wait).
 template <int DIM, int N, bool GEN>
 constexpr bool kEarly = !(DIM == 3 && N >= 4 && !GEN);
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -800,6 +801,8 @@ __global__ void __launch_bounds__(WPB * 32, (GEN || (DIM == 3 && N == 5) ? 16 : 
 #pragma unroll
       for (int c = 0; c < DIM; ++c) {
         const float2 t = fma2(sh, qs[c], mul2(dup2(-eps), q[0][c][p]));
+        // the larger term in the last multiply-add: one rounding of its size (added first, phi's rate was
+        // 4 % further from FP64 on regular hexes)
         f0[c] = fma2(u[0][p], v[c], mul2(M, t));
         f1[c] = mul2(u[1][p], v[c]);
       }
