@@ -60,7 +60,7 @@ typedef TensorOpsT<double> TensorOps;
 
 // The 1D operators in the pairs that the paired-FP32 line kernels use
 // (kline.cuh): outputs (2p, 2p + 1) of a line, or a line's two ends.
-struct LineOps {
+struct alignas(16) LineOps {  // pairs of pairs load as one 16-byte constant (off that boundary kb_line ran 1.4 % more instructions)
   float2 D[kMaxN][4];                 // [input m][output pair p]
   float2 lend[kMaxN];                 // (l_m(-1), l_m(+1))
   float2 gL[4], ngL[4], gR[4], xp[4];  // end lifts (ngL = -gL) and coordinates by point pair
