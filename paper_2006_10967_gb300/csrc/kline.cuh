@@ -22,7 +22,7 @@
 // block-wide kb_tensor executed 796 a point and stage, at 67 % of the issue
 // slots; here 271 on hexes p = 3, at 61 to 66 %), the update kernel (ka_line)
 // moves memory.  Per stage on 64^3 hexes p = 3 (16.8 M points): residual 483 ->
-// 177 us, update 228 -> 175 us (61 bytes of DRAM traffic a point: 5.8 TB/s).
+// 172 us, update 228 -> 182 us (61 bytes of DRAM traffic a point: 5.6 TB/s).
 #pragma once
 #include "ktensor.cuh"
 
@@ -208,7 +208,7 @@ __device__ __forceinline__ void tile_fetch(float* dst, const void* src, int ne, 
 // like the rest.  Every kernel waits before it returns.
 // kEarly: regular hexes of N >= 4 (the large 3D runs) wait first and load their
 // state first: with thousands of blocks a wave there is little to hide (the
-// other order: 64^3 p = 3 360 and 359 us a stage, 32^3 p = 4 124 and 125; it cost
+// other order costs 64^3 p = 3 0.4 % a stage and gains 32^3 p = 4 0.8 %; it cost
 // p = 3 2 % while the solution too was read before the wait).
 template <int DIM, int N, bool GEN>
 constexpr bool kEarly = !(DIM == 3 && N >= 4 && !GEN);
