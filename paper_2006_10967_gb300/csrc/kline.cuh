@@ -206,10 +206,10 @@ __device__ __forceinline__ void tile_fetch(float* dst, const void* src, int ne, 
 // accumulator and flux balances of the update kernels come from the update two
 // kernels before, which is complete by then, but they are read after pdl_wait
 // like the rest.  Every kernel waits before it returns.
-// kEarly: regular hexes of N >= 4 (the large 3D runs) wait first and load their
-// state first: with thousands of blocks a wave there is little to hide (the
-// other order costs 64^3 p = 3 0.4 % a stage and gains 32^3 p = 4 0.8 %; it cost
-// p = 3 2 % while the solution too was read before the wait).
+// kEarly: regular hexes of N >= 4 (the large 3D runs) load their state before the
+// connectivity: with thousands of blocks a wave there is little to hide (64^3
+// p = 3 358 and 350 us a stage; their update kernels' metric and weights still
+// come first, 32^3 p = 4 123.4 and 125.2 us with them after the state).
 template <int DIM, int N, bool GEN>
 constexpr bool kEarly = !(DIM == 3 && N >= 4 && !GEN);
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -1014,9 +1014,10 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
     const float* src = SF == 0 ? ustg : reinterpret_cast<const float*>(A.rp);
     if constexpr (L::DIRECT) {
 #pragma unroll
+      for (int f = 0; f < 2; ++f) grow_get<N>(src + (e * 2 + f) * NU + l * N, y[f]);
+#pragma unroll
       for (int f = 0; f < 2; ++f) {
         const int64_t r = (e * 2 + f) * NU + l * N;
-        grow_get<N>(src + r, y[f]);
         if constexpr (SF >= 1) {
 #pragma unroll
           for (int j = 0; j < N; j += 2) {
@@ -1039,7 +1040,6 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
     if constexpr (SF >= 2)
       if (cons && threadIdx.x < 2 * NEL && gt < 2 * A.E) ta = A.tacc[gt];
   };
-  if constexpr (!kEarly<DIM, N, GEN>) load_state();
   if constexpr (SF >= 1) {
     const float* mc = reinterpret_cast<const float*>(A.mcg) + e * kMetricRec;
     rdet = __ldg(mc + 10);
@@ -1050,6 +1050,7 @@ __global__ void __launch_bounds__(WPB * 32, (DIM == 3 ? 24 : 20) / WPB) ka_line(
     if (SF == 4 && cons && threadIdx.x < 2 * NEL && gt < 2 * A.E)
       rW = *reinterpret_cast<const float2*>(reinterpret_cast<const float*>(A.mcg) + (gt / 2) * kMetricRec + 12);
   }
+  if constexpr (!kEarly<DIM, N, GEN>) load_state();
   int fl[DIM][2];
   [[maybe_unused]] int2 fw[DIM][2];
   [[maybe_unused]] int32_t w2[DIM][2];
