@@ -20,7 +20,7 @@
 //
 // What bounds it: the residual kernel (kb_line) issues instructions (the
 // block-wide kb_tensor executed 796 a point and stage, at 67 % of the issue
-// slots; here 271 on hexes p = 3, at 61 to 66 %), the update kernel (ka_line)
+// slots; here 272 on hexes p = 3, at 61 to 66 %), the update kernel (ka_line)
 // moves memory.  Per stage on 64^3 hexes p = 3 (16.8 M points): residual 483 ->
 // 172 us, update 228 -> 182 us (61 bytes of DRAM traffic a point: 5.6 TB/s).
 #pragma once
